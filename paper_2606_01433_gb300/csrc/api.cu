@@ -1209,6 +1209,7 @@ void setup_impl(gdsw_ctx* c, const gdsw_mesh* mesh, const gdsw_viscosity* visc, 
     double b = 8.0 * (9.0 * M.a_col.size() + 3.0 * M.bt_col.size() + 3.0 * M.b_col.size());
     b += 4.0 * (M.a_col.size() + M.bt_col.size() + M.b_col.size() + 4.0 * M.n) + 8.0 * 27 * M.fluid.size();
     b += 4.0 * (M.asm_uoff.size() + M.asm_unit.size() + M.asm_cta.size());
+    b += 8.0 * kAsmElemValues * double(std::min<int64_t>(kAsmChunk, int64_t(M.fluid.size())));
     b += 80.0 * M.sell_acol.size() + 32.0 * M.sell_bcol.size() + 4.0 * M.sell_row.size();
     for (int l = 0; l < nlev; ++l) {
       const LevelHost& H = c->lh[l];
@@ -1258,6 +1259,7 @@ void setup_impl(gdsw_ctx* c, const gdsw_mesh* mesh, const gdsw_viscosity* visc, 
   c->d_asm_cta = c->arena.upload(M.asm_cta, s);
   c->d_asm_uoff = c->arena.upload(M.asm_uoff, s);
   c->d_asm_unit = c->arena.upload(M.asm_unit, s);
+  c->d_asm_ws = c->arena.alloc<double>(size_t(std::min<int64_t>(kAsmChunk, int64_t(M.fluid.size())) * kAsmElemValues));
   c->n_sell_slices = int64_t(M.sell_aoff.size()) - 1;
   c->d_sell_row = c->arena.upload(M.sell_row, s);
   c->d_sell_aoff = c->arena.upload(M.sell_aoff, s);

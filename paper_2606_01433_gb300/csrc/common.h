@@ -133,6 +133,10 @@ struct DevArena {
 };
 
 inline size_t elem_size(int prec) { return prec == GDSW_FP64 ? 8 : (prec == GDSW_FP32 ? 4 : 2); }
+// assembly workspace: the 405 blocks (9 values) of each fluid element of a chunk.  9120 elements
+// are five full waves of the element kernel (152 SMs, 6 CTAs of 2 elements) and 266 MB.
+constexpr int64_t kAsmChunk = 9120;
+constexpr int64_t kAsmElemValues = 405 * 9;
 inline int64_t pad8(int64_t x) { return (x + 7) & ~int64_t(7); }
 
 // ------------------------------------------------------------------ device task descriptors
@@ -252,6 +256,8 @@ struct MeshHost {
   std::vector<int32_t> asm_uoff;         // per block: first unit (lower blocks own none), nnzb + 1
   std::vector<uint32_t> asm_unit;
   std::vector<int32_t> asm_cta;          // first block of each assembly CTA (<= 256 units), + nnzb
+  std::vector<int64_t> asm_chunk;        // fluid elements assembled at a time: chunk bounds
+  std::vector<int32_t> asm_chunk_cta;    // per chunk: range of the assembly CTAs it touches
   // sliced copy of the velocity rows for the SpMV (32 rows per slice, rows sorted by length
   // inside windows of 1024 rows so that a slice's rows have near-equal lengths): slot
   // j * 32 + lane of slice s holds the j-th block (or B^T entry) of the slice's lane-th row
@@ -392,6 +398,7 @@ struct gdsw_ctx {
   int32_t *d_a_diag = nullptr, *d_a_tpos = nullptr;  // diagonal block of each row, transpose map
   int32_t *d_asm_cta = nullptr, *d_asm_uoff = nullptr;  // assembly work units (see MeshHost)
   uint32_t* d_asm_unit = nullptr;
+  double* d_asm_ws = nullptr;       // element blocks of one chunk (asm_ws_bytes)
   int32_t *d_sell_row = nullptr, *d_sell_acol = nullptr, *d_sell_asrc = nullptr;  // sliced SpMV copy
   int32_t *d_sell_bcol = nullptr, *d_sell_bsrc = nullptr;
   int64_t *d_sell_aoff = nullptr, *d_sell_boff = nullptr;

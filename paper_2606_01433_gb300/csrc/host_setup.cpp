@@ -420,6 +420,30 @@ void build_mesh(MeshHost& M, const gdsw_mesh* m) {
   for (int64_t q = 0; q < nnzb; ++q)
     if (M.asm_uoff[q + 1] - M.asm_uoff[M.asm_cta.back()] > 256) M.asm_cta.push_back(int32_t(q));
   M.asm_cta.push_back(int32_t(nnzb));
+  // chunks of the element kernel and, for each, the CTAs that hold a block of its nodes: the rows
+  // between the smallest and the largest node of the chunk's elements
+  const int64_t nfe = int64_t(M.fluid.size());
+  M.asm_chunk.assign(1, 0);
+  M.asm_chunk_cta.clear();
+  for (int64_t f0 = 0; f0 < nfe; f0 += kAsmChunk) {
+    const int64_t f1 = std::min(nfe, f0 + kAsmChunk);
+    int64_t lo = M.nnodes, hi = -1;
+    for (int64_t f = f0; f < f1; ++f) {
+      const int64_t e = M.fluid[f];
+      const int64_t ex = e % M.nx, ey = (e / M.nx) % M.ny, ez = e / (int64_t(M.nx) * M.ny);
+      const int64_t n0 = 2 * ex + int64_t(M.NX) * (2 * ey + int64_t(M.NY) * 2 * ez);
+      lo = std::min(lo, n0);
+      hi = std::max(hi, n0 + 2 + 2 * int64_t(M.NX) + 2 * int64_t(M.NX) * M.NY);
+    }
+    const int64_t I0 = std::lower_bound(M.vnode.begin(), M.vnode.end(), int32_t(lo)) - M.vnode.begin();
+    const int64_t I1 = std::upper_bound(M.vnode.begin(), M.vnode.end(), int32_t(hi)) - M.vnode.begin();
+    const int32_t b0 = M.a_ptr[I0], b1 = M.a_ptr[I1];
+    const int32_t c0 = int32_t(std::upper_bound(M.asm_cta.begin(), M.asm_cta.end(), b0) - M.asm_cta.begin()) - 1;
+    const int32_t c1 = int32_t(std::lower_bound(M.asm_cta.begin(), M.asm_cta.end(), b1) - M.asm_cta.begin());
+    M.asm_chunk.push_back(f1);
+    M.asm_chunk_cta.push_back(b1 > b0 ? c0 : 0);
+    M.asm_chunk_cta.push_back(b1 > b0 ? c1 : 0);
+  }
   // BT entry (I, P) has the value of B entry (P, I)
   M.bt2b.resize(M.bt_col.size());
   std::atomic<int> basym(0);

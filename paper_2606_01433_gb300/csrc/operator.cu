@@ -206,123 +206,260 @@ __device__ void divergence_entry_p1(int64_t P, int64_t J, const Geo& G, const in
 }
 
 // ------------------------------------------------------------------ a2: assembly
-// On GB300 a warp-wide FP64 instruction holds the FP64 pipe for the same time whether 1 or 32
-// lanes are active, so the assembly is organised for uniform lanes: one thread per work unit
-// (an upper block (I, J >= I) and one fluid element holding both nodes), each unit exactly 27
-// Gauss points.  Per unit the thread accumulates
-//   O[c][d] = sum_q f_q dphi_b,c(q) dphi_a,d(q),   f_q = nu_q w_q (h/2)^3 (2/h)^2,
-// and the element's contribution to the block is tr(O) I + O for the symmetric form 2 nu D:D
-// (Section 3) and tr(O) I for the gradient form nu grad:grad (Section 2).  A CTA holds the
-// units of whole blocks (at most 256); each block sums its units' O in element order in
-// shared memory, then writes itself and, off the diagonal, its transpose (operator symmetric).
-struct SmemTables {
-  double dphi[27][27][3];
-  double wsc[27];
-};
+// Element blocks by sum factorisation, then a gather over the elements of every block.
+//
+// The Q2 basis and the Gauss rule are tensor products, so with f_q = nu_q w_q (h/2)^3 (2/h)^2
+//   G_lm[a, b] = sum_q f_q d_l phi_a(q) d_m phi_b(q),   l, m = x, y, z,
+// factors into three one-dimensional contractions: over q_x (X, per pair a_x, b_x and
+// derivative pattern), over q_y (nine values per q_z for each pair of planar nodes A = (a_x, a_y),
+// B = (b_x, b_y)), over q_z.  The block of nodes (a, b) is K_cd = G_dc + delta_cd tr G for the
+// symmetric form 2 nu D:D (Section 3) and delta_cd tr G for the gradient form (Section 2).
+// An element costs 14 thousand FP64 operations instead of the 133 thousand of a sum over the 27
+// points per pair: the FP64 pipe (1.26 TFLOP/s, one warp instruction per 16 cycles and SM)
+// bounds either form.  A thread owns one of the 45 planar pairs A <= B of an element (both
+// forms of a block from its transpose) and runs its nine (a_z, b_z) with the one-dimensional
+// values of the last contraction as compile-time constants, whose zeros (the middle Gauss point
+// is the middle node) drop out.  Two elements per CTA of 96 threads: 94% of the lanes busy, and
+// 512 elements (the smallest meshes) still give 256 CTAs.  Measured on the 32^3 channel (31
+// thousand elements): 7.09 ms as a sum over the points per pair -> 0.83 ms here (FP64-bound) +
+// 0.69 ms in k_gather_blocks (3 GB, 4.3 TB/s); 756 elements: 167 -> 29 + 25 us.
+//
+// Workspace: unit (a, b) of element e at ws[((a_z 3 + b_z) NT + 45 e + P(A, B)) 9 .. + 9], so a
+// warp's 32 blocks are 2304 contiguous bytes.  It holds kAsmChunk elements (266 MB); larger
+// meshes run chunk by chunk and the gather adds onto the blocks of the chunks before.
+constexpr int kAsmPairs = 45;
 
-__global__ void __launch_bounds__(256) k_assemble_A(const int32_t* __restrict__ asm_cta,
-                                                    const int32_t* __restrict__ asm_uoff,
-                                                    const uint32_t* __restrict__ asm_unit,
-                                                    const int32_t* __restrict__ a_tpos,
-                                                    const double* __restrict__ nu, const RefTables* __restrict__ T,
-                                                    double sc, int form, const double* __restrict__ dn,
-                                                    double* __restrict__ val) {
-  __shared__ SmemTables st;
-  __shared__ double part[256][10];  // per unit: the block's non-trace part, then the trace term
+// one-dimensional Q2 basis / derivative a at Gauss point q
+__host__ __device__ constexpr double gauss_x(int q) { return q == 0 ? -0.7745966692414834 : (q == 1 ? 0.0 : 0.7745966692414834); }
+__host__ __device__ constexpr double q2_v(int a, int q) {
+  const double x = gauss_x(q);
+  return a == 0 ? 0.5 * x * (x - 1.0) : (a == 1 ? 1.0 - x * x : 0.5 * x * (x + 1.0));
+}
+__host__ __device__ constexpr double q2_d(int a, int q) {
+  const double x = gauss_x(q);
+  return a == 0 ? x - 0.5 : (a == 1 ? -2.0 * x : x + 0.5);
+}
+// derivative pattern t of a one-dimensional pair: 0 value-value, 1 value-derivative (of b), 2
+// derivative-derivative
+__host__ __device__ constexpr double q2_pair(int t, int a, int b, int q) {
+  return (t == 2 ? q2_d(a, q) : q2_v(a, q)) * (t == 0 ? q2_v(b, q) : q2_d(b, q));
+}
+// planar pair (A <= B) of an element: its rank and back
+__host__ __device__ constexpr int planar_rank(int A, int B) { return A * 9 - A * (A - 1) / 2 + (B - A); }
+
+// NEWTON adds sum_q f_N (D(u_k) grad phi_a)_c (D(u_k) grad phi_b)_d from the D, N values of k_viscosity.
+template <bool SYM, bool NEWTON>
+__global__ void __launch_bounds__(96) k_element_blocks(const double* __restrict__ nu, const RefTables* __restrict__ T,
+                                                       double sc, const double* __restrict__ dn, int64_t f0,
+                                                       int64_t nfe, double* __restrict__ ws) {
+  constexpr int EPC = 2, NW = 3;
+  __shared__ double t1[3][9][3];             // [pattern][a 3 + b][q]
+  __shared__ double fq[EPC][27];
+  __shared__ double X[EPC][3][9][9];         // [pattern][a_x 3 + b_x][q_y + 3 q_z]
+  __shared__ double stage[NW][32 * 9];
+  __shared__ double tg[NEWTON ? EPC * 27 * 27 * 3 : 1];  // [element][q][a][c]: (D grad phi_a)_c
+  __shared__ double fn[EPC][27];
+  dep_release();
+  const int tid = threadIdx.x;
+  if (tid < 81) {
+    const int p = tid / 27, ab = (tid / 3) % 9, q = tid % 3, a = ab / 3, b = ab % 3;
+    t1[p][ab][q] = (p == 2 ? q2_d(a, q) : q2_v(a, q)) * (p == 0 ? q2_v(b, q) : q2_d(b, q));
+  }
+  dep_wait();
+  const int64_t e0 = int64_t(blockIdx.x) * EPC;
+  const int ne = int(min(int64_t(EPC), nfe - e0));
+  if (tid < EPC * 27) {
+    const int el = tid / 27, q = tid - 27 * el;
+    fq[el][q] = el < ne ? nu[(f0 + e0 + el) * 27 + q] * (T->w[q] * sc) : 0.0;
+    if (NEWTON) fn[el][q] = el < ne ? dn[((f0 + e0 + el) * 27 + q) * 7 + 6] * (T->w[q] * sc) : 0.0;
+  }
+  if (NEWTON) {
+    for (int i = tid; i < EPC * 729; i += 96) {
+      const int el = i / 729, r = i - 729 * el, q = r / 27, a = r - 27 * q;
+      const double* g = dn + ((f0 + e0 + min(el, ne - 1)) * 27 + q) * 7;
+      const double d0 = T->dphi[q][a][0], d1 = T->dphi[q][a][1], d2 = T->dphi[q][a][2];
+      double* o = tg + i * 3;
+      o[0] = g[0] * d0 + g[3] * d1 + g[4] * d2;
+      o[1] = g[3] * d0 + g[1] * d1 + g[5] * d2;
+      o[2] = g[4] * d0 + g[5] * d1 + g[2] * d2;
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < EPC * 243; i += 96) {
+    const int el = i / 243, r = i - 243 * el, p = r / 81, ab = (r / 9) % 9, q23 = r % 9;
+    const double* f = fq[el] + 3 * q23;
+    X[el][p][ab][q23] = fma(t1[p][ab][2], f[2], fma(t1[p][ab][1], f[1], t1[p][ab][0] * f[0]));
+  }
+  __syncthreads();
+  const int el = tid >= kAsmPairs ? 1 : 0;
+  int P = min(tid - kAsmPairs * el, kAsmPairs - 1);  // the last six lanes repeat a pair and store nothing
+  int A = 0;
+  while (P >= planar_rank(A + 1, A + 1)) ++A;
+  const int B = A + (P - planar_rank(A, A));
+  const int ax = A % 3, ay = A / 3, bx = B % 3, by = B / 3;
+  // Y*[q_z]: names give the derivative of a, then of b, taken so far (0 = none)
+  double Yxx[3], Yyy[3], Y00[3], Yxy[3], Yyx[3], Yx0[3], Y0x[3], Yy0[3], Y0y[3];
   {
-    const double* src = &T->dphi[0][0][0];
-    double* dst = &st.dphi[0][0][0];
-    for (int e = threadIdx.x; e < 27 * 27 * 3; e += blockDim.x) dst[e] = src[e];
-    if (threadIdx.x < 27) st.wsc[threadIdx.x] = T->w[threadIdx.x] * sc;
-  }
-  __syncthreads();
-  const int blk0 = asm_cta[blockIdx.x], blk1 = asm_cta[blockIdx.x + 1];
-  const int u0 = asm_uoff[blk0], u1 = asm_uoff[blk1];
-  const int u = u0 + int(threadIdx.x);
-  double O[9], ON[9];
+    double s00[3], s01[3], s10[3], s11[3];
 #pragma unroll
-  for (int c = 0; c < 9; ++c) O[c] = ON[c] = 0.0;
-  if (u < u1) {
-    const uint32_t w = asm_unit[u];
-    const int fe = int(w >> 10), a = int((w >> 5) & 31u), b = int(w & 31u);
-    const double* nq = nu + int64_t(fe) * 27;
-    if (form == GDSW_FORM_SYMMETRIC) {
-      for (int q = 0; q < 27; ++q) {
-        const double f = __ldg(nq + q) * st.wsc[q];
-        const double* da = st.dphi[q][a];
-        const double* db = st.dphi[q][b];
-        const double fa0 = f * da[0], fa1 = f * da[1], fa2 = f * da[2];
+    for (int q = 0; q < 3; ++q) {
+      s00[q] = t1[0][ay * 3 + by][q];
+      s01[q] = t1[1][ay * 3 + by][q];
+      s10[q] = t1[1][by * 3 + ay][q];
+      s11[q] = t1[2][ay * 3 + by][q];
+    }
+    const double* x00 = X[el][0][ax * 3 + bx];
+    const double* x01 = X[el][1][ax * 3 + bx];
+    const double* x10 = X[el][1][bx * 3 + ax];
+    const double* x11 = X[el][2][ax * 3 + bx];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const double dbc = db[c];
-          O[c * 3 + 0] = fma(dbc, fa0, O[c * 3 + 0]);
-          O[c * 3 + 1] = fma(dbc, fa1, O[c * 3 + 1]);
-          O[c * 3 + 2] = fma(dbc, fa2, O[c * 3 + 2]);
+    for (int z = 0; z < 3; ++z) {
+      Yxx[z] = Yyy[z] = Y00[z] = Yxy[z] = Yyx[z] = Yx0[z] = Y0x[z] = Yy0[z] = Y0y[z] = 0.0;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const double v00 = x00[q + 3 * z], v11 = x11[q + 3 * z];
+        Yxx[z] = fma(v11, s00[q], Yxx[z]);
+        Yyy[z] = fma(v00, s11[q], Yyy[z]);
+        Y00[z] = fma(v00, s00[q], Y00[z]);
+        if (SYM) {
+          const double v01 = x01[q + 3 * z], v10 = x10[q + 3 * z];
+          Yxy[z] = fma(v10, s01[q], Yxy[z]);
+          Yyx[z] = fma(v01, s10[q], Yyx[z]);
+          Yx0[z] = fma(v10, s00[q], Yx0[z]);
+          Y0x[z] = fma(v01, s00[q], Y0x[z]);
+          Yy0[z] = fma(v00, s10[q], Yy0[z]);
+          Y0y[z] = fma(v00, s01[q], Y0y[z]);
         }
       }
-      if (dn) {  // Newton term: N (D grad phi_a)_c (D grad phi_b)_d at every Gauss point
+    }
+  }
+  const int warp = tid >> 5, lane = tid & 31;
+  const int nth = kAsmPairs * ne - 32 * warp;          // blocks of this warp (may be more than 32)
+  const int cnt = 9 * max(0, min(32, nth));
+  const int64_t NT = nfe * kAsmPairs;
+  double* out = ws + (e0 * kAsmPairs + 32 * warp) * 9;
+  double* st = stage[warp];
+#pragma unroll
+  for (int az = 0; az < 3; ++az)
+#pragma unroll
+    for (int bz = 0; bz < 3; ++bz) {
+      double xx = 0, yy = 0, zz = 0, xy = 0, yx = 0, xz = 0, zx = 0, yz = 0, zy = 0;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const double c00 = q2_pair(0, az, bz, q), c01 = q2_pair(1, az, bz, q), c10 = q2_pair(1, bz, az, q),
+                     c11 = q2_pair(2, az, bz, q);
+        if (c00 != 0.0) {
+          xx = fma(Yxx[q], c00, xx);
+          yy = fma(Yyy[q], c00, yy);
+          if (SYM) {
+            xy = fma(Yxy[q], c00, xy);
+            yx = fma(Yyx[q], c00, yx);
+          }
+        }
+        if (c11 != 0.0) zz = fma(Y00[q], c11, zz);
+        if (SYM) {
+          if (c01 != 0.0) {
+            xz = fma(Yx0[q], c01, xz);
+            yz = fma(Yy0[q], c01, yz);
+          }
+          if (c10 != 0.0) {
+            zx = fma(Y0x[q], c10, zx);
+            zy = fma(Y0y[q], c10, zy);
+          }
+        }
+      }
+      const double tr = (xx + yy) + zz;
+      double K[9] = {tr, 0, 0, 0, tr, 0, 0, 0, tr};
+      if (SYM) {
+        K[0] += xx;
+        K[1] = yx;
+        K[2] = zx;
+        K[3] = xy;
+        K[4] += yy;
+        K[5] = zy;
+        K[6] = xz;
+        K[7] = yz;
+        K[8] += zz;
+      }
+      if (NEWTON) {
+        const double* ta = tg + el * 2187 + (A + 9 * az) * 3;
+        const double* tb = tg + el * 2187 + (B + 9 * bz) * 3;
+        double N[9] = {};
         for (int q = 0; q < 27; ++q) {
-          const double* g = dn + (int64_t(fe) * 27 + q) * 7;
-          const double Dm[3][3] = {{g[0], g[3], g[4]}, {g[3], g[1], g[5]}, {g[4], g[5], g[2]}};
-          const double f = g[6] * st.wsc[q];
-          const double* da = st.dphi[q][a];
-          const double* db = st.dphi[q][b];
-          double ga[3], gb[3];
+          const double f = fn[el][q];
+          const double b0 = tb[81 * q], b1 = tb[81 * q + 1], b2 = tb[81 * q + 2];
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            ga[c] = Dm[c][0] * da[0] + Dm[c][1] * da[1] + Dm[c][2] * da[2];
-            gb[c] = Dm[c][0] * db[0] + Dm[c][1] * db[1] + Dm[c][2] * db[2];
-          }
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const double fc = f * ga[c];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) ON[c * 3 + d] = fma(fc, gb[d], ON[c * 3 + d]);
+            const double fa = f * ta[81 * q + c];
+            N[3 * c] = fma(fa, b0, N[3 * c]);
+            N[3 * c + 1] = fma(fa, b1, N[3 * c + 1]);
+            N[3 * c + 2] = fma(fa, b2, N[3 * c + 2]);
           }
         }
+#pragma unroll
+        for (int m = 0; m < 9; ++m) K[m] += N[m];
       }
-    } else {  // only the trace is needed
-      for (int q = 0; q < 27; ++q) {
-        const double f = __ldg(nq + q) * st.wsc[q];
-        const double* da = st.dphi[q][a];
-        const double* db = st.dphi[q][b];
-        O[0] = fma(f * da[0], db[0], O[0]);
-        O[4] = fma(f * da[1], db[1], O[4]);
-        O[8] = fma(f * da[2], db[2], O[8]);
-      }
+      __syncwarp();
+#pragma unroll
+      for (int m = 0; m < 9; ++m) st[lane * 9 + m] = K[m];
+      __syncwarp();
+      double* o = out + int64_t(az * 3 + bz) * NT * 9;
+#pragma unroll
+      for (int i = 0; i < 9; ++i)
+        if (lane + 32 * i < cnt) o[lane + 32 * i] = st[lane + 32 * i];
     }
+}
+
+// Blocks of the CTAs [cta0, cta0 + gridDim): every upper block (I, J >= I) sums the units of the
+// elements [f0, f1) in element order -- onto what the chunks before left, if its first unit lies
+// in one of them -- and writes itself and, off the diagonal, its transpose (operator symmetric).
+// A CTA holds the units of whole blocks (at most 256); its threads take single values, nine to a
+// unit or block, so that loads and stores run along the 72-byte blocks.
+__global__ void __launch_bounds__(256) k_gather_blocks(const int32_t* __restrict__ asm_cta, int cta0,
+                                                       const int32_t* __restrict__ asm_uoff,
+                                                       const uint32_t* __restrict__ asm_unit,
+                                                       const int32_t* __restrict__ a_tpos,
+                                                       const double* __restrict__ ws, int64_t f0, int64_t f1,
+                                                       double* __restrict__ val) {
+  __shared__ int64_t uaddr[256];   // workspace offset of the unit (transposed blocks: -1 - offset)
+  __shared__ double part[256 * 9];
+  __shared__ int32_t in[257];      // units of the chunk before unit u (its range is contiguous in a block)
+  dep_release();
+  const int blk0 = asm_cta[cta0 + blockIdx.x], blk1 = asm_cta[cta0 + blockIdx.x + 1];
+  const int u0 = asm_uoff[blk0], nu = asm_uoff[blk1] - u0;
+  const int64_t NT = (f1 - f0) * kAsmPairs;
+  for (int u = threadIdx.x; u < nu; u += 256) {
+    const uint32_t w = asm_unit[u0 + u];
+    const int64_t fe = w >> 10;
+    const int a = int((w >> 5) & 31u), b = int(w & 31u);
+    const int A = a % 9, az = a / 9, B = b % 9, bz = b / 9;
+    const bool tr = A > B;
+    const int64_t z = tr ? bz * 3 + az : az * 3 + bz;
+    const int64_t off = (z * NT + (fe - f0) * kAsmPairs + (tr ? planar_rank(B, A) : planar_rank(A, B))) * 9;
+    uaddr[u] = tr ? -1 - off : off;
+    in[u] = fe >= f0 && fe < f1;
   }
-#pragma unroll
-  for (int c = 0; c < 9; ++c) part[threadIdx.x][c] = form == GDSW_FORM_SYMMETRIC ? O[c] + ON[c] : 0.0;
-  part[threadIdx.x][9] = O[0] + O[4] + O[8];
   __syncthreads();
-  for (int blk = blk0 + int(threadIdx.x); blk < blk1; blk += blockDim.x) {
-    const int v0 = asm_uoff[blk], v1 = asm_uoff[blk + 1];
-    if (v1 == v0) continue;  // a lower block: written as the transpose of its upper partner
-    double S[10];
-#pragma unroll
-    for (int c = 0; c < 10; ++c) S[c] = part[v0 - u0][c];
-    for (int v = v0 + 1; v < v1; ++v)
-#pragma unroll
-      for (int c = 0; c < 10; ++c) S[c] += part[v - u0][c];
-    const double tr = S[9];
-    double out[9];
-#pragma unroll
-    for (int c = 0; c < 9; ++c) out[c] = S[c];
-    out[0] += tr;
-    out[4] += tr;
-    out[8] += tr;
-    double* vp = val + int64_t(blk) * 9;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) vp[c] = out[c];
+  dep_wait();
+  for (int i = threadIdx.x; i < nu * 9; i += 256) {
+    const int u = i / 9, m = i - 9 * u;
+    if (!in[u]) continue;
+    const int64_t s = uaddr[u];
+    part[i] = s >= 0 ? ws[s + m] : ws[-1 - s + (m % 3) * 3 + m / 3];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < (blk1 - blk0) * 9; i += 256) {
+    const int q = i / 9, m = i - 9 * q, blk = blk0 + q;
+    const int v0 = asm_uoff[blk] - u0, v1 = asm_uoff[blk + 1] - u0;
+    int v = v0;
+    while (v < v1 && !in[v]) ++v;
+    if (v == v1) continue;  // a lower block, or no unit in this chunk
+    double* vp = val + int64_t(blk) * 9 + m;
+    double s = v == v0 ? part[v * 9 + m] : *vp + part[v * 9 + m];
+    for (++v; v < v1 && in[v]; ++v) s += part[v * 9 + m];
+    *vp = s;
     const int tb = a_tpos[blk];
-    if (tb != blk) {
-      double* wp = val + int64_t(tb) * 9;
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) wp[d * 3 + c] = out[c * 3 + d];
-    }
+    if (tb != blk) val[int64_t(tb) * 9 + (m % 3) * 3 + m / 3] = s;
   }
 }
 
@@ -588,11 +725,21 @@ void launch_assembly(gdsw_ctx* c, cudaStream_t s, bool newton) {
   double* aval = c->d_val;
   double* btval = c->d_val + 9 * c->nnzb;
   double* bval = btval + 3 * c->nbt;
-  const int ncta = int(c->mesh.asm_cta.size()) - 1;
-  if (ncta > 0)
-    k_assemble_A<<<ncta, 256, 0, s>>>(c->d_asm_cta, c->d_asm_uoff, c->d_asm_unit, c->d_a_tpos, c->d_nu, T,
-                                      0.5 * c->mesh.h, c->form, newton ? c->d_dn : nullptr, aval);
-  check_launch("k_assemble_A");
+  for (size_t q = 0; q + 1 < c->mesh.asm_chunk.size(); ++q) {
+    const int64_t f0 = c->mesh.asm_chunk[q], f1 = c->mesh.asm_chunk[q + 1];
+    const int cta0 = c->mesh.asm_chunk_cta[2 * q], cta1 = c->mesh.asm_chunk_cta[2 * q + 1];
+    auto element = c->form != GDSW_FORM_SYMMETRIC ? k_element_blocks<false, false>
+                   : newton                       ? k_element_blocks<true, true>
+                                                  : k_element_blocks<true, false>;
+    launch_chained(element, dim3(unsigned((f1 - f0 + 1) / 2)), dim3(96), 0, s, c->d_nu, T, 0.5 * c->mesh.h,
+                   c->d_dn, f0, f1 - f0, c->d_asm_ws);
+    check_launch("k_element_blocks");
+    if (cta1 > cta0) {
+      launch_chained(k_gather_blocks, dim3(unsigned(cta1 - cta0)), dim3(256), 0, s, c->d_asm_cta, cta0,
+                     c->d_asm_uoff, c->d_asm_unit, c->d_a_tpos, c->d_asm_ws, f0, f1, aval);
+      check_launch("k_gather_blocks");
+    }
+  }
   if (c->b_assembled) {  // B = -(q, div u) depends on the mesh only, not on the viscosity
     launch_sell_fill(c, false, s);
     return;

@@ -1,0 +1,51 @@
+"""The operator kernels at the sizes where their launch shapes change: one element (half an element
+CTA), an odd count, more elements than the assembly workspace holds (two chunks), both forms and
+both pressure elements, against the FP64 oracle.
+
+Tolerance: an entry is the sum of at most 8 x 27 products of five factors, each rounded a few
+times, and the products' magnitudes sum to a few times the largest entry: 216 x 4 x 1.1e-16 of it,
+rounded up to 1e-13.  Vectors (lifting, products) add at most 8 such terms per row in another
+order: the same bound on the relative 2-norm.
+"""
+import numpy as np
+import pytest
+
+from paper_2606_01433_gb300 import inputs as I
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+TOL = 1e-13
+
+
+@pytest.fixture(scope="module")
+def lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2606_01433_gb300 import gdsw
+    gdsw.load()
+    return gdsw
+
+
+def _problem(m, form, pressure):
+    kw = dict(uk_seed=3, lam=1.0, n=0.5, nu_inf=1e-3) if form == "symmetric" else {}
+    return I.box_problem(*m, (1, 1, 1), levels=2, form=form, pressure=pressure, **kw)
+
+
+@pytest.mark.parametrize("form", ["symmetric", "gradient"])
+@pytest.mark.parametrize("m,pressure", [((1, 1, 1), "q1"), ((1, 1, 2), "p1disc"), ((3, 3, 3), "q1"),
+                                        ((5, 3, 2), "p1disc"), ((21, 21, 21), "q1")])
+def test_assembled_operator(lib, m, pressure, form):
+    from oracle import fem
+    p = _problem(m, form, pressure)
+    S = fem.assemble(p)
+    ctx = lib.Context(p, levels=1)
+    A, O = ctx.gdsw_matrix_csr(), S["A"]
+    assert A.shape == O.shape
+    scale = abs(O).max() if O.nnz else 1.0
+    assert abs(A - O).max() <= TOL * scale
+    # assembled again in place: the same numbers bit for bit
+    ctx.gdsw_reassemble()
+    assert np.array_equal(ctx.gdsw_matrix_csr().data, A.data)
+    ctx.close()
