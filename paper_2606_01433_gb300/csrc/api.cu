@@ -1249,7 +1249,6 @@ void setup_impl(gdsw_ctx* c, const gdsw_mesh* mesh, const gdsw_viscosity* visc, 
   upload_tables(c, s);
   c->d_mask = c->arena.upload(M.mask, s);
   c->d_fluid = c->arena.upload(M.fluid, s);
-  c->d_felem = c->arena.upload(M.felem, s);
   c->d_vnode = c->arena.upload(M.vnode, s);
   c->d_pnode = c->arena.upload(M.pnode, s);
   c->d_a_ptr = c->arena.upload(M.a_ptr, s);
@@ -1275,19 +1274,12 @@ void setup_impl(gdsw_ctx* c, const gdsw_mesh* mesh, const gdsw_viscosity* visc, 
   c->d_b_ptr = c->arena.upload(M.b_ptr, s);
   c->d_b_col = c->arena.upload(M.b_col, s);
   c->d_bt2b = c->arena.upload(M.bt2b, s);
-  c->d_ad_ptr = c->arena.upload(M.ad_ptr, s);
-  c->d_ad_col = c->arena.upload(M.ad_col, s);
-  c->d_bd_ptr = c->arena.upload(M.bd_ptr, s);
-  c->d_bd_col = c->arena.upload(M.bd_col, s);
-  {
-    std::vector<int32_t> rows;
-    for (int64_t r = 0; r < M.nv; ++r)
-      if (M.ad_ptr[r + 1] > M.ad_ptr[r]) rows.push_back(int32_t(r));
-    for (int64_t P = 0; P < M.np; ++P)
-      if (M.bd_ptr[P + 1] > M.bd_ptr[P]) rows.push_back(int32_t(M.nv + P));
-    c->n_lift_rows = int64_t(rows.size());
-    c->d_lift_rows = rows.empty() ? nullptr : c->arena.upload(rows, s);
-  }
+  c->d_lift_elem = c->arena.upload(M.lift_elem, s);
+  c->d_lift_mask = c->arena.upload(M.lift_mask, s);
+  c->d_lift_dof = c->arena.upload(M.lift_dof, s);
+  c->d_lift_ptr = c->arena.upload(M.lift_ptr, s);
+  c->d_lift_src = c->arena.upload(M.lift_src, s);
+  c->d_lift_work = c->arena.alloc<double>(size_t(kLiftValues) * M.lift_elem.size());
   c->d_sweep_flag = c->arena.alloc<unsigned>(1);
   GDSW_CUDA(cudaMemsetAsync(c->d_sweep_flag, 0, sizeof(unsigned), s));
   c->d_gdir = c->arena.upload(M.g, s);

@@ -248,8 +248,10 @@ struct MeshHost {
   std::vector<int32_t> b_ptr, b_col;     // pressure rows x velocity node cols
   std::vector<int32_t> bt2b;             // BT entry -> B entry with the same value
   std::vector<int32_t> a_diag, a_tpos;   // position of block (I,I); position of block (J,I) for (I,J)
-  std::vector<int32_t> ad_ptr, ad_col;   // velocity rows x Dirichlet nodes with g != 0 (node ids)
-  std::vector<int32_t> bd_ptr, bd_col;   // pressure rows x Dirichlet nodes with g != 0
+  // lifting: the fluid elements with a nonzero Dirichlet datum, the bit mask of those nodes, and per
+  // affected dof its contributions (89 values per lift element: 27 x 3 velocity, 8 pressure)
+  std::vector<int32_t> lift_elem, lift_dof, lift_ptr, lift_src;
+  std::vector<uint32_t> lift_mask;
   // assembly work units: one (upper block (I, J >= I), shared fluid element) pair each, listed
   // block by block (elements in increasing index); packed fluid element << 10 | a << 5 | b
   // with a, b the local Q2 node numbers of I and J in that element
@@ -405,9 +407,9 @@ struct gdsw_ctx {
   double *d_sell_aval = nullptr, *d_sell_btval = nullptr;
   int64_t n_sell_slices = 0;
   int32_t *d_b_ptr = nullptr, *d_b_col = nullptr, *d_bt2b = nullptr;
-  int32_t *d_ad_ptr = nullptr, *d_ad_col = nullptr, *d_bd_ptr = nullptr, *d_bd_col = nullptr;
-  int32_t* d_lift_rows = nullptr;   // rows (velocity node, or nv + pressure node) with a Dirichlet neighbour
-  int64_t n_lift_rows = 0;
+  int32_t *d_lift_elem = nullptr, *d_lift_dof = nullptr, *d_lift_ptr = nullptr, *d_lift_src = nullptr;
+  uint32_t* d_lift_mask = nullptr;
+  double* d_lift_work = nullptr;    // contributions of the lift elements
   bool b_assembled = false;         // B does not depend on the viscosity: assembled once
   unsigned* d_sweep_flag = nullptr; // set by a persistent sweep whose wait ran out
   double* d_gdir = nullptr;         // Dirichlet datum, 3 per node

@@ -12,6 +12,7 @@
 #include <cmath>
 
 #include "common.h"
+#include "kernels.h"
 
 namespace gdsw {
 
@@ -185,41 +186,28 @@ static void element_nodes(const MeshHost& M, int64_t e, int64_t out[27]) {
 }
 
 // P1-disc patterns (Section 2 element pair): pressure row 4 f + k couples to the free velocity
-// nodes of fluid element f (and, for the lifting, to its Dirichlet nodes with a nonzero datum);
+// nodes of fluid element f;
 // velocity node I couples to the four pressure dofs of every fluid element holding it.  All
 // lists ascending (node order equals velocity-index order; fluid rank order equals element order).
 static void build_p1disc_patterns(MeshHost& M) {
   const int64_t nf = int64_t(M.fluid.size());
-  std::vector<int32_t> rv(nf * 27), rn(nf * 27), dv(nf * 27), dn(nf * 27);
+  std::vector<int32_t> rv(nf * 27), rn(nf);
   parallel_for(nf, [&](int64_t f) {
     int64_t nd[27];
     element_nodes(M, M.fluid[f], nd);
     std::sort(nd, nd + 27);
-    int a = 0, b = 0;
-    for (int q = 0; q < 27; ++q) {
-      const int64_t v = nd[q];
-      if (M.vidx[v] >= 0) rv[f * 27 + a++] = M.vidx[v];
-      const uint8_t t = M.tags[v];
-      const bool nz = M.g[3 * v] != 0.0 || M.g[3 * v + 1] != 0.0 || M.g[3 * v + 2] != 0.0;
-      if ((t == GDSW_TAG_WALL || t == GDSW_TAG_INFLOW) && nz) dv[f * 27 + b++] = int32_t(v);
-    }
+    int a = 0;
+    for (int q = 0; q < 27; ++q)
+      if (M.vidx[nd[q]] >= 0) rv[f * 27 + a++] = M.vidx[nd[q]];
     rn[f] = a;
-    dn[f] = b;
   });
   M.b_ptr.assign(4 * nf + 1, 0);
-  M.bd_ptr.assign(4 * nf + 1, 0);
   for (int64_t f = 0; f < nf; ++f)
-    for (int k = 0; k < 4; ++k) {
-      M.b_ptr[4 * f + k + 1] = M.b_ptr[4 * f + k] + rn[f];
-      M.bd_ptr[4 * f + k + 1] = M.bd_ptr[4 * f + k] + dn[f];
-    }
+    for (int k = 0; k < 4; ++k) M.b_ptr[4 * f + k + 1] = M.b_ptr[4 * f + k] + rn[f];
   M.b_col.resize(M.b_ptr[4 * nf]);
-  M.bd_col.resize(M.bd_ptr[4 * nf]);
   parallel_for(nf, [&](int64_t f) {
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 4; ++k)
       std::copy(rv.begin() + f * 27, rv.begin() + f * 27 + rn[f], M.b_col.begin() + M.b_ptr[4 * f + k]);
-      std::copy(dv.begin() + f * 27, dv.begin() + f * 27 + dn[f], M.bd_col.begin() + M.bd_ptr[4 * f + k]);
-    }
   });
   // velocity rows: the fluid elements holding the node, ascending
   M.bt_ptr.assign(M.nv + 1, 0);
@@ -308,28 +296,22 @@ void build_mesh(MeshHost& M, const gdsw_mesh* m) {
   M.n = M.nu + M.np;
   GDSW_CHECK(M.n < (int64_t(1) << 31), GDSW_ERR_INVALID_ARG, "problem too large for int32 dof indices");
 
-  // neighbour lists per row node, all three kinds from one scan of the neighbours: free
-  // velocity nodes, pressure nodes, Dirichlet nodes with a nonzero datum (the only ones the
-  // lifting needs); lists in increasing index
-  auto build = [&](const std::vector<int32_t>& rows, std::vector<int32_t>* ptr[3], std::vector<int32_t>* col[3]) {
+  // neighbour lists per row node, both kinds from one scan of the neighbours: free velocity nodes
+  // and pressure nodes; lists in increasing index
+  auto build = [&](const std::vector<int32_t>& rows, std::vector<int32_t>* ptr[2], std::vector<int32_t>* col[2]) {
     const int64_t nr = int64_t(rows.size());
-    std::vector<std::vector<int32_t>> tmp[3];
-    for (int k = 0; k < 3; ++k)
+    std::vector<std::vector<int32_t>> tmp[2];
+    for (int k = 0; k < 2; ++k)
       if (ptr[k]) tmp[k].resize(nr);
     parallel_for(nr, [&](int64_t r) {
       for_neighbors(M, rows[r], [&](int64_t w) {
         if (ptr[0] && M.vidx[w] >= 0) tmp[0][r].push_back(M.vidx[w]);
         if (ptr[1] && M.pidx[w] >= 0) tmp[1][r].push_back(M.pidx[w]);
-        if (ptr[2]) {
-          const uint8_t t = M.tags[w];
-          const bool nz = M.g[3 * w] != 0.0 || M.g[3 * w + 1] != 0.0 || M.g[3 * w + 2] != 0.0;
-          if ((t == GDSW_TAG_WALL || t == GDSW_TAG_INFLOW) && nz) tmp[2][r].push_back(int32_t(w));
-        }
       });
-      for (int k = 0; k < 3; ++k)
+      for (int k = 0; k < 2; ++k)
         if (ptr[k]) std::sort(tmp[k][r].begin(), tmp[k][r].end());
     });
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < 2; ++k) {
       if (!ptr[k]) continue;
       ptr[k]->assign(nr + 1, 0);
       for (int64_t r = 0; r < nr; ++r) (*ptr[k])[r + 1] = (*ptr[k])[r] + int32_t(tmp[k][r].size());
@@ -340,11 +322,11 @@ void build_mesh(MeshHost& M, const gdsw_mesh* m) {
     }
   };
   {
-    std::vector<int32_t>* vp[3] = {&M.a_ptr, &M.bt_ptr, &M.ad_ptr};
-    std::vector<int32_t>* vc[3] = {&M.a_col, &M.bt_col, &M.ad_col};
+    std::vector<int32_t>* vp[2] = {&M.a_ptr, &M.bt_ptr};
+    std::vector<int32_t>* vc[2] = {&M.a_col, &M.bt_col};
     build(M.vnode, vp, vc);
-    std::vector<int32_t>* pp[3] = {&M.b_ptr, nullptr, &M.bd_ptr};
-    std::vector<int32_t>* pc[3] = {&M.b_col, nullptr, &M.bd_col};
+    std::vector<int32_t>* pp[2] = {&M.b_ptr, nullptr};
+    std::vector<int32_t>* pc[2] = {&M.b_col, nullptr};
     build(M.pnode, pp, pc);
   }
   if (M.pdisc) {
@@ -355,6 +337,48 @@ void build_mesh(MeshHost& M, const gdsw_mesh* m) {
       GDSW_CHECK(M.vidx[nd[13]] >= 0, GDSW_ERR_INVALID_ARG, "P1-disc: an element centre node has no free velocity");
     }
     build_p1disc_patterns(M);
+  }
+  // lifting: elements with a nonzero Dirichlet datum; contributions of an affected dof in element order
+  {
+    std::vector<int32_t> cnt(M.n + 1, 0);
+    std::vector<std::pair<int32_t, int32_t>> entry;  // (dof, position in the contribution array)
+    for (int64_t f = 0; f < int64_t(M.fluid.size()); ++f) {
+      int64_t nd[27];
+      element_nodes(M, M.fluid[f], nd);
+      uint32_t mask = 0;
+      for (int a = 0; a < 27; ++a) {
+        const uint8_t t = M.tags[nd[a]];
+        if (t != GDSW_TAG_WALL && t != GDSW_TAG_INFLOW) continue;
+        if (M.g[3 * nd[a]] != 0.0 || M.g[3 * nd[a] + 1] != 0.0 || M.g[3 * nd[a] + 2] != 0.0) mask |= 1u << a;
+      }
+      if (!mask) continue;
+      const int64_t base = int64_t(M.lift_elem.size()) * kLiftValues;
+      GDSW_CHECK(base + kLiftValues < (int64_t(1) << 31), GDSW_ERR_INVALID_ARG, "too many Dirichlet elements");
+      M.lift_elem.push_back(int32_t(f));
+      M.lift_mask.push_back(mask);
+      auto add = [&](int64_t dof, int pos) {
+        ++cnt[dof + 1];
+        entry.push_back({int32_t(dof), int32_t(base + pos)});
+      };
+      for (int a = 0; a < 27; ++a)
+        if (M.vidx[nd[a]] >= 0)
+          for (int c = 0; c < 3; ++c) add(3 * int64_t(M.vidx[nd[a]]) + c, 3 * a + c);
+      if (M.pdisc) {
+        for (int k = 0; k < 4; ++k) add(M.nu + 4 * f + k, 81 + k);
+      } else {
+        for (int k = 0; k < 8; ++k) add(M.nu + M.pidx[nd[2 * (k & 1) + 6 * ((k >> 1) & 1) + 18 * (k >> 2)]], 81 + k);
+      }
+    }
+    M.lift_ptr.assign(1, 0);
+    for (int64_t d = 0; d < M.n; ++d) {
+      if (cnt[d + 1] > 0) {
+        M.lift_dof.push_back(int32_t(d));
+        M.lift_ptr.push_back(M.lift_ptr.back() + cnt[d + 1]);
+      }
+      cnt[d + 1] += cnt[d];
+    }
+    M.lift_src.resize(entry.size());
+    for (const auto& e : entry) M.lift_src[cnt[e.first]++] = e.second;
   }
   // symmetric velocity pattern: diagonal block of each row and the transpose of each block
   M.a_diag.assign(M.nv, -1);

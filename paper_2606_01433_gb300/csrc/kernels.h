@@ -26,7 +26,10 @@ struct RefTables {
   double psi[27][8];        // [q][P]
   double p1[27][4];         // [q][k]: P1-disc basis 1, xi, eta, zeta
   double w[27];
+  double div[8][27][3];     // [P][b][d]: -int psi_P d_d phi_b on the reference element
+  double div1[4][27][3];    // the same for the P1-disc basis
 };
+constexpr int kLiftValues = 89;  // per lift element: 27 x 3 velocity and up to 8 pressure contributions
 void host_tables(RefTables& T);
 
 // dense.cu

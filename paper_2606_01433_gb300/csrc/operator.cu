@@ -39,6 +39,19 @@ void host_tables(RefTables& T) {
           for (int py = 0; py < 2; ++py)
             for (int px = 0; px < 2; ++px) T.psi[q][px + 2 * py + 4 * pz] = q1(px, x) * q1(py, y) * q1(pz, z);
       }
+  for (int b = 0; b < 27; ++b)
+    for (int d = 0; d < 3; ++d) {
+      for (int k = 0; k < 8; ++k) {
+        double s = 0.0;
+        for (int q = 0; q < 27; ++q) s -= T.w[q] * T.psi[q][k] * T.dphi[q][b][d];
+        T.div[k][b][d] = s;
+      }
+      for (int k = 0; k < 4; ++k) {
+        double s = 0.0;
+        for (int q = 0; q < 27; ++q) s -= T.w[q] * T.p1[q][k] * T.dphi[q][b][d];
+        T.div1[k][b][d] = s;
+      }
+    }
 }
 
 struct Geo {
@@ -61,45 +74,113 @@ __device__ __forceinline__ int shared_range(int a, int b, int n, int& e0) {
   return e1 >= e0 ? e1 - e0 + 1 : 0;
 }
 
+// one-dimensional Q2 basis / derivative a at Gauss point q
+__host__ __device__ constexpr double gauss_x(int q) { return q == 0 ? -0.7745966692414834 : (q == 1 ? 0.0 : 0.7745966692414834); }
+__host__ __device__ constexpr double q2_v(int a, int q) {
+  const double x = gauss_x(q);
+  return a == 0 ? 0.5 * x * (x - 1.0) : (a == 1 ? 1.0 - x * x : 0.5 * x * (x + 1.0));
+}
+__host__ __device__ constexpr double q2_d(int a, int q) {
+  const double x = gauss_x(q);
+  return a == 0 ? x - 0.5 : (a == 1 ? -2.0 * x : x + 0.5);
+}
+
+// ------------------------------------------------------------------ sum factorisation on one element
+// Values of the 27 nodes of an element -> reference gradients at its 27 Gauss points, one axis at a
+// time (the Q2 basis is a tensor product: 72 multiply-adds per point and component triple instead
+// of 243).  Thread q = 0..26 of the element owns node q, then the partial results of index q, then
+// Gauss point q (x fastest throughout); u, s, t are the element's shared arrays [c][27], `sync` is
+// a barrier over the element's threads.
+struct Grad1D {
+  double v[3][3], d[3][3];   // [basis][point]
+};
+__device__ __forceinline__ void fill_grad1d(Grad1D& B, int tid) {
+  if (tid < 9) {
+    B.v[tid / 3][tid % 3] = q2_v(tid / 3, tid % 3);
+    B.d[tid / 3][tid % 3] = q2_d(tid / 3, tid % 3);
+  }
+}
+template <typename Sync>
+__device__ __forceinline__ void element_gradient(const Grad1D& B, int q, bool active, double (*u)[27],
+                                                 double (*s)[3][27], double (*t)[3][27], double gr[3][3],
+                                                 Sync sync) {
+  const int x = q % 3, y = (q / 3) % 3, z = q / 9;
+  if (active)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {  // along x: values s[0], derivatives s[1]
+      const double* p = u[c] + q - x;
+      s[0][c][q] = fma(p[2], B.v[2][x], fma(p[1], B.v[1][x], p[0] * B.v[0][x]));
+      s[1][c][q] = fma(p[2], B.d[2][x], fma(p[1], B.d[1][x], p[0] * B.d[0][x]));
+    }
+  sync();
+  if (active)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {  // along y: dx t[0], dy t[1], no derivative t[2]
+      const double* p = s[0][c] + q - 3 * y;
+      const double* d = s[1][c] + q - 3 * y;
+      t[0][c][q] = fma(d[6], B.v[2][y], fma(d[3], B.v[1][y], d[0] * B.v[0][y]));
+      t[1][c][q] = fma(p[6], B.d[2][y], fma(p[3], B.d[1][y], p[0] * B.d[0][y]));
+      t[2][c][q] = fma(p[6], B.v[2][y], fma(p[3], B.v[1][y], p[0] * B.v[0][y]));
+    }
+  sync();
+  if (active)
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int l = 0; l < 3; ++l) {
+        const double* p = t[l][c] + q - 9 * z;
+        const double(*b)[3] = l == 2 ? B.d : B.v;
+        gr[c][l] = fma(p[18], b[2][z], fma(p[9], b[1][z], p[0] * b[0][z]));
+      }
+}
+
 // ------------------------------------------------------------------ a1: Carreau viscosity
 // dn (optional, Newton linearisation of Section 3): per Gauss point D(u_k) (xx, yy, zz, xy, xz,
 // yz) and N = 4 nu'(gamma_dot) / gamma_dot = 4 (nu0 - nu_inf)(n - 1) lambda^2
 // (1 + (lambda gamma_dot)^2)^((n - 3)/2), the weight of the Newton term
-// int N (D(u_k):D(w)) (D(u_k):D(v)) of the Carreau operator's derivative
-__global__ void k_viscosity(const int32_t* __restrict__ fluid, int64_t nfe, const double* __restrict__ uk,
-                            const RefTables* __restrict__ T, Geo G, int form, int has_uk, double nu0, double nu_inf,
-                            double lam, double ncar, double* __restrict__ nu, double* __restrict__ dn) {
-  int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (t >= nfe * 27) return;
-  int64_t fe = t / 27;
-  int q = int(t - fe * 27);
+// int N (D(u_k):D(w)) (D(u_k):D(v)) of the Carreau operator's derivative.
+// Thread per Gauss point, eight elements per CTA (216 of 256 threads), the gradient by sum
+// factorisation; the FP64 pipe bounds it (the power function is now most of the work): 0.55 -> 0.33
+// ms on the 32^3 channel, 32 -> 16 us at 756 elements.
+constexpr int kViscElems = 8;
+__global__ void __launch_bounds__(256) k_viscosity(const int32_t* __restrict__ fluid, int64_t nfe,
+                                                   const double* __restrict__ uk, Geo G, int form, int has_uk,
+                                                   double nu0, double nu_inf, double lam, double ncar,
+                                                   double* __restrict__ nu, double* __restrict__ dn) {
+  __shared__ Grad1D B;
+  __shared__ double u[kViscElems][3][27], s[kViscElems][2][3][27], w[kViscElems][3][3][27];
+  dep_release();
+  dep_wait();
+  const int el = threadIdx.x / 27, q = threadIdx.x - 27 * el;
+  const int64_t fe = int64_t(blockIdx.x) * kViscElems + el, t = fe * 27 + q;
+  const bool active = el < kViscElems && fe < nfe;
   if (!has_uk || form == GDSW_FORM_GRADIENT) {
+    if (!active) return;
     nu[t] = nu0;
     if (dn)
       for (int k = 0; k < 7; ++k) dn[t * 7 + k] = 0.0;
     return;
   }
-  int e = fluid[fe];
-  int ex = e % G.nx, ey = (e / G.nx) % G.ny, ez = e / (G.nx * G.ny);
-  double gr[3][3] = {};
-  for (int a = 0; a < 27; ++a) {
-    int ax = a % 3, ay = (a / 3) % 3, az = a / 9;
-    int64_t v = (2 * ex + ax) + int64_t(G.NX) * ((2 * ey + ay) + int64_t(G.NY) * (2 * ez + az));
-    const double* dp = T->dphi[q][a];
+  fill_grad1d(B, threadIdx.x);
+  if (active) {
+    const int e = fluid[fe];
+    const int ex = e % G.nx, ey = (e / G.nx) % G.ny, ez = e / (G.nx * G.ny);
+    const int64_t v = (2 * ex + q % 3) + int64_t(G.NX) * ((2 * ey + (q / 3) % 3) + int64_t(G.NY) * (2 * ez + q / 9));
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      double u = uk[3 * v + c];
-#pragma unroll
-      for (int l = 0; l < 3; ++l) gr[c][l] = fma(u, dp[l], gr[c][l]);
-    }
+    for (int c = 0; c < 3; ++c) u[el][c][q] = uk[3 * v + c];
   }
-  const double s = 2.0 / G.h;
+  __syncthreads();
+  double gr[3][3];
+  const int se = active ? el : 0;
+  element_gradient(B, q, active, u[se], s[se], w[se], gr, [] { __syncthreads(); });
+  if (!active) return;
+  const double sc = 2.0 / G.h;
   double dd = 0.0;  // D : D
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
-      double d = 0.5 * s * (gr[c][l] + gr[l][c]);
+      double d = 0.5 * sc * (gr[c][l] + gr[l][c]);
       dd = fma(d, d, dd);
     }
   double gdot = sqrt(2.0 * dd);
@@ -107,56 +188,18 @@ __global__ void k_viscosity(const int32_t* __restrict__ fluid, int64_t nfe, cons
   nu[t] = nu_inf + (nu0 - nu_inf) * pow(1.0 + lg * lg, 0.5 * (ncar - 1.0));
   if (dn) {
     double* o = dn + t * 7;
-    o[0] = s * gr[0][0];
-    o[1] = s * gr[1][1];
-    o[2] = s * gr[2][2];
-    o[3] = 0.5 * s * (gr[0][1] + gr[1][0]);
-    o[4] = 0.5 * s * (gr[0][2] + gr[2][0]);
-    o[5] = 0.5 * s * (gr[1][2] + gr[2][1]);
+    o[0] = sc * gr[0][0];
+    o[1] = sc * gr[1][1];
+    o[2] = sc * gr[2][2];
+    o[3] = 0.5 * sc * (gr[0][1] + gr[1][0]);
+    o[4] = 0.5 * sc * (gr[0][2] + gr[2][0]);
+    o[5] = 0.5 * sc * (gr[1][2] + gr[2][1]);
     o[6] = 4.0 * (nu0 - nu_inf) * (ncar - 1.0) * lam * lam * pow(1.0 + lg * lg, 0.5 * (ncar - 3.0));
   }
 }
 
-// 3x3 velocity block between nodes I and J (Section 2 gradient form / Section 3 symmetric form)
-__device__ void velocity_block(int64_t I, int64_t J, const Geo& G, const uint8_t* mask, const int32_t* felem,
-                               const double* nu, const RefTables* T, int form, double out[9]) {
-  int ii, ij, ik, ji, jj, jk;
-  node_ijk(I, G, ii, ij, ik);
-  node_ijk(J, G, ji, jj, jk);
-#pragma unroll
-  for (int c = 0; c < 9; ++c) out[c] = 0.0;
-  int e0x, e0y, e0z;
-  int nxr = shared_range(ii, ji, G.nx, e0x), nyr = shared_range(ij, jj, G.ny, e0y), nzr = shared_range(ik, jk, G.nz, e0z);
-  const double sc = 0.5 * G.h;  // (h/2)^3 * (2/h)^2
-  for (int cz = 0; cz < nzr; ++cz)
-    for (int cy = 0; cy < nyr; ++cy)
-      for (int cx = 0; cx < nxr; ++cx) {
-        int ex = e0x + cx, ey = e0y + cy, ez = e0z + cz;
-        int64_t e = ex + int64_t(G.nx) * (ey + int64_t(G.ny) * ez);
-        if (!mask[e]) continue;
-        int fe = felem[e];
-        int a = (ii - 2 * ex) + 3 * (ij - 2 * ey) + 9 * (ik - 2 * ez);
-        int b = (ji - 2 * ex) + 3 * (jj - 2 * ey) + 9 * (jk - 2 * ez);
-        const double* nq = nu + int64_t(fe) * 27;
-        for (int q = 0; q < 27; ++q) {
-          const double* da = T->dphi[q][a];
-          const double* db = T->dphi[q][b];
-          double f = nq[q] * T->w[q] * sc;
-          double g = da[0] * db[0] + da[1] * db[1] + da[2] * db[2];
-          out[0] = fma(f, g, out[0]);
-          out[4] = fma(f, g, out[4]);
-          out[8] = fma(f, g, out[8]);
-          if (form == GDSW_FORM_SYMMETRIC) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-#pragma unroll
-              for (int d = 0; d < 3; ++d) out[c * 3 + d] = fma(f, da[d] * db[c], out[c * 3 + d]);
-          }
-        }
-      }
-}
-
-// pressure-velocity entry: -int psi_P d_d phi_J over shared fluid elements, d = 0..2
+// pressure-velocity entry: -int psi_P d_d phi_J over shared fluid elements, d = 0..2 (the
+// reference element's integrals are tabulated: they are the same on every cube of the mesh)
 __device__ void divergence_entry(int64_t P, int64_t J, const Geo& G, const uint8_t* mask, const RefTables* T,
                                  double out[3]) {
   int pi, pj, pk, ji, jj, jk;
@@ -174,13 +217,8 @@ __device__ void divergence_entry(int64_t P, int64_t J, const Geo& G, const uint8
         if (!mask[e]) continue;
         int pl = ((pi - 2 * ex) >> 1) + 2 * ((pj - 2 * ey) >> 1) + 4 * ((pk - 2 * ez) >> 1);
         int b = (ji - 2 * ex) + 3 * (jj - 2 * ey) + 9 * (jk - 2 * ez);
-        for (int q = 0; q < 27; ++q) {
-          double f = -T->w[q] * sc * T->psi[q][pl];
-          const double* db = T->dphi[q][b];
-          out[0] = fma(f, db[0], out[0]);
-          out[1] = fma(f, db[1], out[1]);
-          out[2] = fma(f, db[2], out[2]);
-        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) out[d] = fma(sc, T->div[pl][b][d], out[d]);
       }
 }
 
@@ -195,14 +233,8 @@ __device__ void divergence_entry_p1(int64_t P, int64_t J, const Geo& G, const in
   node_ijk(J, G, ji, jj, jk);
   const int b = (ji - 2 * ex) + 3 * (jj - 2 * ey) + 9 * (jk - 2 * ez);
   const double sc = 0.25 * G.h * G.h;
-  out[0] = out[1] = out[2] = 0.0;
-  for (int q = 0; q < 27; ++q) {
-    const double f = -T->w[q] * sc * T->p1[q][k];
-    const double* db = T->dphi[q][b];
-    out[0] = fma(f, db[0], out[0]);
-    out[1] = fma(f, db[1], out[1]);
-    out[2] = fma(f, db[2], out[2]);
-  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) out[d] = sc * T->div1[k][b][d];
 }
 
 // ------------------------------------------------------------------ a2: assembly
@@ -229,16 +261,6 @@ __device__ void divergence_entry_p1(int64_t P, int64_t J, const Geo& G, const in
 // meshes run chunk by chunk and the gather adds onto the blocks of the chunks before.
 constexpr int kAsmPairs = 45;
 
-// one-dimensional Q2 basis / derivative a at Gauss point q
-__host__ __device__ constexpr double gauss_x(int q) { return q == 0 ? -0.7745966692414834 : (q == 1 ? 0.0 : 0.7745966692414834); }
-__host__ __device__ constexpr double q2_v(int a, int q) {
-  const double x = gauss_x(q);
-  return a == 0 ? 0.5 * x * (x - 1.0) : (a == 1 ? 1.0 - x * x : 0.5 * x * (x + 1.0));
-}
-__host__ __device__ constexpr double q2_d(int a, int q) {
-  const double x = gauss_x(q);
-  return a == 0 ? x - 0.5 : (a == 1 ? -2.0 * x : x + 0.5);
-}
 // derivative pattern t of a one-dimensional pair: 0 value-value, 1 value-derivative (of b), 2
 // derivative-derivative
 __host__ __device__ constexpr double q2_pair(int t, int a, int b, int q) {
@@ -493,51 +515,105 @@ __global__ void k_copy_bt(const int32_t* __restrict__ bt2b, int64_t nbt, const d
   btval[e * 3 + 2] = bval[s * 3 + 2];
 }
 
-// b = -A_(free, D) g_D.  One warp per row that has a Dirichlet neighbour with g != 0 (the
-// rows are listed at set-up; every other entry of b is zero); the lanes take the row's
-// Dirichlet neighbours and the warp sums them with a fixed butterfly.
-__global__ void __launch_bounds__(256) k_lift(const int32_t* __restrict__ rows, int64_t nrows,
-                                              const int32_t* ad_ptr, const int32_t* ad_col, const int32_t* vnode,
-                                              int64_t nv, const int32_t* bd_ptr, const int32_t* bd_col,
-                                              const int32_t* pnode, const int32_t* pfluid, Geo G,
-                                              const uint8_t* mask, const int32_t* felem, const double* nu,
-                                              const RefTables* T, int form, const double* g, double* b) {
-  const int64_t w = blockIdx.x * int64_t(blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
-  if (w >= nrows) return;
-  const int64_t row = rows[w];
-  if (row < nv) {
-    double acc[3] = {0, 0, 0};
-    for (int e = ad_ptr[row] + lane; e < ad_ptr[row + 1]; e += 32) {
-      int64_t J = ad_col[e];
-      double blk[9];
-      velocity_block(vnode[row], J, G, mask, felem, nu, T, form, blk);
+// b = -A_(free, D) g_D, element by element: the operator applied to the Dirichlet field on the
+// elements that carry a nonzero datum (listed at set-up; every other entry of b is zero), then the
+// sum over those elements per affected dof in element order.  One warp per element, lane = Gauss
+// point / node; gradient, stress and test gradients by sum factorisation.  The block of every
+// (row, Dirichlet node) pair, one lane each as before, was a serial chain of 27 points x 8
+// elements: 147 us whatever the mesh and 0.80 ms on the 32^3 channel; now 14 + 5 and 18 + 7 us.
+__global__ void __launch_bounds__(128) k_lift_elements(const int32_t* __restrict__ lift_elem,
+                                                       const uint32_t* __restrict__ lift_mask, int64_t nle,
+                                                       const int32_t* __restrict__ fluid, Geo G, int form, int pdisc,
+                                                       const double* __restrict__ nu, const RefTables* __restrict__ T,
+                                                       const double* __restrict__ g, double* __restrict__ lw) {
+  __shared__ Grad1D B;
+  __shared__ double su[4][3][27], ss[4][3][3][27], st[4][3][3][27];
+  __shared__ double sdiv[4][27];
+  dep_release();
+  dep_wait();
+  fill_grad1d(B, threadIdx.x);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, q = threadIdx.x & 31;
+  const int64_t le = int64_t(blockIdx.x) * 4 + warp;
+  if (le >= nle) return;
+  const bool active = q < 27;
+  const int64_t fe = lift_elem[le];
+  double (*u)[27] = su[warp];
+  double (*s)[3][27] = ss[warp];
+  double (*t)[3][27] = st[warp];
+  if (active) {
+    const int e = fluid[fe];
+    const int ex = e % G.nx, ey = (e / G.nx) % G.ny, ez = e / (G.nx * G.ny);
+    const int64_t v = (2 * ex + q % 3) + int64_t(G.NX) * ((2 * ey + (q / 3) % 3) + int64_t(G.NY) * (2 * ez + q / 9));
+    const bool dir = (lift_mask[le] >> q) & 1u;
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) acc[c] = fma(blk[c * 3 + d], g[3 * J + d], acc[c]);
-    }
+    for (int c = 0; c < 3; ++c) u[c][q] = dir ? g[3 * v + c] : 0.0;
+  }
+  __syncwarp();
+  double gr[3][3];
+  element_gradient(B, q, active, u, s, t, gr, [] { __syncwarp(); });
+  __syncwarp();
+  const int x = q % 3, y = (q / 3) % 3, z = q / 9;
+  if (active) {
+    const double w = T->w[q], f = nu[fe * 27 + q] * w * (0.5 * G.h);
+    sdiv[warp][q] = (gr[0][0] + gr[1][1] + gr[2][2]) * w * (0.25 * G.h * G.h);
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-    if (lane < 3) b[3 * row + lane] = -(lane == 0 ? acc[0] : (lane == 1 ? acc[1] : acc[2]));
-  } else {
-    const int64_t P = row - nv;
-    double acc = 0.0;
-    for (int e = bd_ptr[P] + lane; e < bd_ptr[P + 1]; e += 32) {
-      int64_t J = bd_col[e];
-      double v[3];
-      if (pfluid)
-        divergence_entry_p1(P, J, G, pfluid, T, v);
-      else
-        divergence_entry(pnode[P], J, G, mask, T, v);
-      acc = fma(v[0], g[3 * J], fma(v[1], g[3 * J + 1], fma(v[2], g[3 * J + 2], acc)));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) b[3 * nv + P] = -acc;
+      for (int l = 0; l < 3; ++l) s[c][l][q] = f * (form == GDSW_FORM_SYMMETRIC ? gr[c][l] + gr[l][c] : gr[c][l]);
   }
+  __syncwarp();
+  if (active)  // test functions along z
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int l = 0; l < 3; ++l) {
+        const double* p = s[c][l] + q - 9 * z;
+        const double* b = l == 2 ? B.d[z] : B.v[z];
+        t[c][l][q] = fma(p[18], b[2], fma(p[9], b[1], p[0] * b[0]));
+      }
+  __syncwarp();
+  if (active)  // along y: s[c][0] still needs the x derivative, s[c][1] the x value
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double *p0 = t[c][0] + q - 3 * y, *p1 = t[c][1] + q - 3 * y, *p2 = t[c][2] + q - 3 * y;
+      double a = 0.0, b = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        a = fma(p0[3 * k], B.v[y][k], a);
+        b = fma(p1[3 * k], B.d[y][k], fma(p2[3 * k], B.v[y][k], b));
+      }
+      s[c][0][q] = a;
+      s[c][1][q] = b;
+    }
+  __syncwarp();
+  double* o = lw + le * kLiftValues;
+  if (active)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double *p0 = s[c][0] + q - x, *p1 = s[c][1] + q - x;
+      double a = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) a = fma(p0[k], B.d[x][k], fma(p1[k], B.v[x][k], a));
+      o[3 * q + c] = -a;
+    }
+  if (q < (pdisc ? 4 : 8)) {
+    double a = 0.0;
+    for (int k = 0; k < 27; ++k) a = fma(sdiv[warp][k], pdisc ? T->p1[k][q] : T->psi[k][q], a);
+    o[81 + q] = a;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_lift_gather(const int32_t* __restrict__ dof, const int32_t* __restrict__ ptr,
+                                                     const int32_t* __restrict__ src, int64_t ndof,
+                                                     const double* __restrict__ lw, double* __restrict__ b) {
+  dep_release();
+  dep_wait();
+  const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (i >= ndof) return;
+  double a = 0.0;
+  for (int32_t e = ptr[i]; e < ptr[i + 1]; ++e) a += lw[src[e]];
+  b[dof[i]] = a;
 }
 
 // ------------------------------------------------------------------ a3: SpMV
@@ -550,6 +626,8 @@ __global__ void __launch_bounds__(256) k_lift(const int32_t* __restrict__ rows, 
 // y = A x or y = b - A x.
 __global__ void k_sell_fill(const int32_t* __restrict__ src, int64_t nslots, int m, const double* __restrict__ from,
                             double* __restrict__ to) {
+  dep_release();
+  dep_wait();
   const int64_t slot = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (slot >= nslots) return;
   const int64_t g = slot >> 5;
@@ -683,6 +761,8 @@ void upload_tables(gdsw_ctx* c, cudaStream_t s) {
 // solve order); the Dirichlet nodes keep their data g (copied before this kernel)
 __global__ void k_picard_velocity(const int32_t* __restrict__ vnode, int64_t nv, const double* __restrict__ x,
                                   double* __restrict__ uk) {
+  dep_release();
+  dep_wait();
   const int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (q >= 3 * nv) return;
   const int64_t I = q / 3;
@@ -704,18 +784,17 @@ void launch_picard_velocity(gdsw_ctx* c, const double* x, cudaStream_t s) {
   const int64_t nv = c->mesh.nv;
   GDSW_CUDA(cudaMemcpyAsync(c->d_uk, c->d_gdir, sizeof(double) * 3 * c->mesh.nnodes, cudaMemcpyDeviceToDevice, s));
   if (nv > 0) {
-    k_picard_velocity<<<int((3 * nv + 255) / 256), 256, 0, s>>>(c->d_vnode, nv, x, c->d_uk);
+    launch_chained(k_picard_velocity, dim3(unsigned((3 * nv + 255) / 256)), dim3(256), 0, s, c->d_vnode, nv, x,
+                   c->d_uk);
     check_launch("k_picard_velocity");
   }
   c->has_uk = true;
 }
 
 void launch_viscosity(gdsw_ctx* c, cudaStream_t s) {
-  int64_t nfe = int64_t(c->mesh.fluid.size());
-  int64_t n = nfe * 27;
-  k_viscosity<<<int((n + 255) / 256), 256, 0, s>>>(c->d_fluid, nfe, c->d_uk, static_cast<RefTables*>(c->d_tables),
-                                                  geo(c), c->form, c->has_uk ? 1 : 0, c->nu0, c->nu_inf, c->lam,
-                                                  c->ncar, c->d_nu, c->d_dn);
+  const int64_t nfe = int64_t(c->mesh.fluid.size());
+  launch_chained(k_viscosity, dim3(unsigned((nfe + kViscElems - 1) / kViscElems)), dim3(256), 0, s, c->d_fluid, nfe,
+                 c->d_uk, geo(c), c->form, c->has_uk ? 1 : 0, c->nu0, c->nu_inf, c->lam, c->ncar, c->d_nu, c->d_dn);
   check_launch("k_viscosity");
 }
 
@@ -757,16 +836,17 @@ void launch_assembly(gdsw_ctx* c, cudaStream_t s, bool newton) {
 }
 
 void launch_lift(gdsw_ctx* c, double* b, cudaStream_t s) {
-  int64_t nv = c->mesh.nv, np = c->mesh.np;
   // every entry of b not written below (rows without a Dirichlet neighbour) is zero
-  GDSW_CUDA(cudaMemsetAsync(b, 0, size_t(3 * nv + np) * sizeof(double), s));
-  if (c->n_lift_rows == 0) return;
-  k_lift<<<int((c->n_lift_rows + 7) / 8), 256, 0, s>>>(c->d_lift_rows, c->n_lift_rows, c->d_ad_ptr, c->d_ad_col,
-                                                       c->d_vnode, nv, c->d_bd_ptr, c->d_bd_col, c->d_pnode,
-                                                       c->mesh.pdisc ? c->d_fluid : nullptr, geo(c),
-                                                       c->d_mask, c->d_felem, c->d_nu,
-                                                       static_cast<RefTables*>(c->d_tables), c->form, c->d_gdir, b);
-  check_launch("k_lift");
+  GDSW_CUDA(cudaMemsetAsync(b, 0, size_t(c->mesh.n) * sizeof(double), s));
+  const int64_t nle = int64_t(c->mesh.lift_elem.size()), nd = int64_t(c->mesh.lift_dof.size());
+  if (nle == 0 || nd == 0) return;
+  launch_chained(k_lift_elements, dim3(unsigned((nle + 3) / 4)), dim3(128), 0, s, c->d_lift_elem, c->d_lift_mask, nle,
+                 c->d_fluid, geo(c), c->form, c->mesh.pdisc ? 1 : 0, c->d_nu, static_cast<RefTables*>(c->d_tables),
+                 c->d_gdir, c->d_lift_work);
+  check_launch("k_lift_elements");
+  launch_chained(k_lift_gather, dim3(unsigned((nd + 255) / 256)), dim3(256), 0, s, c->d_lift_dof, c->d_lift_ptr,
+                 c->d_lift_src, nd, c->d_lift_work, b);
+  check_launch("k_lift_gather");
 }
 
 void launch_spmv(gdsw_ctx* c, const double* x, double* y, const double* rhs, cudaStream_t s) {
@@ -785,12 +865,13 @@ void launch_sell_fill(gdsw_ctx* c, bool with_bt, cudaStream_t s) {
   const MeshHost& M = c->mesh;
   const int64_t na = int64_t(M.sell_acol.size()), nb = int64_t(M.sell_bcol.size());
   if (na > 0) {
-    k_sell_fill<<<int((na + 255) / 256), 256, 0, s>>>(c->d_sell_asrc, na, 9, c->d_val, c->d_sell_aval);
+    launch_chained(k_sell_fill, dim3(unsigned((na + 255) / 256)), dim3(256), 0, s, c->d_sell_asrc, na, 9, c->d_val,
+                   c->d_sell_aval);
     check_launch("k_sell_fill");
   }
   if (with_bt && nb > 0) {
-    k_sell_fill<<<int((nb + 255) / 256), 256, 0, s>>>(c->d_sell_bsrc, nb, 3, c->d_val + 9 * c->nnzb,
-                                                      c->d_sell_btval);
+    launch_chained(k_sell_fill, dim3(unsigned((nb + 255) / 256)), dim3(256), 0, s, c->d_sell_bsrc, nb, 3,
+                   c->d_val + 9 * c->nnzb, c->d_sell_btval);
     check_launch("k_sell_fill");
   }
 }

@@ -49,3 +49,26 @@ def test_assembled_operator(lib, m, pressure, form):
     ctx.gdsw_reassemble()
     assert np.array_equal(ctx.gdsw_matrix_csr().data, A.data)
     ctx.close()
+
+
+@pytest.mark.parametrize("form", ["symmetric", "gradient"])
+@pytest.mark.parametrize("m,pressure", [((1, 1, 2), "q1"), ((3, 3, 3), "p1disc"), ((5, 3, 2), "q1"), ((9, 4, 7), "p1disc")])
+def test_viscosity_and_lifting(lib, m, pressure, form):
+    """Gauss-point viscosity and lifted right-hand side: element counts around the eight elements of
+    a viscosity CTA and the four of a lifting CTA; a Dirichlet datum on wall and inflow nodes."""
+    from oracle import fem
+    p = _problem(m, form, pressure)
+    rng = np.random.default_rng(5)
+    dirichlet = np.isin(p.tags, (I.TAG_WALL, I.TAG_INFLOW))
+    p.g[dirichlet & (rng.random(p.n_nodes) < 0.4)] = rng.standard_normal(3)
+    p.g[~dirichlet] = 7.0   # not a datum: must not be read
+    S = fem.assemble(p)
+    ctx = lib.Context(p, levels=1)
+    nu = ctx.gdsw_viscosity_values()
+    assert np.linalg.norm(nu - S["nu_q"]) <= TOL * np.linalg.norm(S["nu_q"])
+    b = torch.full((ctx.n,), float("nan"), dtype=torch.float64, device="cuda")
+    ctx.gdsw_rhs_lift(b)
+    bo = fem.lifted_rhs(S)
+    torch.cuda.synchronize()
+    assert np.linalg.norm(b.cpu().numpy() - bo) <= TOL * max(np.linalg.norm(bo), 1e-300)
+    ctx.close()
