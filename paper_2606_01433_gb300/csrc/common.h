@@ -137,6 +137,8 @@ inline size_t elem_size(int prec) { return prec == GDSW_FP64 ? 8 : (prec == GDSW
 // are five full waves of the element kernel (152 SMs, 6 CTAs of 2 elements) and 266 MB.
 constexpr int64_t kAsmChunk = 9120;
 constexpr int64_t kAsmElemValues = 405 * 9;
+// velocity nodes up to which the SpMV uses slices of 8 rows (build_sell)
+constexpr int64_t kSellNarrow = 45000;
 inline int64_t pad8(int64_t x) { return (x + 7) & ~int64_t(7); }
 
 // ------------------------------------------------------------------ device task descriptors
@@ -260,10 +262,12 @@ struct MeshHost {
   std::vector<int32_t> asm_cta;          // first block of each assembly CTA (<= 256 units), + nnzb
   std::vector<int64_t> asm_chunk;        // fluid elements assembled at a time: chunk bounds
   std::vector<int32_t> asm_chunk_cta;    // per chunk: range of the assembly CTAs it touches
-  // sliced copy of the velocity rows for the SpMV (32 rows per slice, rows sorted by length
-  // inside windows of 1024 rows so that a slice's rows have near-equal lengths): slot
-  // j * 32 + lane of slice s holds the j-th block (or B^T entry) of the slice's lane-th row
-  std::vector<int32_t> sell_row;         // nslices * 32: velocity row or -1
+  // sliced copy of the velocity rows for the SpMV (sell_c = 32 or 8 rows per slice, rows sorted by
+  // length inside windows of 1024 rows so that a slice's rows have near-equal lengths; CW = 32 /
+  // sell_c): slot (j / CW) * 32 + r * CW + j % CW of slice s holds the j-th block (or B^T entry)
+  // of the slice's r-th row
+  int sell_c = 32;
+  std::vector<int32_t> sell_row;         // nslices * sell_c: velocity row or -1
   std::vector<int64_t> sell_aoff, sell_boff;  // nslices + 1: first block / B^T slot of each slice
   std::vector<int32_t> sell_acol, sell_asrc;  // per block slot: column node, source block (-1: pad)
   std::vector<int32_t> sell_bcol, sell_bsrc;  // per B^T slot: pressure column, source entry (-1: pad)

@@ -139,36 +139,56 @@ static void build_sell(MeshHost& M) {
       return x < y;
     });
   });
-  const int64_t ns = (nv + 31) / 32;
-  M.sell_row.assign(ns * 32, -1);
+  // Slices of C rows; a slot group of 32 holds CW = 32 / C consecutive blocks of each.  Wide slices
+  // (32 rows, one block each) end in the fewest partial sums; small operators take narrow ones,
+  // whose longest row is a quarter of the FP64 work of one SM's longest slice (k_spmv).
+  const int C = nv <= kSellNarrow ? 8 : 32, CW = 32 / C;
+  M.sell_c = C;
+  // slices numbered by decreasing length (equal lengths in row order), so that a launch over them
+  // starts with the longest and ends with the shortest
+  const int64_t ns = (nv + C - 1) / C;
+  {
+    std::vector<int32_t> len(ns, 0), rank(ns);
+    for (int64_t sl = 0; sl < ns; ++sl) {
+      rank[sl] = int32_t(sl);
+      for (int64_t r = sl * C; r < std::min(nv, sl * C + C); ++r) len[sl] = std::max(len[sl], alen(order[r]));
+    }
+    if (nv % C) len[ns - 1] = -1;  // the partly filled slice stays last
+    std::stable_sort(rank.begin(), rank.end(), [&](int32_t x, int32_t y) { return len[x] > len[y]; });
+    std::vector<int32_t> by_length(nv);
+    for (int64_t sl = 0, p = 0; sl < ns; ++sl)
+      for (int64_t r = int64_t(rank[sl]) * C; r < std::min(nv, int64_t(rank[sl]) * C + C); ++r) by_length[p++] = order[r];
+    order.swap(by_length);
+  }
+  M.sell_row.assign(ns * C, -1);
   M.sell_aoff.assign(ns + 1, 0);
   M.sell_boff.assign(ns + 1, 0);
   for (int64_t sl = 0; sl < ns; ++sl) {
     int la = 0, lb = 0;
-    for (int l = 0; l < 32 && sl * 32 + l < nv; ++l) {
-      const int32_t r = order[sl * 32 + l];
-      M.sell_row[sl * 32 + l] = r;
+    for (int l = 0; l < C && sl * C + l < nv; ++l) {
+      const int32_t r = order[sl * C + l];
+      M.sell_row[sl * C + l] = r;
       la = std::max(la, alen(r));
       lb = std::max(lb, blen(r));
     }
-    M.sell_aoff[sl + 1] = M.sell_aoff[sl] + int64_t(la) * 32;
-    M.sell_boff[sl + 1] = M.sell_boff[sl] + int64_t(lb) * 32;
+    M.sell_aoff[sl + 1] = M.sell_aoff[sl] + int64_t((la + CW - 1) / CW) * 32;
+    M.sell_boff[sl + 1] = M.sell_boff[sl] + int64_t((lb + CW - 1) / CW) * 32;
   }
   M.sell_acol.assign(M.sell_aoff[ns], 0);
   M.sell_asrc.assign(M.sell_aoff[ns], -1);
   M.sell_bcol.assign(M.sell_boff[ns], 0);
   M.sell_bsrc.assign(M.sell_boff[ns], -1);
   parallel_for(ns, [&](int64_t sl) {
-    for (int l = 0; l < 32; ++l) {
-      const int32_t r = M.sell_row[sl * 32 + l];
+    for (int l = 0; l < C; ++l) {
+      const int32_t r = M.sell_row[sl * C + l];
       if (r < 0) continue;
       for (int j = 0; j < alen(r); ++j) {
-        const int64_t slot = M.sell_aoff[sl] + int64_t(j) * 32 + l;
+        const int64_t slot = M.sell_aoff[sl] + int64_t(j / CW) * 32 + l * CW + j % CW;
         M.sell_acol[slot] = M.a_col[M.a_ptr[r] + j];
         M.sell_asrc[slot] = M.a_ptr[r] + j;
       }
       for (int j = 0; j < blen(r); ++j) {
-        const int64_t slot = M.sell_boff[sl] + int64_t(j) * 32 + l;
+        const int64_t slot = M.sell_boff[sl] + int64_t(j / CW) * 32 + l * CW + j % CW;
         M.sell_bcol[slot] = M.bt_col[M.bt_ptr[r] + j];
         M.sell_bsrc[slot] = M.bt_ptr[r] + j;
       }

@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(256) k_lift_gather(const int32_t* __restrict__
 // so each FP64 warp instruction has all 32 lanes busy.  Slot group g (32 slots, one per lane)
 // keeps its 3x3 blocks component-major: value m of lane l at g * 288 + m * 32 + l (B^T: at
 // g * 96 + m * 32 + l), so every value load is one coalesced 256-byte access.
-// Pressure rows: one warp per row streaming the contiguous 3-vectors of B.  FP64 throughout;
+// Pressure rows: LPR lanes per row, lane = entry (a contiguous 3-vector of B).  FP64 throughout;
 // y = A x or y = b - A x.
 __global__ void k_sell_fill(const int32_t* __restrict__ src, int64_t nslots, int m, const double* __restrict__ from,
                             double* __restrict__ to) {
@@ -636,106 +636,143 @@ __global__ void k_sell_fill(const int32_t* __restrict__ src, int64_t nslots, int
   for (int c = 0; c < m; ++c) to[g * (32 * m) + c * 32 + lane] = e >= 0 ? from[int64_t(e) * m + c] : 0.0;
 }
 
-__device__ __forceinline__ void sell_block(const int32_t* __restrict__ acol, const double* __restrict__ aval,
-                                           const double* __restrict__ x, int64_t g, int lane, double& a0, double& a1,
-                                           double& a2) {
-  const int64_t j = __ldg(acol + g * 32 + lane);
-  const double x0 = __ldg(x + 3 * j), x1 = __ldg(x + 3 * j + 1), x2 = __ldg(x + 3 * j + 2);
-  const double* v = aval + g * 288 + lane;
-  const double v0 = __ldcs(v), v1 = __ldcs(v + 32), v2 = __ldcs(v + 64), v3 = __ldcs(v + 96), v4 = __ldcs(v + 128),
-               v5 = __ldcs(v + 160), v6 = __ldcs(v + 192), v7 = __ldcs(v + 224), v8 = __ldcs(v + 256);
-  a0 = fma(v2, x2, fma(v1, x1, fma(v0, x0, a0)));
-  a1 = fma(v5, x2, fma(v4, x1, fma(v3, x0, a1)));
-  a2 = fma(v8, x2, fma(v7, x1, fma(v6, x0, a2)));
+// operator values: evict-first when the operator is larger than L2, kept there otherwise
+template <bool STREAM>
+__device__ __forceinline__ double ldv(const double* p) {
+  return STREAM ? __ldcs(p) : __ldg(p);
 }
 
-// Velocity part: CTA b takes slices 2b and 2b + 1, four warps per slice; warp k of a slice
-// takes the slot groups g = g0 + k, g0 + k + 4, ... (two in flight), and the four partial
-// sums of a row are added in warp order.  CTAs from ceil(nslices / 2) on take 8 pressure rows.
-__global__ void __launch_bounds__(256) k_spmv(const int32_t* __restrict__ sell_row, const int64_t* __restrict__ aoff,
-                                              const int32_t* __restrict__ acol, const double* __restrict__ aval,
-                                              const int64_t* __restrict__ boff, const int32_t* __restrict__ bcol,
-                                              const double* __restrict__ btval, int64_t nslices,
-                                              const int32_t* __restrict__ b_ptr, const int32_t* __restrict__ b_col,
-                                              const double* __restrict__ bval, int64_t nv, int64_t np,
-                                              const double* __restrict__ x, double* __restrict__ y,
-                                              const double* __restrict__ rhs) {
-  __shared__ double red[8][3][32];
+struct SpmvArgs {
+  const int32_t* sell_row;
+  const int64_t* aoff;
+  const int32_t* acol;
+  const double* aval;
+  const int64_t* boff;
+  const int32_t* bcol;
+  const double* btval;
+  int64_t nslices;
+  const int32_t *b_ptr, *b_col;
+  const double* bval;
+  int64_t nv, np;
+  const double* x;
+  double* y;
+  const double* rhs;
+};
+
+// W warps share a slice of C rows (32, or 8 with four lanes per row): warp w takes the slot groups
+// w, w + W, ... (two in flight); the partial sums of a row are added over its lanes, then in warp
+// order.  NWARP warps a CTA.  Slices are numbered by decreasing length (build_sell) and the
+// pressure rows come last, so the launch ends on its shortest CTAs.
+// Bounds: the FP64 pipe (one warp instruction per 16 cycles and SM) for large operators -- 152
+// million multiply-adds, 241 us, on the 32^3 channel: 264 us, 286 before the numbering by length
+// and the shared butterflies of the pressure rows.  For small ones the pipe of the one SM that
+// holds a slice of the longest rows (125 blocks x 32 rows: 1200 warp instructions, 9 us) and the
+// chain of dependent column and vector loads along a row: hence slices of 8 rows, four lanes and up
+// to four warps a row, one slice a CTA, columns one pass ahead, values left in L2.
+// Launched in plain stream order: with programmatic dependent launch the CTAs are placed beside the
+// previous kernel's, unevenly, and the 8^3 product took 19 instead of 12 us.
+template <int C, int W, int NWARP, int LPR>
+__global__ void __launch_bounds__(32 * NWARP) k_spmv(const SpmvArgs a) {
+  constexpr int SPC = NWARP / W, CW = 32 / C;
+  constexpr bool STREAM = C == 32;
+  __shared__ double red[NWARP][3][C];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t nu = 3 * nv;
-  const int64_t vblocks = (nslices + 1) / 2;
-  // launched in plain stream order (chained, it measured slower than the launch latency it
-  // hid); it lets its chained successor start early
+  const int64_t nu = 3 * a.nv;
+  const int64_t vblocks = (a.nslices + SPC - 1) / SPC;
+  const double* __restrict__ x = a.x;
   dep_release();
   if (blockIdx.x < vblocks) {
-    const int64_t sl = 2 * int64_t(blockIdx.x) + (warp >> 2);
-    const int sub = warp & 3;
+    const int64_t sl = SPC * int64_t(blockIdx.x) + warp / W;
+    const int sub = warp % W;
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    if (sl < nslices) {
-      const int64_t g0 = aoff[sl] >> 5, g1 = aoff[sl + 1] >> 5;
-      int64_t g = g0 + sub;
-      // two slot groups per pass, their loads independent of the accumulators (so both are in
+    if (sl < a.nslices) {
+      const int64_t g0 = a.aoff[sl] >> 5, g1 = a.aoff[sl + 1] >> 5;
+      const int64_t h0 = a.boff[sl] >> 5, h1 = a.boff[sl + 1] >> 5;
+      // NG slot groups per pass, their loads independent of the accumulators (so all are in
       // flight at once) and their products chained into the same three sums: no extra FP64
-      // adds to merge partial sums, since the FP64 pipe, not memory, bounds this loop
-      for (; g + 4 < g1; g += 8) {
-        const int64_t j = __ldg(acol + g * 32 + lane), k = __ldg(acol + (g + 4) * 32 + lane);
-        const double* v = aval + g * 288 + lane;
-        const double* w = aval + (g + 4) * 288 + lane;
-        double vv[9], ww[9];
+      // adds to merge partial sums.  The columns run one pass ahead: a pass waits for one load
+      // (its vector entries), not for two in a row.
+      constexpr int NG = 2;
+      int32_t j[NG];
+      auto columns = [&](int64_t g) {
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-          vv[q] = __ldcs(v + 32 * q);
-          ww[q] = __ldcs(w + 32 * q);
-        }
-        const double x0 = __ldg(x + 3 * j), x1 = __ldg(x + 3 * j + 1), x2 = __ldg(x + 3 * j + 2);
-        const double y0 = __ldg(x + 3 * k), y1 = __ldg(x + 3 * k + 1), y2 = __ldg(x + 3 * k + 2);
-        a0 = fma(vv[2], x2, fma(vv[1], x1, fma(vv[0], x0, a0)));
-        a1 = fma(vv[5], x2, fma(vv[4], x1, fma(vv[3], x0, a1)));
-        a2 = fma(vv[8], x2, fma(vv[7], x1, fma(vv[6], x0, a2)));
-        a0 = fma(ww[2], y2, fma(ww[1], y1, fma(ww[0], y0, a0)));
-        a1 = fma(ww[5], y2, fma(ww[4], y1, fma(ww[3], y0, a1)));
-        a2 = fma(ww[8], y2, fma(ww[7], y1, fma(ww[6], y0, a2)));
+        for (int k = 0; k < NG; ++k) j[k] = g + k * W < g1 ? __ldg(a.acol + (g + k * W) * 32 + lane) : 0;
+      };
+      columns(g0 + sub);
+      for (int64_t g = g0 + sub; g < g1; g += NG * W) {
+        double v[NG][9], xv[NG][3];
+#pragma unroll
+        for (int k = 0; k < NG; ++k)
+#pragma unroll
+          for (int q = 0; q < 3; ++q) xv[k][q] = __ldg(x + 3 * int64_t(j[k]) + q);
+#pragma unroll
+        for (int k = 0; k < NG; ++k)
+          if (k == 0 || g + k * W < g1)
+#pragma unroll
+            for (int q = 0; q < 9; ++q) v[k][q] = ldv<STREAM>(a.aval + (g + k * W) * 288 + lane + 32 * q);
+        columns(g + NG * W);
+#pragma unroll
+        for (int k = 0; k < NG; ++k)
+          if (k == 0 || g + k * W < g1) {
+            a0 = fma(v[k][2], xv[k][2], fma(v[k][1], xv[k][1], fma(v[k][0], xv[k][0], a0)));
+            a1 = fma(v[k][5], xv[k][2], fma(v[k][4], xv[k][1], fma(v[k][3], xv[k][0], a1)));
+            a2 = fma(v[k][8], xv[k][2], fma(v[k][7], xv[k][1], fma(v[k][6], xv[k][0], a2)));
+          }
       }
-      if (g < g1) sell_block(acol, aval, x, g, lane, a0, a1, a2);
-      const int64_t h0 = boff[sl] >> 5, h1 = boff[sl + 1] >> 5;
-      for (int64_t h = h0 + sub; h < h1; h += 4) {
-        const double xp = __ldg(x + nu + __ldg(bcol + h * 32 + lane));
-        const double* v = btval + h * 96 + lane;
-        a0 = fma(__ldcs(v + 0), xp, a0);
-        a1 = fma(__ldcs(v + 32), xp, a1);
-        a2 = fma(__ldcs(v + 64), xp, a2);
+#pragma unroll 2
+      for (int64_t h = h0 + sub; h < h1; h += W) {
+        const double xp = __ldg(x + nu + __ldg(a.bcol + h * 32 + lane));
+        const double* v = a.btval + h * 96 + lane;
+        a0 = fma(ldv<STREAM>(v + 0), xp, a0);
+        a1 = fma(ldv<STREAM>(v + 32), xp, a1);
+        a2 = fma(ldv<STREAM>(v + 64), xp, a2);
       }
     }
-    red[warp][0][lane] = a0;
-    red[warp][1][lane] = a1;
-    red[warp][2][lane] = a2;
-    __syncthreads();
-    if (sub == 0 && sl < nslices) {
-      const int32_t row = sell_row[sl * 32 + lane];
-      if (row >= 0) {
-        const int64_t o = 3 * int64_t(row);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          double t = red[warp][c][lane];
+    for (int o = CW / 2; o > 0; o >>= 1) {
+      a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+      a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+      a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+    }
+    if (lane % CW == 0) {
+      red[warp][0][lane / CW] = a0;
+      red[warp][1][lane / CW] = a1;
+      red[warp][2][lane / CW] = a2;
+    }
+    if (W > 1)
+      __syncthreads();
+    else
+      __syncwarp();
+    if (sub == 0 && sl < a.nslices) {
+      for (int i = lane; i < 3 * C; i += 32) {
+        const int r = i % C, c = i / C;
+        const int32_t row = a.sell_row[sl * C + r];
+        if (row < 0) continue;
+        double t = red[warp][c][r];
 #pragma unroll
-          for (int k = 1; k < 4; ++k) t += red[warp + k][c][lane];
-          y[o + c] = rhs ? rhs[o + c] - t : t;
-        }
+        for (int k = 1; k < W; ++k) t += red[warp + k][c][r];
+        const int64_t o = 3 * int64_t(row) + c;
+        a.y[o] = a.rhs ? a.rhs[o] - t : t;
       }
     }
   } else {
-    const int64_t P = (int64_t(blockIdx.x) - vblocks) * 8 + warp;
-    if (P >= np) return;
-    const int64_t f0 = int64_t(b_ptr[P]) * 3, f1 = int64_t(b_ptr[P + 1]) * 3;
+    // LPR lanes per pressure row, four entries of a lane in flight; one butterfly over the LPR lanes
+    // serves all rows of the warp
+    constexpr int RPW = 32 / LPR;
+    const int64_t P = ((int64_t(blockIdx.x) - vblocks) * NWARP + warp) * RPW + lane / LPR;
+    const int sub = lane % LPR;
+    const int32_t e0 = P < a.np ? a.b_ptr[P] : 0, e1 = P < a.np ? a.b_ptr[P + 1] : 0;
     double acc = 0.0;
-    for (int64_t f = f0 + lane; f < f1; f += 32) {
-      const int64_t e = f / 3;
-      const int d = int(f - 3 * e);
-      acc = fma(__ldcs(bval + f), __ldg(x + 3 * int64_t(b_col[e]) + d), acc);
+#pragma unroll 4
+    for (int32_t e = e0 + sub; e < e1; e += LPR) {
+      const int64_t j = 3 * int64_t(__ldg(a.b_col + e));
+      const double* v = a.bval + 3 * int64_t(e);
+      acc = fma(ldv<STREAM>(v + 2), __ldg(x + j + 2),
+                fma(ldv<STREAM>(v + 1), __ldg(x + j + 1), fma(ldv<STREAM>(v), __ldg(x + j), acc)));
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) y[nu + P] = rhs ? rhs[nu + P] - acc : acc;
+    for (int o = LPR / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (sub == 0 && P < a.np) a.y[nu + P] = a.rhs ? a.rhs[nu + P] - acc : acc;
   }
 }
 
@@ -849,15 +886,31 @@ void launch_lift(gdsw_ctx* c, double* b, cudaStream_t s) {
   check_launch("k_lift_gather");
 }
 
-void launch_spmv(gdsw_ctx* c, const double* x, double* y, const double* rhs, cudaStream_t s) {
-  const int64_t nv = c->mesh.nv, np = c->mesh.np;
-  const double* bval = c->d_val + 9 * c->nnzb + 3 * c->nbt;
-  const int64_t ns = c->n_sell_slices;
-  const int64_t blocks = (ns + 1) / 2 + (np + 7) / 8;
-  k_spmv<<<int(blocks), 256, 0, s>>>(c->d_sell_row, c->d_sell_aoff, c->d_sell_acol, c->d_sell_aval,
-                                     c->d_sell_boff, c->d_sell_bcol, c->d_sell_btval, ns, c->d_b_ptr, c->d_b_col,
-                                     bval, nv, np, x, y, rhs);
+template <int C, int W, int NWARP, int LPR>
+static void spmv_as(const SpmvArgs& a, cudaStream_t s) {
+  constexpr int SPC = NWARP / W, RPC = NWARP * (32 / LPR);
+  const unsigned grid = unsigned((a.nslices + SPC - 1) / SPC + (a.np + RPC - 1) / RPC);
+  k_spmv<C, W, NWARP, LPR><<<grid, 32 * NWARP, 0, s>>>(a);
   check_launch("k_spmv");
+}
+
+// The form of k_spmv by the operator's size; each line between two sizes is where the two forms
+// beside it were equally fast (us per product, unit cubes of m^3 elements, m = 8 / 12 / 16 / 20 /
+// 32): 8 rows 4 warps 12 / 23 / 49, 8 rows 2 warps 14 / 24 / 45, 32 rows 4 warps - / 46 / 43 / 72 /
+// 286; before 25 / 50 / 62 / 102 / 306.  (32 rows with 2 warps: 283 at m = 32, but longer sums.)
+void launch_spmv(gdsw_ctx* c, const double* x, double* y, const double* rhs, cudaStream_t s) {
+  const int64_t nv = c->mesh.nv, np = c->mesh.np, ns = c->n_sell_slices;
+  const double* bval = c->d_val + 9 * c->nnzb + 3 * c->nbt;
+  const SpmvArgs a{c->d_sell_row, c->d_sell_aoff, c->d_sell_acol, c->d_sell_aval, c->d_sell_boff, c->d_sell_bcol,
+                   c->d_sell_btval, ns, c->d_b_ptr, c->d_b_col, bval, nv, np, x, y, rhs};
+  if (c->mesh.sell_c == 8) {
+    if (nv <= 14000)
+      spmv_as<8, 4, 4, 32>(a, s);
+    else
+      spmv_as<8, 2, 4, 16>(a, s);
+  } else {
+    spmv_as<32, 4, 4, 8>(a, s);
+  }
 }
 
 // refresh the sliced copy of A (after every assembly) and of B^T (once B is assembled)

@@ -72,3 +72,26 @@ def test_viscosity_and_lifting(lib, m, pressure, form):
     torch.cuda.synchronize()
     assert np.linalg.norm(b.cpu().numpy() - bo) <= TOL * max(np.linalg.norm(bo), 1e-300)
     ctx.close()
+
+
+@pytest.mark.parametrize("m,pressure", [((1, 1, 1), "q1"), ((1, 2, 1), "p1disc"), ((8, 8, 8), "q1"), ((13, 12, 11), "q1"),
+                                        ((13, 12, 13), "p1disc"), ((18, 19, 17), "q1")])
+def test_products(lib, m, pressure):
+    """y = A x and b - A x in every form of the product: slices of 8 rows with four and two warps,
+    slices of 32 rows, and a partly filled last slice, against the assembled matrix.  A row has up
+    to 375 + 27 terms: 402 x 1.1e-16, on the norms of |A| |x|."""
+    p = _problem(m, "symmetric", pressure)
+    ctx = lib.Context(p, levels=1)
+    A = ctx.gdsw_matrix_csr()
+    rng = np.random.default_rng(7)
+    x, b = rng.standard_normal(ctx.n), rng.standard_normal(ctx.n)
+    xd, bd = torch.from_numpy(x).cuda(), torch.from_numpy(b).cuda()
+    y = torch.full_like(xd, float("nan"))
+    r = torch.full_like(xd, float("nan"))
+    ctx.gdsw_spmv(xd, y)
+    ctx.gdsw_residual(bd, xd, r)
+    torch.cuda.synchronize()
+    bound = 402 * 1.1e-16 * (abs(A) @ abs(x) + abs(b))
+    assert np.all(abs(y.cpu().numpy() - A @ x) <= bound)
+    assert np.all(abs(r.cpu().numpy() - (b - A @ x)) <= bound)
+    ctx.close()
