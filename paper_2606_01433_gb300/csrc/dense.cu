@@ -3,6 +3,8 @@
 // block-LDU sweeps with explicit inverse diagonal blocks), and the set-up kernels that
 // build those factors: a batched GEMM and a batched blocked Gauss-Jordan inverse with
 // partial pivoting.
+#include <cooperative_groups.h>
+
 #include <cfloat>
 
 #include "common.h"
@@ -572,10 +574,13 @@ void set_gemv_smem_limits() {
 }
 
 // ------------------------------------------------------------------ batched GEMM (set-up)
-// 64x64 output tile per CTA, 256 threads computing 4x4 each, K staged 16 at a time.
+// 64x64 output tile per CTA, 256 threads computing 4x4 each, K staged 16 at a time.  Few tiles with
+// a long K (the Galerkin products X^T Y: a hundred columns, ten thousand rows) would leave most SMs
+// idle -- 8 CTAs took 13.8 ms -- so run_gemm_engine cuts K into gridDim.y slices: raw products go to
+// `part` and k_gemm_slices adds them in slice order.
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemm(const GemmTaskP* __restrict__ tasks, const int32_t* __restrict__ tile_task,
-                                              const int32_t* __restrict__ tile_id) {
+                                              const int32_t* __restrict__ tile_id, T* __restrict__ part) {
   __shared__ T As[16][64 + 1];
   __shared__ T Bs[16][64 + 1];
   const GemmTaskP t = tasks[tile_task[blockIdx.x]];
@@ -585,8 +590,10 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmTaskP* __restrict__ task
   const T* B = static_cast<const T*>(t.b);
   T* C = static_cast<T*>(t.c);
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const int steps = (t.K + 15) / 16, S = gridDim.y;
+  const int kbeg = int(int64_t(steps) * blockIdx.y / S) * 16, kend = min(t.K, int(int64_t(steps) * (blockIdx.y + 1) / S) * 16);
   T acc[4][4] = {};
-  for (int k0 = 0; k0 < t.K; k0 += 16) {
+  for (int k0 = kbeg; k0 < kend; k0 += 16) {
     for (int e = threadIdx.x; e < 16 * 64; e += 256) {
       int kk = e / 64, mm = e % 64;
       int gm = tm * 64 + mm, gk = k0 + kk;
@@ -613,6 +620,14 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmTaskP* __restrict__ task
     }
     __syncthreads();
   }
+  if (S > 1) {
+    T* out = part + (int64_t(blockIdx.y) * gridDim.x + blockIdx.x) * 4096;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) out[(ty * 4 + i) * 64 + tx * 4 + j] = acc[i][j];
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     int gm = tm * 64 + ty * 4 + i;
@@ -627,6 +642,25 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmTaskP* __restrict__ task
       *cp = v;
     }
   }
+}
+
+// C = alpha (sum of the slices' products) + beta C for the tiles of a sliced k_gemm
+template <typename T>
+__global__ void __launch_bounds__(256) k_gemm_slices(const GemmTaskP* __restrict__ tasks,
+                                                     const int32_t* __restrict__ tile_task,
+                                                     const int32_t* __restrict__ tile_id, int S,
+                                                     const T* __restrict__ part) {
+  const GemmTaskP t = tasks[tile_task[blockIdx.x]];
+  const int tiles_n = (t.N + 63) / 64;
+  const int tm = tile_id[blockIdx.x] / tiles_n, tn = tile_id[blockIdx.x] % tiles_n;
+  const int e = blockIdx.y * 256 + threadIdx.x, gm = tm * 64 + e / 64, gn = tn * 64 + e % 64;
+  if (gm >= t.M || gn >= t.N) return;
+  T s = T(0);
+  for (int k = 0; k < S; ++k) s += part[(int64_t(k) * gridDim.x + blockIdx.x) * 4096 + e];
+  T* cp = static_cast<T*>(t.c) + int64_t(gm) * t.ldc + gn;
+  T v = T(t.alpha) * s;
+  if (t.beta != 0.0) v += T(t.beta) * *cp;
+  *cp = v;
 }
 
 // ------------------------------------------------------------------ FP32 GEMM tiles
@@ -777,8 +811,18 @@ void run_gemm_engine(DevArena& tmp, const std::vector<GemmTaskP>& tasks, cudaStr
   if (!tt.empty()) {
     int32_t* d_tt = tmp.upload(tt, s);
     int32_t* d_ti = tmp.upload(ti, s);
-    k_gemm<T><<<int(tt.size()), 256, 0, s>>>(d_t, d_tt, d_ti);
+    // slices of K: enough CTAs for two per SM, at least 256 products each
+    int kmax = 0;
+    for (const auto& t : tasks) kmax = std::max(kmax, t.K);
+    const int ntl = int(tt.size()), S = std::max(1, std::min(304 / ntl, kmax / 256));
+    T* part = S > 1 ? tmp.alloc<T>(size_t(S) * ntl * 4096) : nullptr;
+    k_gemm<T><<<dim3(ntl, S), 256, 0, s>>>(d_t, d_tt, d_ti, part);
     check_launch("k_gemm");
+    if (S > 1) {
+      k_gemm_slices<T><<<dim3(ntl, 16), 256, 0, s>>>(d_t, d_tt, d_ti, S, part);
+      check_launch("k_gemm_slices");
+      tmp.release(part);
+    }
   }
   if (!bt.empty()) {
     int32_t* d_bt = tmp.upload(bt, s);
@@ -794,79 +838,230 @@ template void run_gemm_engine<float>(DevArena&, const std::vector<GemmTaskP>&, c
 // ------------------------------------------------------------------ batched Gauss-Jordan inverse
 // In-place inversion of square blocks with partial pivoting, blocked by panels of NB
 // columns: (1) LU with partial pivoting of the remaining rows of the panel chooses the
-// pivot rows, (2) those rows are swapped into place, (3) the NB x NB pivot block D is
-// inverted, (4) the block sweep A_PP <- D^-1, A_Pj <- D^-1 A_Pj, A_iP <- -A_iP D^-1,
-// A_ij <- A_ij - A_iP D^-1 A_Pj is applied as a rank-NB update, and (5) at the end the
-// columns are permuted back in reverse pivot order.
+// pivot rows, (2) the NB x NB block D of their entries is inverted, (3) the rows are swapped into
+// place and the block sweep A_PP <- D^-1, A_Pj <- D^-1 A_Pj, A_iP <- -A_iP D^-1,
+// A_ij <- A_ij - A_iP D^-1 A_Pj is applied as a rank-NB update, and (4) at the end the
+// columns are permuted back.
 constexpr int GJ_NB = 32;
+constexpr int kGjClusterRows = 8 * 512;  // rows of a panel that a cluster of 8 CTAs holds in registers
 
+// What a panel leaves for the sweep, per task: the rows chosen (their position before the panel's
+// swaps) and, per row at the panel's own positions, where it went if it was not chosen (else -1).
+struct GjSwaps {
+  int32_t from[GJ_NB], to[GJ_NB];
+};
+
+// A pivot candidate: larger magnitude first, then the smaller position.  The magnitude's bits + 1
+// (0: no candidate; a NaN counts as zero), split in two words for 64-bit types.
+struct GjBest {
+  unsigned hi, lo, npos;  // npos = ~position
+};
+__device__ __forceinline__ GjBest gj_key(float v, int pos) {
+  const float a = fabsf(v);
+  return {(a >= 0.f ? __float_as_uint(a) : 0u) + 1u, 0u, ~unsigned(pos)};
+}
+__device__ __forceinline__ GjBest gj_key(double v, int pos) {
+  const double a = fabs(v);
+  const unsigned long long b = (a >= 0.0 ? (unsigned long long)__double_as_longlong(a) : 0ull) + 1ull;
+  return {unsigned(b >> 32), unsigned(b), ~unsigned(pos)};
+}
+__device__ __forceinline__ double gj_magnitude(const GjBest& k, float) { return double(__uint_as_float(k.hi - 1u)); }
+__device__ __forceinline__ double gj_magnitude(const GjBest& k, double) {
+  return __longlong_as_double((long long)(((unsigned long long)k.hi << 32 | k.lo) - 1ull));
+}
 template <typename T>
-__global__ void __launch_bounds__(256) k_gj_panel(const InvTaskP* tasks, int kb, T* scratch, int64_t scr_stride,
-                                                  int32_t* piv, int64_t piv_stride, double* minpiv) {
-  const InvTaskP t = tasks[blockIdx.x];
-  if (kb >= t.n) return;
-  T* A = static_cast<T*>(t.a);
-  const int w = min(GJ_NB, t.n - kb), rows = t.n - kb;
-  T* P = scratch + int64_t(t.id) * scr_stride;  // rows x GJ_NB
-  int32_t* pv = piv + int64_t(t.id) * piv_stride;
-  for (int e = threadIdx.x; e < rows * w; e += blockDim.x) {
-    int r = e / w, c = e % w;
-    P[int64_t(r) * GJ_NB + c] = A[int64_t(kb + r) * t.ld + kb + c];
+__device__ __forceinline__ GjBest gj_warp_best(GjBest k) {
+  GjBest b;
+  b.hi = __reduce_max_sync(0xffffffffu, k.hi);
+  bool in = k.hi == b.hi;
+  if (sizeof(T) == 8) {
+    b.lo = __reduce_max_sync(0xffffffffu, in ? k.lo : 0u);
+    in = in && k.lo == b.lo;
+  } else {
+    b.lo = 0u;
   }
-  __syncthreads();
-  __shared__ double bv[256];
-  __shared__ int bi[256];
-  __shared__ T prow[GJ_NB];
-  for (int j = 0; j < w; ++j) {
-    double best = -1.0;
-    int besti = rows;
-    for (int r = j + threadIdx.x; r < rows; r += blockDim.x) {
-      double a = fabs(double(P[int64_t(r) * GJ_NB + j]));
-      if (a > best) { best = a; besti = r; }
+  b.npos = __reduce_max_sync(0xffffffffu, in ? k.npos : 0u);
+  return b;
+}
+
+// D^-1 by Gauss-Jordan in one warp (pivot order fixed by the panel LU, so no further pivoting); lane =
+// column, its entries in registers.  The rows rotate by one per step, so that the pivot row is always
+// the first register and the loop stays rolled (32 steps bring them back; steps beyond the block's
+// size meet the unit rows that pad it).
+template <typename T>
+__device__ __forceinline__ void gj_dinv_warp(T (&D)[GJ_NB], T* out) {
+  const int c = threadIdx.x & 31;
+#pragma unroll 1
+  for (int k = 0; k < GJ_NB; ++k) {
+    T p = __shfl_sync(0xffffffffu, D[0], k);
+    if (p == T(0)) p = T(1);
+    const T inv = T(1) / p;
+    const T rk = D[0];
+#pragma unroll
+    for (int r = 1; r < GJ_NB; ++r) {
+      const T ck = __shfl_sync(0xffffffffu, D[r], k);
+      D[r - 1] = c == k ? -ck * inv : D[r] - ck * rk * inv;
     }
-    bv[threadIdx.x] = best;
-    bi[threadIdx.x] = besti;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if (threadIdx.x < o) {
-        double a = bv[threadIdx.x + o];
-        int ia = bi[threadIdx.x + o];
-        if (a > bv[threadIdx.x] || (a == bv[threadIdx.x] && ia < bi[threadIdx.x])) {
-          bv[threadIdx.x] = a;
-          bi[threadIdx.x] = ia;
-        }
+    D[GJ_NB - 1] = c == k ? inv : rk * inv;
+  }
+#pragma unroll
+  for (int r = 0; r < GJ_NB; ++r) out[r * GJ_NB + c] = D[r];
+}
+
+// Pivot choice and D^-1 of one panel, R rows of the panel per thread in registers, a cluster of CTAs
+// per matrix.  Per column: every warp finds its best row (two or three integer warp reductions),
+// the CTA its best warp; that warp copies the row to every CTA of the cluster (distributed shared
+// memory), and after one cluster barrier all threads know the pivot row and eliminate theirs.  Rows
+// are not moved: a thread keeps the position its row has after the swaps so far.  The chain of a
+// column is latency only -- one block and one cluster barrier, 1.3 us -- so the panel's time hardly
+// depends on the matrix size; with the panel in one CTA's shared memory a column took 13 us at 2000
+// rows (eight matrices: eight CTAs at work).  The loop over the columns stays rolled (a row shifts by
+// one register per column): unrolled 32 times it was bound by instruction fetches, 3 us per column.
+// Panel, pivot block, swaps and E, F of eight 2000-row matrices: 489 -> 57 us (five launches -> two).
+template <typename T, int NT, int R>
+__global__ void __launch_bounds__(NT) k_gj_panel_rows(const InvTaskP* __restrict__ tasks, int kb, int CL,
+                                                      int32_t* __restrict__ rowid, int64_t rowid_stride,
+                                                      GjSwaps* __restrict__ swaps, T* __restrict__ dinv,
+                                                      double* __restrict__ minpiv) {
+  constexpr int NW = NT / 32, V = 16 / sizeof(T), NCH = GJ_NB / V, CMAX = 8;
+  __shared__ GjBest wbest[2][NW];
+  __shared__ GjBest cbest[2][CMAX];
+  __shared__ __align__(16) T stage[2][GJ_NB];
+  __shared__ __align__(16) T prow[2][CMAX][GJ_NB];
+  __shared__ int32_t s_from[GJ_NB];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const InvTaskP t = tasks[blockIdx.x / CL];
+  if (kb >= t.n) return;  // the whole cluster
+  const int rank = int(blockIdx.x) % CL;
+  const int w = min(GJ_NB, t.n - kb), rows = t.n - kb;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const T* A = static_cast<const T*>(t.a);
+  int32_t* id = rowid + int64_t(t.id) * rowid_stride + kb;
+  T v[R][GJ_NB];
+  int pos[R], myid[R];
+  bool live[R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int r = (rank * R + q) * NT + int(threadIdx.x);
+    live[q] = r < rows;
+    pos[q] = r;
+    myid[q] = live[q] ? id[r] : 0;
+    const T* p = A + int64_t(kb + r) * t.ld + kb;
+#pragma unroll
+    for (int c = 0; c < GJ_NB; c += V) {
+      if (live[q] && c < w) {  // the padded row holds the whole vector
+        const uint4 raw = *reinterpret_cast<const uint4*>(p + c);
+        const T* e = reinterpret_cast<const T*>(&raw);
+#pragma unroll
+        for (int u = 0; u < V; ++u) v[q][c + u] = e[u];
+      } else {
+#pragma unroll
+        for (int u = 0; u < V; ++u) v[q][c + u] = T(0);
       }
+    }
+  }
+  double least = DBL_MAX;
+  if (CL > 1) cl.sync();  // every CTA of the cluster runs before its shared memory is written
+#pragma unroll 1
+  for (int j = 0; j < w; ++j) {  // v[q][0] is column j: eliminating a row shifts it by one column
+    constexpr GjBest none = {0u, 0u, 0u};
+    const int buf = j & 1;
+    GjBest k = live[0] ? gj_key(v[0][0], pos[0]) : none;
+#pragma unroll
+    for (int q = 1; q < R; ++q)
+      if (live[q]) {
+        const GjBest o = gj_key(v[q][0], pos[q]);
+        if (o.hi > k.hi || (o.hi == k.hi && (o.lo > k.lo || (o.lo == k.lo && o.npos > k.npos)))) k = o;
+      }
+    GjBest b = gj_warp_best<T>(k);
+    if (lane == 0) wbest[buf][warp] = b;
+    __syncthreads();
+    b = gj_warp_best<T>(lane < NW ? wbest[buf][lane] : none);  // the CTA's
+    // the owner's warp passes the row on (warp 0 if the CTA has no row left)
+    const bool some = (b.hi | b.lo) != 0u;
+    bool own = false;
+#pragma unroll
+    for (int q = 0; q < R; ++q) own = own || (some && live[q] && ~unsigned(pos[q]) == b.npos);
+    const bool push = some ? __any_sync(0xffffffffu, own) : warp == 0;
+    if (push) {
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+        if (some && live[q] && ~unsigned(pos[q]) == b.npos)
+#pragma unroll
+          for (int c = 0; c < GJ_NB; c += V) {
+            uint4 raw;
+            T* e = reinterpret_cast<T*>(&raw);
+#pragma unroll
+            for (int u = 0; u < V; ++u) e[u] = v[q][c + u];
+            *reinterpret_cast<uint4*>(&stage[buf][c]) = raw;
+          }
+      __syncwarp();
+      for (int i = lane; i < CL * NCH; i += 32) {
+        const uint4 raw = *reinterpret_cast<const uint4*>(&stage[buf][(i % NCH) * V]);
+        *reinterpret_cast<uint4*>(cl.map_shared_rank(&prow[buf][rank][(i % NCH) * V], i / NCH)) = raw;
+      }
+      if (lane < CL) *cl.map_shared_rank(&cbest[buf][rank], lane) = b;
+    }
+    if (CL > 1)
+      cl.sync();
+    else
       __syncthreads();
+    const GjBest mine = lane < CL ? cbest[buf][lane] : none;
+    b = gj_warp_best<T>(mine);
+    const int src = __ffs(__ballot_sync(0xffffffffu, mine.hi == b.hi && mine.lo == b.lo && mine.npos == b.npos)) - 1;
+    const int p = int(~b.npos);
+    least = fmin(least, gj_magnitude(b, T(0)));
+    T pr[GJ_NB];
+#pragma unroll
+    for (int c = 0; c < GJ_NB; c += V) {
+      const uint4 raw = *reinterpret_cast<const uint4*>(&prow[buf][src][c]);
+      const T* e = reinterpret_cast<const T*>(&raw);
+#pragma unroll
+      for (int u = 0; u < V; ++u) pr[c + u] = e[u];
     }
-    const int p = bi[0];
-    const double pmag = bv[0];
-    if (threadIdx.x == 0) {
-      pv[kb + j] = kb + p;
-      if (pmag < minpiv[t.id]) minpiv[t.id] = pmag;
-    }
-    // swap rows j and p of the panel copy
-    if (p != j)
-      for (int c = threadIdx.x; c < w; c += blockDim.x) {
-        T a = P[int64_t(j) * GJ_NB + c];
-        P[int64_t(j) * GJ_NB + c] = P[int64_t(p) * GJ_NB + c];
-        P[int64_t(p) * GJ_NB + c] = a;
-      }
-    __syncthreads();
-    for (int c = threadIdx.x; c < w; c += blockDim.x) prow[c] = P[int64_t(j) * GJ_NB + c];
-    __syncthreads();
-    T d = prow[j];
+    T d = pr[0];
     if (d == T(0)) d = T(1);  // singular: recorded through minpiv, keep the numbers finite
-    for (int r = j + 1 + threadIdx.x; r < rows; r += blockDim.x) {
-      T* pr = P + int64_t(r) * GJ_NB;
-      T l = pr[j] / d;
-      pr[j] = l;
-      for (int c = j + 1; c < w; ++c) pr[c] -= l * prow[c];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      if (!live[q]) continue;
+      if (pos[q] == p) {  // chosen: its position before the swaps goes to the first CTA
+        pos[q] = j;
+        live[q] = false;
+        *cl.map_shared_rank(&s_from[j], 0) = (rank * R + q) * NT + int(threadIdx.x);
+        continue;
+      }
+      if (pos[q] == j) pos[q] = p;
+      const T l = v[q][0] / d;
+#pragma unroll
+      for (int c = 1; c < GJ_NB; ++c) v[q][c - 1] = v[q][c] - l * pr[c];
     }
+  }
+  if (CL > 1)
+    cl.sync();
+  else
     __syncthreads();
+  GjSwaps* S = swaps + t.id;
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int r = (rank * R + q) * NT + int(threadIdx.x);
+    if (r >= rows) continue;
+    if (pos[q] != r) id[pos[q]] = myid[q];
+    if (r < w) S->to[r] = pos[q] >= w ? kb + pos[q] : -1;
+  }
+  if (rank != 0) return;
+  if (int(threadIdx.x) < w) S->from[threadIdx.x] = kb + s_from[threadIdx.x];
+  if (threadIdx.x == 0 && least < minpiv[t.id]) minpiv[t.id] = least;
+  if (warp == 0) {
+    T D[GJ_NB];
+#pragma unroll
+    for (int r = 0; r < GJ_NB; ++r)
+      D[r] = (r < w && lane < w) ? A[int64_t(kb + s_from[r]) * t.ld + kb + lane] : T(r == lane ? 1 : 0);
+    gj_dinv_warp<T>(D, dinv + int64_t(t.id) * GJ_NB * GJ_NB);
   }
 }
 
-// Pivot choice for one panel, faster form: 1024 threads; the first RS rows of the panel copy
+// Pivot choice for a panel of more rows than a cluster's registers hold: one CTA of 1024 threads; the first RS rows of the panel copy
 // live in shared memory (row stride NB + 1), the rest in the global scratch; the column
 // maximum is found with warp shuffles (largest magnitude, smallest row on ties -- the same
 // pivots as the tree reduction above), and the rank-1 elimination runs one warp per row,
@@ -974,87 +1169,113 @@ __global__ void __launch_bounds__(1024) k_gj_panel_fast(const InvTaskP* tasks, i
   }
 }
 
-// swap the chosen pivot rows into place across the full width of the matrix
+// The swaps of a panel that k_gj_panel_fast chose (more rows than a cluster's registers hold): the same
+// GjSwaps and row numbers from its sequence of transpositions, and D^-1.
 template <typename T>
-__global__ void k_gj_swap(const InvTaskP* tasks, int kb, const int32_t* piv, int64_t piv_stride) {
-  const InvTaskP t = tasks[blockIdx.y];
-  if (kb >= t.n) return;
-  int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= t.n) return;
-  T* A = static_cast<T*>(t.a);
-  const int32_t* pv = piv + int64_t(t.id) * piv_stride;
-  const int w = min(GJ_NB, t.n - kb);
-  for (int j = 0; j < w; ++j) {
-    int p = pv[kb + j];
-    if (p != kb + j) {
-      T a = A[int64_t(kb + j) * t.ld + c];
-      A[int64_t(kb + j) * t.ld + c] = A[int64_t(p) * t.ld + c];
-      A[int64_t(p) * t.ld + c] = a;
-    }
-  }
-}
-
-// invert the w x w pivot block (pivot order fixed by the panel LU, so no further pivoting)
-template <typename T>
-__global__ void __launch_bounds__(256) k_gj_dinv(const InvTaskP* tasks, int kb, T* dinv) {
+__global__ void __launch_bounds__(32) k_gj_maps(const InvTaskP* __restrict__ tasks, int kb,
+                                                const int32_t* __restrict__ piv, int64_t piv_stride,
+                                                int32_t* __restrict__ rowid, int64_t rowid_stride,
+                                                GjSwaps* __restrict__ swaps, T* __restrict__ dinv) {
   const InvTaskP t = tasks[blockIdx.x];
   if (kb >= t.n) return;
+  const int w = min(GJ_NB, t.n - kb), lane = threadIdx.x;
+  const int32_t* pv = piv + int64_t(t.id) * piv_stride + kb;
+  int32_t* id = rowid + int64_t(t.id) * rowid_stride;
+  // positions touched: the panel's own and the pivots'; at[] = the row (by position before) now there
+  __shared__ int32_t where[2 * GJ_NB], at[2 * GJ_NB], ids[2 * GJ_NB], n;
+  if (lane == 0) {
+    n = w;
+    for (int j = 0; j < w; ++j) where[j] = at[j] = kb + j;
+    for (int j = 0; j < w; ++j) {
+      int e = 0;
+      while (e < n && where[e] != pv[j]) ++e;
+      if (e == n) {
+        where[n] = at[n] = pv[j];
+        ++n;
+      }
+      const int32_t a = at[j];
+      at[j] = at[e];
+      at[e] = a;
+    }
+  }
+  __syncwarp();
+  for (int e = lane; e < n; e += 32) ids[e] = id[at[e]];
+  __syncwarp();
+  for (int e = lane; e < n; e += 32) id[where[e]] = ids[e];
+  GjSwaps* S = swaps + t.id;
+  if (lane < w) {
+    S->from[lane] = at[lane];
+    int32_t to = -1;
+    for (int e = w; e < n; ++e)
+      if (at[e] == kb + lane) to = where[e];
+    S->to[lane] = to;
+  }
+  T D[GJ_NB];
   const T* A = static_cast<const T*>(t.a);
-  const int w = min(GJ_NB, t.n - kb);
-  __shared__ T D[GJ_NB][GJ_NB + 1];
-  __shared__ T colk[GJ_NB], rk[GJ_NB];
-  for (int e = threadIdx.x; e < GJ_NB * GJ_NB; e += blockDim.x) {
-    int r = e / GJ_NB, c = e % GJ_NB;
-    D[r][c] = (r < w && c < w) ? A[int64_t(kb + r) * t.ld + kb + c] : T(r == c ? 1 : 0);
-  }
-  __syncthreads();
-  const int r0 = threadIdx.x / GJ_NB, c = threadIdx.x % GJ_NB;  // 8 rows x 32 cols per pass
-  for (int k = 0; k < w; ++k) {
-    if (threadIdx.x < GJ_NB) {
-      colk[threadIdx.x] = D[threadIdx.x][k];
-      rk[threadIdx.x] = D[k][threadIdx.x];
-    }
-    __syncthreads();
-    T p = rk[k];
-    if (p == T(0)) p = T(1);
-    const T inv = T(1) / p;
-    for (int rr = r0; rr < GJ_NB; rr += 8) {
-      T v;
-      if (rr == k) v = (c == k) ? inv : rk[c] * inv;
-      else v = (c == k) ? -colk[rr] * inv : D[rr][c] - colk[rr] * rk[c] * inv;
-      D[rr][c] = v;
-    }
-    __syncthreads();
-  }
-  T* out = dinv + int64_t(t.id) * GJ_NB * GJ_NB;
-  for (int e = threadIdx.x; e < GJ_NB * GJ_NB; e += blockDim.x) out[e] = D[e / GJ_NB][e % GJ_NB];
+#pragma unroll
+  for (int r = 0; r < GJ_NB; ++r) D[r] = (r < w && lane < w) ? A[int64_t(at[r]) * t.ld + kb + lane] : T(r == lane ? 1 : 0);
+  gj_dinv_warp<T>(D, dinv + int64_t(t.id) * GJ_NB * GJ_NB);
 }
 
-// Fp = D^-1 A[P, :] (w x n) and E = A[:, P] (n x w) saved before the update
+// F = D^-1 A[P, :] (w x n) from the chosen rows where they are, E = A[:, P] (n x w) of the swapped
+// matrix, and the displaced rows moved to their new positions.  One thread per column for the first
+// and the last (it has read its column of the chosen rows before it overwrites them), one per row for
+// E; a displaced row is read at its old position, which nothing writes here.
 template <typename T>
-__global__ void k_gj_fe(const InvTaskP* tasks, int kb, const T* dinv, T* Fp, T* E, int64_t stride) {
+__global__ void __launch_bounds__(128) k_gj_fe(const InvTaskP* __restrict__ tasks, int kb,
+                                               const GjSwaps* __restrict__ swaps, const T* __restrict__ dinv,
+                                               T* __restrict__ Fp, T* __restrict__ E, int64_t stride) {
+  constexpr int V = 16 / sizeof(T);
   const InvTaskP t = tasks[blockIdx.y];
-  if (kb >= t.n) return;
-  const T* A = static_cast<const T*>(t.a);
+  if (kb >= t.n || int(blockIdx.x) * 128 >= t.n) return;
+  __shared__ __align__(16) T Ds[GJ_NB * GJ_NB];
+  __shared__ GjSwaps S;
+  T* A = static_cast<T*>(t.a);
   const int w = min(GJ_NB, t.n - kb);
   const T* Di = dinv + int64_t(t.id) * GJ_NB * GJ_NB;
+  for (int e = threadIdx.x; e < GJ_NB * GJ_NB; e += 128) Ds[e] = Di[e];
+  if (threadIdx.x < GJ_NB) {
+    S.from[threadIdx.x] = int(threadIdx.x) < w ? swaps[t.id].from[threadIdx.x] : 0;
+    S.to[threadIdx.x] = int(threadIdx.x) < w ? swaps[t.id].to[threadIdx.x] : -1;
+  }
+  __syncthreads();
   T* F = Fp + int64_t(t.id) * stride;
   T* Ee = E + int64_t(t.id) * stride;
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const int idx = blockIdx.x * 128 + threadIdx.x;
   if (idx >= t.n) return;
-  // column idx of Fp
-  T col[GJ_NB];
+  {
+    T col[GJ_NB];
 #pragma unroll
-  for (int q = 0; q < GJ_NB; ++q) col[q] = q < w ? A[int64_t(kb + q) * t.ld + idx] : T(0);
-  for (int r = 0; r < w; ++r) {
-    T s = T(0);
+    for (int q = 0; q < GJ_NB; ++q) col[q] = q < w ? A[int64_t(S.from[q]) * t.ld + idx] : T(0);
+    for (int r = 0; r < w; ++r) {
+      T s = T(0);
 #pragma unroll
-    for (int q = 0; q < GJ_NB; ++q) s = fma(Di[r * GJ_NB + q], col[q], s);
-    F[int64_t(r) * t.ld + idx] = s;
+      for (int q = 0; q < GJ_NB; q += V) {
+        T dv[V];
+        *reinterpret_cast<uint4*>(dv) = *reinterpret_cast<const uint4*>(&Ds[r * GJ_NB + q]);
+#pragma unroll
+        for (int u = 0; u < V; ++u) s = fma(dv[u], col[q + u], s);
+      }
+      F[int64_t(r) * t.ld + idx] = s;
+    }
+#pragma unroll
+    for (int r = 0; r < GJ_NB; ++r) col[r] = S.to[r] >= 0 ? A[int64_t(kb + r) * t.ld + idx] : T(0);
+#pragma unroll
+    for (int r = 0; r < GJ_NB; ++r)
+      if (S.to[r] >= 0) A[int64_t(S.to[r]) * t.ld + idx] = col[r];
   }
-  // row idx of E
+  if (idx >= kb && idx < kb + w) return;  // pivot rows: not used by the sweep
+  int src = idx;
 #pragma unroll
-  for (int q = 0; q < GJ_NB; ++q) Ee[int64_t(idx) * GJ_NB + q] = q < w ? A[int64_t(idx) * t.ld + kb + q] : T(0);
+  for (int r = 0; r < GJ_NB; ++r)
+    if (S.to[r] == idx) src = kb + r;
+  const T* p = A + int64_t(src) * t.ld + kb;
+  // a row that is displaced by another thread's columns is not read here; the others do not change
+  for (int q = 0; q < GJ_NB; q += V) {
+    uint4 raw = make_uint4(0, 0, 0, 0);
+    if (q < w) raw = *reinterpret_cast<const uint4*>(p + q);
+    *reinterpret_cast<uint4*>(Ee + int64_t(idx) * GJ_NB + q) = raw;
+  }
 }
 
 template <typename T>
@@ -1185,6 +1406,22 @@ __global__ void __launch_bounds__(256, 2) k_gj_update_f32(const InvTaskP* __rest
 #pragma unroll
       for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
   }
+  if (m0 + 128 <= t.n && n0 + 128 <= t.n && (m0 >= kb + w || m0 + 128 <= kb) && (n0 >= kb + w || n0 + 128 <= kb)) {
+    // a whole tile off the pivot rows and columns (most): 16-byte stores
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int li = gemm_row(i);
+      float* row = Am + int64_t(m0 + li) * t.ld + n0;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int lj = gemm_col(4 * h);
+        const float4 c = *reinterpret_cast<const float4*>(Cs + li * GJU_LD + lj);
+        *reinterpret_cast<float4*>(row + lj) = make_float4(c.x - acc[i][4 * h], c.y - acc[i][4 * h + 1],
+                                                           c.z - acc[i][4 * h + 2], c.w - acc[i][4 * h + 3]);
+      }
+    }
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int li = gemm_row(i), gi = m0 + li;
@@ -1212,21 +1449,61 @@ __global__ void __launch_bounds__(256, 2) k_gj_update_f32(const InvTaskP* __rest
   }
 }
 
+// A^-1 = X P for the inverse X of the row-permuted matrix: column i of X belongs to the row that
+// ended at position i.  A CTA permutes whole rows through shared memory.
 template <typename T>
-__global__ void k_gj_colperm(const InvTaskP* tasks, const int32_t* piv, int64_t piv_stride) {
+__global__ void __launch_bounds__(256) k_gj_colperm(const InvTaskP* __restrict__ tasks,
+                                                    const int32_t* __restrict__ rowid, int64_t rowid_stride, int rows) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* buf = reinterpret_cast<T*>(smem_raw);
   const InvTaskP t = tasks[blockIdx.y];
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= t.n) return;
-  T* A = static_cast<T*>(t.a) + int64_t(r) * t.ld;
-  const int32_t* pv = piv + int64_t(t.id) * piv_stride;
-  for (int j = t.n - 1; j >= 0; --j) {
-    int p = pv[j];
-    if (p != j) {
-      T a = A[j];
-      A[j] = A[p];
-      A[p] = a;
-    }
+  const int32_t* id = rowid + int64_t(t.id) * rowid_stride;
+  const int r1 = min(t.n, (int(blockIdx.x) + 1) * rows);
+  for (int r = blockIdx.x * rows; r < r1; ++r) {
+    T* A = static_cast<T*>(t.a) + int64_t(r) * t.ld;
+    for (int c = threadIdx.x; c < t.n; c += 256) buf[id[c]] = A[c];
+    __syncthreads();
+    for (int c = threadIdx.x; c < t.n; c += 256) A[c] = buf[c];
+    __syncthreads();
   }
+}
+
+// The same for rows that do not fit in shared memory: GJ_NB rows at a time to the scratch and back
+template <typename T>
+__global__ void __launch_bounds__(256) k_gj_colperm_wide(const InvTaskP* __restrict__ tasks,
+                                                         const int32_t* __restrict__ rowid, int64_t rowid_stride, int r0,
+                                                         T* __restrict__ scratch, int64_t stride, int back) {
+  const InvTaskP t = tasks[blockIdx.z];
+  const int r = r0 + int(blockIdx.y), c = blockIdx.x * 256 + int(threadIdx.x);
+  if (r >= t.n || c >= t.n) return;
+  T* A = static_cast<T*>(t.a) + int64_t(r) * t.ld;
+  T* S = scratch + int64_t(t.id) * stride + int64_t(blockIdx.y) * t.ld;
+  if (back)
+    A[c] = S[c];
+  else
+    S[rowid[int64_t(t.id) * rowid_stride + c]] = A[c];
+}
+
+__global__ void k_iota_rows(int32_t* p, int64_t stride, int64_t n) {
+  const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (i < n) p[i] = int32_t(i % stride);
+}
+
+template <typename T, int NT, int R>
+static void gj_panel_rows(const InvTaskP* tasks, int nt, int kb, int CL, int32_t* rowid, int64_t rowid_stride,
+                          GjSwaps* swaps, T* dinv, double* minpiv, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(nt) * CL);
+  cfg.blockDim = dim3(NT);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = unsigned(CL);
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  GDSW_CUDA(cudaLaunchKernelEx(&cfg, k_gj_panel_rows<T, NT, R>, tasks, kb, CL, rowid, rowid_stride, swaps, dinv, minpiv));
 }
 
 __global__ void k_fill_d(double* p, double v, int64_t n) {
@@ -1256,11 +1533,16 @@ void run_inverse(DevArena& tmp, const std::vector<InvTaskP>& tasks_in, std::vect
   for (const InvTaskP& t : tasks) ldmax = std::max(ldmax, t.ld);
   // F rows have the matrices' leading dimension
   const int64_t stride = std::max<int64_t>(pad8(nmax), ldmax) * GJ_NB;
-  T* scratch = tmp.alloc<T>(size_t(nq) * stride);
   T* Fp = tmp.alloc<T>(size_t(nq) * stride);
   T* E = tmp.alloc<T>(size_t(nq) * stride);
   T* dinv = tmp.alloc<T>(size_t(nq) * GJ_NB * GJ_NB);
-  int32_t* piv = tmp.alloc<int32_t>(size_t(nq) * nmax);
+  int32_t* rowid = tmp.alloc<int32_t>(size_t(nq) * nmax);
+  GjSwaps* swaps = tmp.alloc<GjSwaps>(size_t(nq));
+  k_iota_rows<<<unsigned((nq * nmax + 255) / 256), 256, 0, s>>>(rowid, nmax, nq * nmax);
+  // panels of more rows than a cluster's registers hold: one CTA per matrix, pivots in piv, scratch
+  const bool wide = nmax > kGjClusterRows;
+  T* scratch = wide ? tmp.alloc<T>(size_t(nq) * stride) : nullptr;
+  int32_t* piv = wide ? tmp.alloc<int32_t>(size_t(nq) * nmax) : nullptr;
   double* d_min = tmp.alloc<double>(nq);
   k_fill_d<<<int((nq + 255) / 256), 256, 0, s>>>(d_min, DBL_MAX, nq);
   InvTaskP* d_tasks = tmp.upload(tasks, s);
@@ -1275,16 +1557,33 @@ void run_inverse(DevArena& tmp, const std::vector<InvTaskP>& tasks_in, std::vect
   }
   int32_t* d_tt = tmp.upload(tt, s);
   int32_t* d_ti = tmp.upload(ti, s);
-  dim3 gcol((nmax + 255) / 256, nt);
+  const dim3 gcol((nmax + 127) / 128, nt);
   const size_t panel_smem = size_t(200) * 1024;
   const int panel_rs = int(panel_smem / ((GJ_NB + 1) * sizeof(T)));
-  GDSW_CUDA(cudaFuncSetAttribute(k_gj_panel_fast<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(panel_smem)));
+  if (wide)
+    GDSW_CUDA(cudaFuncSetAttribute(k_gj_panel_fast<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(panel_smem)));
   GDSW_CUDA(cudaFuncSetAttribute(k_gj_update_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GJU_SMEM)));
   for (int kb = 0; kb < nmax; kb += GJ_NB) {
-    k_gj_panel_fast<T><<<nt, 1024, panel_smem, s>>>(d_tasks, kb, scratch, stride, piv, nmax, d_min, panel_rs);
-    k_gj_swap<T><<<gcol, 256, 0, s>>>(d_tasks, kb, piv, nmax);
-    k_gj_dinv<T><<<nt, 256, 0, s>>>(d_tasks, kb, dinv);
-    k_gj_fe<T><<<gcol, 256, 0, s>>>(d_tasks, kb, dinv, Fp, E, stride);
+    // one thread per row of the panel; matrices of a few warps take smaller CTAs
+    const int rows = nmax - kb;
+    auto cluster = [&](int per_cta) {
+      int c = 1;
+      while (c * per_cta < rows) c *= 2;
+      return c;
+    };
+    if (rows <= 64)
+      gj_panel_rows<T, 64, 1>(d_tasks, nt, kb, 1, rowid, nmax, swaps, dinv, d_min, s);
+    else if (rows <= 128)
+      gj_panel_rows<T, 128, 1>(d_tasks, nt, kb, 1, rowid, nmax, swaps, dinv, d_min, s);
+    else if (rows <= 8 * 256)
+      gj_panel_rows<T, 256, 1>(d_tasks, nt, kb, cluster(256), rowid, nmax, swaps, dinv, d_min, s);
+    else if (rows <= kGjClusterRows)
+      gj_panel_rows<T, 256, 2>(d_tasks, nt, kb, cluster(512), rowid, nmax, swaps, dinv, d_min, s);
+    else {
+      k_gj_panel_fast<T><<<nt, 1024, panel_smem, s>>>(d_tasks, kb, scratch, stride, piv, nmax, d_min, panel_rs);
+      k_gj_maps<T><<<nt, 32, 0, s>>>(d_tasks, kb, piv, nmax, rowid, nmax, swaps, dinv);
+    }
+    k_gj_fe<T><<<gcol, 128, 0, s>>>(d_tasks, kb, swaps, dinv, Fp, E, stride);
     if (sizeof(T) == 4)
       k_gj_update_f32<<<int(tt.size()), 256, GJU_SMEM, s>>>(d_tasks, d_tt, d_ti, kb, reinterpret_cast<const float*>(dinv),
                                                      reinterpret_cast<const float*>(Fp),
@@ -1293,13 +1592,29 @@ void run_inverse(DevArena& tmp, const std::vector<InvTaskP>& tasks_in, std::vect
       k_gj_update<T><<<int(tt.size()), 256, 0, s>>>(d_tasks, d_tt, d_ti, kb, dinv, Fp, E, stride);
     check_launch("gauss-jordan panel");
   }
-  k_gj_colperm<T><<<gcol, 256, 0, s>>>(d_tasks, piv, nmax);
-  check_launch("k_gj_colperm");
+  const size_t row_bytes = size_t(nmax) * sizeof(T);
+  if (row_bytes <= size_t(200) * 1024) {
+    constexpr int kRows = 8;
+    GDSW_CUDA(cudaFuncSetAttribute(k_gj_colperm<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    k_gj_colperm<T><<<dim3((nmax + kRows - 1) / kRows, nt), 256, row_bytes, s>>>(d_tasks, rowid, nmax, kRows);
+    check_launch("k_gj_colperm");
+  } else {
+    for (int r0 = 0; r0 < nmax; r0 += GJ_NB)
+      for (int back = 0; back < 2; ++back) {
+        k_gj_colperm_wide<T><<<dim3((nmax + 255) / 256, GJ_NB, nt), 256, 0, s>>>(d_tasks, rowid, nmax, r0, Fp, stride,
+                                                                                 back);
+        check_launch("k_gj_colperm_wide");
+      }
+  }
   GDSW_CUDA(cudaMemcpyAsync(minpiv.data(), d_min, sizeof(double) * nq, cudaMemcpyDeviceToHost, s));
   GDSW_CUDA(cudaStreamSynchronize(s));
   for (size_t q = 0; q < tasks_in.size(); ++q)
     if (tasks_in[q].n == 0) minpiv[q] = 1.0;
-  tmp.release(scratch); tmp.release(Fp); tmp.release(E); tmp.release(dinv); tmp.release(piv);
+  if (wide) {
+    tmp.release(scratch);
+    tmp.release(piv);
+  }
+  tmp.release(Fp); tmp.release(E); tmp.release(dinv); tmp.release(rowid); tmp.release(swaps);
   tmp.release(d_min); tmp.release(d_tasks); tmp.release(d_tt); tmp.release(d_ti);
 }
 template void run_inverse<double>(DevArena&, const std::vector<InvTaskP>&, std::vector<double>&, cudaStream_t);
