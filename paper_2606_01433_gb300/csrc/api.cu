@@ -6,7 +6,6 @@
 #include <cmath>
 #include <cstring>
 #include <numeric>
-#include <tuple>
 
 #include "common.h"
 #include "kernels.h"
@@ -595,7 +594,6 @@ static std::vector<int64_t> phi_offsets(const CoarseSpace& C, std::vector<int32_
 // segment lists for A0 = sum of keyed contributions, built on the host
 struct SegList {
   std::vector<int64_t> key, ptr, pos;
-  std::vector<double> w;  // per entry weight (empty: all 1)
 };
 static SegList make_segments(std::vector<std::pair<int64_t, int64_t>>& kv) {
   std::stable_sort(kv.begin(), kv.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
@@ -612,31 +610,12 @@ static SegList make_segments(std::vector<std::pair<int64_t, int64_t>>& kv) {
   return L;
 }
 
-// the same with a weight per entry: kvw = (key, source position, weight)
-static SegList make_segments_w(std::vector<std::tuple<int64_t, int64_t, double>>& kvw) {
-  std::stable_sort(kvw.begin(), kvw.end(),
-                   [](const auto& a, const auto& b) { return std::get<0>(a) < std::get<0>(b); });
-  SegList L;
-  L.ptr.push_back(0);
-  for (size_t q = 0; q < kvw.size(); ++q) {
-    if (q == 0 || std::get<0>(kvw[q]) != std::get<0>(kvw[q - 1])) {
-      if (q > 0) L.ptr.push_back(int64_t(q));
-      L.key.push_back(std::get<0>(kvw[q]));
-    }
-    L.pos.push_back(std::get<1>(kvw[q]));
-    L.w.push_back(std::get<2>(kvw[q]));
-  }
-  if (!kvw.empty()) L.ptr.push_back(int64_t(kvw.size()));
-  return L;
-}
-
 static void run_segments(gdsw_ctx* c, SegList& L, const double* src, double* dst, DevArena& tmp) {
   if (L.key.empty()) return;
   int64_t* k = tmp.upload(L.key, c->stream);
   int64_t* p = tmp.upload(L.ptr, c->stream);
   int64_t* q = tmp.upload(L.pos, c->stream);
-  double* w = L.w.empty() ? nullptr : tmp.upload(L.w, c->stream);
-  segsum(k, p, q, w, int64_t(L.key.size()), src, dst, c->stream);
+  segsum(k, p, q, int64_t(L.key.size()), src, dst, c->stream);
 }
 
 // ------------------------------------------------------------------ factor storage
@@ -825,39 +804,8 @@ static void level1_coarse(gdsw_ctx* c, double* A0, double& minpiv) {
       SegList L = make_segments(kv);
       run_segments(c, L, Z, A0, tmp);
     }
-    {
-      // interface-interface couplings: positions into the value array
-      const MeshHost& M = c->mesh;
-      // (Phi_G^T A_GG Phi_G)_{kl} = sum over entries (a, k, w_a) and (b, l, w_b) of w_a w_b A_ab
-      std::vector<std::tuple<int64_t, int64_t, double>> kvw;
-      const int64_t bt0 = 9 * c->nnzb, b0 = bt0 + 3 * c->nbt;
-      for (int k = 0; k < C.n0; ++k) {
-        std::vector<std::tuple<int, int64_t, double>> row;
-        auto add = [&](int64_t b, int64_t pos, double wa) {
-          for (int32_t e = gamma_ptr[b]; e < gamma_ptr[b + 1]; ++e) row.emplace_back(C.gcol[e], pos, wa * C.gval[e]);
-        };
-        for (int32_t e = C.rg_ptr[k]; e < C.rg_ptr[k + 1]; ++e) {
-          int64_t a = C.rg_dof[e];
-          const double wa = C.rg_val[e];
-          if (a < M.nu) {
-            int64_t I = a / 3;
-            int cc = int(a - 3 * I);
-            for (int32_t blk = M.a_ptr[I]; blk < M.a_ptr[I + 1]; ++blk)
-              for (int d = 0; d < 3; ++d) add(3 * int64_t(M.a_col[blk]) + d, int64_t(blk) * 9 + cc * 3 + d, wa);
-            for (int32_t q = M.bt_ptr[I]; q < M.bt_ptr[I + 1]; ++q) add(M.nu + M.bt_col[q], bt0 + int64_t(q) * 3 + cc, wa);
-          } else {
-            int64_t P = a - M.nu;
-            for (int32_t q = M.b_ptr[P]; q < M.b_ptr[P + 1]; ++q)
-              for (int d = 0; d < 3; ++d) add(3 * int64_t(M.b_col[q]) + d, b0 + int64_t(q) * 3 + d, wa);
-          }
-        }
-        std::stable_sort(row.begin(), row.end(),
-                         [](const auto& x, const auto& y) { return std::get<0>(x) < std::get<0>(y); });
-        for (auto& pr : row) kvw.emplace_back(int64_t(k) * n0 + std::get<0>(pr), std::get<1>(pr), std::get<2>(pr));
-      }
-      SegList L = make_segments_w(kvw);
-      run_segments(c, L, c->d_val, A0, tmp);
-    }
+    // interface-interface couplings
+    gamma_gamma(tmp, A, c->ld[0].rg_ptr, c->ld[0].rg_dof, c->ld[0].rg_val, d_gc, d_gcol, d_gval, n0, A0, s);
     // store Phi_I^T in the storage precision
     std::vector<int32_t> phild;
     std::vector<int64_t> phioff = phi_offsets(C, phild);

@@ -5,6 +5,8 @@
 //  - the right-hand sides -A_IGamma Phi_Gamma of the coarse-basis extension, and the
 //    pieces of the Galerkin product A_0 = Phi^T A Phi;
 //  - dense gathers and basis assembly on the coarse levels.
+#include <algorithm>
+
 #include "common.h"
 #include "kernels.h"
 #include "setup.h"
@@ -165,25 +167,120 @@ __global__ void k_yint(MatView A, SlabView S, const int32_t* __restrict__ ilocal
   }
 }
 
-// A0[key] += sum of (w *) src[pos] over a segment (deterministic list order; w null = 1)
+// A0[key] += sum of src[pos] over a segment (deterministic list order)
 __global__ void k_segsum(const int64_t* __restrict__ key, const int64_t* __restrict__ ptr,
-                         const int64_t* __restrict__ pos, const double* __restrict__ w, int64_t nseg,
-                         const double* __restrict__ src, double* __restrict__ dst) {
+                         const int64_t* __restrict__ pos, int64_t nseg, const double* __restrict__ src,
+                         double* __restrict__ dst) {
   int64_t s = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (s >= nseg) return;
   double acc = 0.0;
-  if (w)
-    for (int64_t e = ptr[s]; e < ptr[s + 1]; ++e) acc = fma(w[e], src[pos[e]], acc);
-  else
-    for (int64_t e = ptr[s]; e < ptr[s + 1]; ++e) acc += src[pos[e]];
+  for (int64_t e = ptr[s]; e < ptr[s + 1]; ++e) acc += src[pos[e]];
   dst[key[s]] += acc;
 }
 
-void segsum(const int64_t* key, const int64_t* ptr, const int64_t* pos, const double* w, int64_t nseg,
-            const double* src, double* dst, cudaStream_t s) {
+void segsum(const int64_t* key, const int64_t* ptr, const int64_t* pos, int64_t nseg, const double* src, double* dst,
+            cudaStream_t s) {
   if (nseg == 0) return;
-  k_segsum<<<int((nseg + 255) / 256), 256, 0, s>>>(key, ptr, pos, w, nseg, src, dst);
+  k_segsum<<<int((nseg + 255) / 256), 256, 0, s>>>(key, ptr, pos, nseg, src, dst);
   check_launch("k_segsum");
+}
+
+// Phi_Gamma^T A_GammaGamma Phi_Gamma: a warp runs over one of gridDim.y shares of the interface dofs
+// that carry coarse column k = blockIdx.x (value w_a) and over the nonzeros of their rows; a nonzero of
+// column b adds w_a w_b A_ab to entry (k, l) of the share's matrix for every Phi_Gamma entry
+// (b, l, w_b).  Lanes that meet in one l are summed in lane order by the lowest of them, so every
+// entry is one sum in list order, without atomics.  Bound by the latency of those additions (one
+// read-modify-write in L2 per 32 nonzeros).  Listing and sorting the products on the host instead took
+// 458 ms on the 32^3 channel and 30 of the 238 ms of a 16^3 set-up.
+__global__ void __launch_bounds__(32) k_gamma_gamma(MatView A, const int32_t* __restrict__ rg_ptr,
+                                                    const int32_t* __restrict__ rg_dof,
+                                                    const double* __restrict__ rg_val,
+                                                    const int32_t* __restrict__ gamma_ptr,
+                                                    const int32_t* __restrict__ gcol, const double* __restrict__ gval,
+                                                    int64_t n0, double* A0) {
+  const int k = blockIdx.x, lane = threadIdx.x;
+  double* row = A0 + (int64_t(blockIdx.y) * n0 + k) * n0;
+  auto add = [&](int64_t b, double v, bool on) {  // every lane of the warp
+    int32_t e = on ? gamma_ptr[b] : 0;
+    const int32_t e1 = on ? gamma_ptr[b + 1] : 0;
+    unsigned todo = __ballot_sync(0xffffffffu, e < e1);
+    while (todo) {
+      if ((todo >> lane) & 1u) {
+        const int l = gcol[e];
+        const double p = v * gval[e];
+        const unsigned same = __match_any_sync(todo, l);
+        const int first = __ffs(same) - 1;
+        double s = first == lane ? row[l] : 0.0;
+        // groups take their members in lane order, all groups at once
+        unsigned rest = same;
+        while (__any_sync(todo, rest != 0u)) {
+          const double q = __shfl_sync(todo, p, rest ? __ffs(rest) - 1 : lane);
+          if (rest) s += q;
+          rest &= rest - 1u;
+        }
+        if (first == lane) row[l] = s;
+        ++e;
+      }
+      __syncwarp();
+      todo = __ballot_sync(0xffffffffu, e < e1);
+    }
+  };
+  const int64_t q0 = rg_ptr[k], nq = rg_ptr[k + 1] - q0;
+  const int64_t q1 = q0 + nq * (blockIdx.y + 1) / gridDim.y;
+  for (int64_t q = q0 + nq * blockIdx.y / gridDim.y; q < q1; ++q) {
+    const int64_t g = rg_dof[q];
+    const double wa = rg_val[q];
+    if (g < A.nu) {
+      const int64_t I = g / 3;
+      const int c = int(g - 3 * I);
+      const int32_t b0 = A.a_ptr[I], nb = 3 * (A.a_ptr[I + 1] - b0);
+      for (int32_t i0 = 0; i0 < nb; i0 += 32) {
+        const int32_t i = i0 + lane, blk = b0 + i / 3, d = i % 3;
+        const bool on = i < nb;
+        add(on ? 3 * int64_t(A.a_col[blk]) + d : 0, on ? wa * A.aval[int64_t(blk) * 9 + c * 3 + d] : 0.0, on);
+      }
+      for (int32_t e0 = A.bt_ptr[I]; e0 < A.bt_ptr[I + 1]; e0 += 32) {
+        const int32_t e = e0 + lane;
+        const bool on = e < A.bt_ptr[I + 1];
+        add(on ? A.nu + A.bt_col[e] : 0, on ? wa * A.btval[int64_t(e) * 3 + c] : 0.0, on);
+      }
+    } else {
+      const int64_t P = g - A.nu;
+      const int32_t b0 = A.b_ptr[P], nb = 3 * (A.b_ptr[P + 1] - b0);
+      for (int32_t i0 = 0; i0 < nb; i0 += 32) {
+        const int32_t i = i0 + lane, e = b0 + i / 3, d = i % 3;
+        const bool on = i < nb;
+        add(on ? 3 * int64_t(A.b_col[e]) + d : 0, on ? wa * A.bval[int64_t(e) * 3 + d] : 0.0, on);
+      }
+    }
+  }
+}
+
+// A0 += the sum of the shares, in order
+__global__ void __launch_bounds__(256) k_add_shares(const double* __restrict__ part, int shares, int64_t n,
+                                                    double* __restrict__ A0) {
+  const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (i >= n) return;
+  double s = 0.0;
+  for (int k = 0; k < shares; ++k) s += part[k * n + i];
+  A0[i] += s;
+}
+
+// A0 += Phi_Gamma^T A_GammaGamma Phi_Gamma; eight shares per coarse column (fewer if their matrices
+// would exceed 1 GB)
+void gamma_gamma(DevArena& tmp, const MatView& A, const int32_t* rg_ptr, const int32_t* rg_dof, const double* rg_val,
+                 const int32_t* gamma_ptr, const int32_t* gcol, const double* gval, int64_t n0, double* A0,
+                 cudaStream_t s) {
+  if (n0 == 0) return;
+  const int shares = int(std::max<int64_t>(1, std::min<int64_t>(8, (int64_t(1) << 27) / (n0 * n0))));
+  double* part = tmp.alloc<double>(size_t(shares) * n0 * n0);
+  GDSW_CUDA(cudaMemsetAsync(part, 0, size_t(shares) * n0 * n0 * sizeof(double), s));
+  k_gamma_gamma<<<dim3(unsigned(n0), unsigned(shares)), 32, 0, s>>>(A, rg_ptr, rg_dof, rg_val, gamma_ptr, gcol, gval,
+                                                                    n0, part);
+  check_launch("k_gamma_gamma");
+  k_add_shares<<<unsigned((n0 * n0 + 255) / 256), 256, 0, s>>>(part, shares, n0 * n0, A0);
+  check_launch("k_add_shares");
+  tmp.release(part);
 }
 
 // ------------------------------------------------------------------ dense helpers (coarse levels)

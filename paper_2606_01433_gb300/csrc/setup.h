@@ -28,9 +28,11 @@ struct SlabView {
 template <typename T>
 void extract_slabs(const MatView& A, const SlabView& S, int64_t p0, int64_t p1, int i0, int separate,
                    const int32_t* map, T* fac, int* err, cudaStream_t s);
-void segsum(const int64_t* key, const int64_t* ptr, const int64_t* pos, const double* w, int64_t nseg, const double* src,
-            double* dst,
+void segsum(const int64_t* key, const int64_t* ptr, const int64_t* pos, int64_t nseg, const double* src, double* dst,
             cudaStream_t s);
+void gamma_gamma(DevArena& tmp, const MatView& A, const int32_t* rg_ptr, const int32_t* rg_dof, const double* rg_val,
+                 const int32_t* gamma_ptr, const int32_t* gcol, const double* gval, int64_t n0, double* A0,
+                 cudaStream_t s);
 template <typename T>
 void gather_dense(const double* A, int64_t n, const int32_t* dofs, const int64_t* doff, const int32_t* part_of_row,
                   int64_t nrows, const int64_t* out_off, const int32_t* out_ld, T* out, cudaStream_t s);
