@@ -247,8 +247,9 @@ int gdsw_newton_step(gdsw_ctx* ctx, double* x, gdsw_solve_info* info);
  * FGMRES preconditioned by V-cycles.  A smoothing step is a multiplicative sweep over the
  * eight element colours (parity of the voxel indices): r = b - A z, then every patch e of the
  * colour adds omega A_e^{-1} r_e to z; FP64 smoothing forms r with the FP64 SpMV, FP32
- * smoothing only on the rows the colour's patches touch, with FP32 operator values copied
- * when the multigrid is created (re-create it after re-assembling a grid's operator).  The multigrid object does not own the grid
+ * smoothing in FP32 products with the operator as it is when the multigrid is created (an FP32
+ * copy of its viscosity, or of its values if it is a Newton Jacobian; re-create the multigrid
+ * after re-assembling a grid's operator).  The multigrid object does not own the grid
  * contexts; destroy it before them.  Errors as for the other calls; a failed create leaves
  * its reason in gdsw_mg_last_error(NULL). */
 typedef struct gdsw_mg gdsw_mg;

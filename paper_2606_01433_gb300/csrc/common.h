@@ -414,6 +414,7 @@ struct gdsw_ctx {
   int32_t *d_lift_elem = nullptr, *d_lift_dof = nullptr, *d_lift_ptr = nullptr, *d_lift_src = nullptr;
   uint32_t* d_lift_mask = nullptr;
   double* d_lift_work = nullptr;    // contributions of the lift elements
+  bool jacobian = false;            // the assembled operator holds the Newton term
   bool b_assembled = false;         // B does not depend on the viscosity: assembled once
   unsigned* d_sweep_flag = nullptr; // set by a persistent sweep whose wait ran out
   double* d_gdir = nullptr;         // Dirichlet datum, 3 per node

@@ -21,12 +21,14 @@
 // A smoothing step sweeps the eight colours: r = b - A z, then one warp per patch of the colour
 // computes A_e^{-1} r_e and adds omega times it to z (no two patches of a colour share a dof, so
 // the additions need no ordering).  FP64 smoothing forms r with the full FP64 SpMV; FP32
-// smoothing forms it only on the rows the colour's patches touch (about (3/4)^3 of them), with
-// an FP32 copy of the operator taken when the multigrid is created.
+// smoothing forms A z element by element from an FP32 copy of the viscosity taken when the multigrid
+// is created (from FP32 operator values on the rows a colour's patches touch, if the operator holds
+// the Newton term).
 #include <algorithm>
 #include <cmath>
 
 #include "common.h"
+#include "element.h"
 #include "kernels.h"
 #include "setup.h"
 
@@ -36,7 +38,11 @@ void apply_precond(gdsw_ctx* c, const double* r, double* z, cudaStream_t s);
 static thread_local std::string g_mg_create_error;  // why the last gdsw_mg_create of this thread failed
 
 constexpr int PMAX = 96;  // padded patch size (27 x 3 velocity + 8 pressure dofs at most)
+constexpr int VT = 64;    // threads of a Vanka CTA (a warp per patch): small CTAs spread 512 patches over the SMs
+constexpr int64_t kPrefetchBytes = int64_t(80) << 20;  // patch inverses fetched ahead: most of L2
+constexpr int ES = 96;    // values of an element residual: 27 x 3 velocity, 8 pressure, padding
 
+struct ElementTables;
 struct MgGrid {
   gdsw_ctx* ctx = nullptr;
   int64_t n = 0;
@@ -46,8 +52,18 @@ struct MgGrid {
   int32_t* d_pdof = nullptr;   // npatch x PMAX dofs, -1 padding
   void* d_pinv = nullptr;      // npatch x PMAX x PMAX, column-major inverse (FP32 or FP64)
   double minpiv = 0;
-  // FP32 smoothing: an FP32 copy of the operator's values (taken at creation) and, per colour,
-  // the velocity-node and pressure rows its patches touch (the residual is formed there only)
+  // FP32 smoothing, matrix-free (d_f32 set): per element, in patch order, the velocity index of its
+  // 27 nodes and the pressure index of its 8 vertices (-1: none), the viscosity times quadrature weight
+  // at its Gauss points in two FP32 words (taken at creation), the element residuals (ES values each), and per
+  // velocity node / pressure dof the positions of its contributions
+  int32_t *d_evel = nullptr, *d_epre = nullptr;
+  float2* d_f32 = nullptr;
+  float *d_eres = nullptr, *d_zf = nullptr;  // d_zf: FP32 copy of the iterate
+  ElementTables* d_tables = nullptr;
+  int32_t *d_vptr = nullptr, *d_vsrc = nullptr, *d_pptr = nullptr, *d_psrc = nullptr;
+  // FP32 smoothing of an operator with the Newton term (d_a32 set): an FP32 copy of its values (taken
+  // at creation) and, per colour, the velocity-node and pressure rows its patches touch (the residual is
+  // formed there only)
   float *d_a32 = nullptr, *d_bt32 = nullptr, *d_b32 = nullptr;
   int32_t* d_rows = nullptr;   // per colour: velocity nodes, then pressure indices
   int64_t vrow_off[9] = {0}, prow_off[9] = {0};
@@ -76,6 +92,7 @@ namespace gdsw {
 // ------------------------------------------------------------------ host symbolic work
 struct PatchHost {
   std::vector<int32_t> dof;  // npatch x PMAX
+  std::vector<int32_t> felem;  // fluid element of each patch
   int64_t off[9] = {0};
 };
 
@@ -112,9 +129,53 @@ static PatchHost build_patches(const MeshHost& M) {
       std::sort(d.begin(), d.end());
       GDSW_CHECK(int(d.size()) <= PMAX, GDSW_ERR_INVALID_ARG, "Vanka patch larger than its padding");
       std::copy(d.begin(), d.end(), P.dof.begin() + size_t(q) * PMAX);
+      P.felem.push_back(M.felem[e]);
       ++q;
     }
   return P;
+}
+
+// nodes of every element (patch order) and where each velocity node and pressure dof finds its
+// contributions among the element residuals (elements in patch order)
+struct ElementHost {
+  std::vector<int32_t> vel, pre, vptr, vsrc, pptr, psrc;
+};
+static ElementHost element_lists(const MeshHost& M, const PatchHost& P) {
+  const int64_t np = int64_t(P.felem.size());
+  GDSW_CHECK(np * ES < (int64_t(1) << 31), GDSW_ERR_INVALID_ARG, "too many elements for the multigrid smoother");
+  ElementHost E;
+  E.vel.resize(size_t(np) * 27);
+  E.pre.resize(size_t(np) * 8);
+  E.vptr.assign(size_t(M.nv) + 1, 0);
+  E.pptr.assign(size_t(M.np) + 1, 0);
+  for (int64_t q = 0; q < np; ++q) {
+    const int64_t e = M.fluid[P.felem[q]];
+    const int ex = int(e % M.nx), ey = int((e / M.nx) % M.ny), ez = int(e / (int64_t(M.nx) * M.ny));
+    for (int a = 0; a < 27; ++a) {
+      const int x = a % 3, y = (a / 3) % 3, z = a / 9;
+      const int64_t node = (2 * ex + x) + int64_t(M.NX) * ((2 * ey + y) + int64_t(M.NY) * (2 * ez + z));
+      const int32_t v = M.vidx[node];
+      E.vel[q * 27 + a] = v;
+      if (v >= 0) ++E.vptr[v + 1];
+      if ((x | y | z) % 2 == 0) {
+        const int32_t pr = M.pidx[node];
+        E.pre[q * 8 + x / 2 + y + 2 * z] = pr;
+        if (pr >= 0) ++E.pptr[pr + 1];
+      }
+    }
+  }
+  for (int64_t v = 0; v < M.nv; ++v) E.vptr[v + 1] += E.vptr[v];
+  for (int64_t v = 0; v < M.np; ++v) E.pptr[v + 1] += E.pptr[v];
+  E.vsrc.resize(E.vptr[M.nv]);
+  E.psrc.resize(E.pptr[M.np]);
+  std::vector<int32_t> vf(E.vptr.begin(), E.vptr.end() - 1), pf(E.pptr.begin(), E.pptr.end() - 1);
+  for (int64_t q = 0; q < np; ++q) {
+    for (int a = 0; a < 27; ++a)
+      if (E.vel[q * 27 + a] >= 0) E.vsrc[vf[E.vel[q * 27 + a]]++] = int32_t(q * ES + 3 * a);
+    for (int k = 0; k < 8; ++k)
+      if (E.pre[q * 8 + k] >= 0) E.psrc[pf[E.pre[q * 8 + k]]++] = int32_t(q * ES + 81 + k);
+  }
+  return E;
 }
 
 // per colour, the velocity nodes and pressure indices that its patches touch (sorted)
@@ -336,39 +397,212 @@ __global__ void k_patch_store(const double* __restrict__ inv, const int32_t* __r
   }
 }
 
-// one warp per patch of a colour: z[d] += omega A_e^{-1} r[d]; lane owns rows lane + 32 k
-template <typename TM>
-__global__ void __launch_bounds__(256) k_vanka(const int32_t* __restrict__ pdof, const TM* __restrict__ pinv,
+// FP32 tables of the element operator, values and their rounding errors: the one-dimensional basis and
+// the element's -int psi_k d_c phi_a as [(8 c + k) / 4][a][k % 4]
+struct ElementTables {
+  alignas(16) float div[6][32][4];
+  float divl[6][32][4];
+  Grad1D<float> B;
+};
+
+// A_e z_e of every element in FP32, matrix-free: one warp per element, lane = node, then Gauss point,
+// then node; gradient, stress and test integrals by sum factorisation, the divergence from
+// tabulated integrals (ten thousand products per element: FP32 is cheap here, while any FP64
+// instruction, conversions included, holds the pipe for 16 cycles -- hence z in FP32, zf, kept beside
+// z by the smoother).  With the assembled rows each colour of a sweep read the 36-byte blocks of the rows its patches touch, 425 MB of a
+// 32^3 grid; the elements read z and 27 viscosities each and write 12 MB, which stays in L2.
+// Measured per colour (both launches): 32^3 grid ~145 -> 73 us, 16^3 ~30 -> 17 us; several elements
+// per warp, with the tables kept in registers, were slower (84 and 21 us: half the warps).  Against FP64
+// smoothing the error of a V-cycle is 2.7e-7 (3.2e-7 with assembled rows), of one sweep from random
+// data 2.1e-7 (2.1e-7).
+__global__ void __launch_bounds__(128) k_element_residuals(const int32_t* __restrict__ evel,
+                                                           const int32_t* __restrict__ epre,
+                                                           const float2* __restrict__ f32, int64_t ne, int form,
+                                                           const ElementTables* __restrict__ T, int64_t nu,
+                                                           const float* zf, float* __restrict__ out,
+                                                           const char* __restrict__ next, int64_t next_bytes) {
+  __shared__ Grad1D<float> B;
+  __shared__ float su[4][3][27], ss[4][3][3][27], st[4][3][3][27], sp[4][8];
+  dep_release();
+  if (threadIdx.x < sizeof(Grad1D<float>) / 4)
+    reinterpret_cast<float*>(&B)[threadIdx.x] = reinterpret_cast<const float*>(&T->B)[threadIdx.x];
+  const int warp = threadIdx.x >> 5, q = threadIdx.x & 31;
+  const int64_t e = int64_t(blockIdx.x) * 4 + warp;
+  const bool here = e < ne, active = here && q < 27;
+  const int32_t v = active ? evel[e * 27 + q] : -1;
+  const int32_t p = here && q < 8 ? epre[e * 8 + q] : -1;
+  const float2 f = active ? f32[e * 27 + q] : make_float2(0.f, 0.f);
+  float dt[24], dl[24];
+#pragma unroll
+  for (int k = 0; k < 24; k += 4) {
+    const float4 h = *reinterpret_cast<const float4*>(T->div[k / 4][q]);  // zero from lane 27 on
+    const float4 l = *reinterpret_cast<const float4*>(T->divl[k / 4][q]);
+    dt[k] = h.x, dt[k + 1] = h.y, dt[k + 2] = h.z, dt[k + 3] = h.w;
+    dl[k] = l.x, dl[k + 1] = l.y, dl[k + 2] = l.z, dl[k + 3] = l.w;
+  }
+  // this colour's patch inverses, which the next launch streams: DRAM is idle here
+  for (int64_t b = (int64_t(blockIdx.x) * 128 + threadIdx.x) * 128; b < next_bytes; b += int64_t(gridDim.x) * 128 * 128)
+    prefetch_l2(next + b);
+  __syncthreads();
+  dep_wait();
+  if (!here) return;
+  float (*u)[27] = su[warp];
+  float (*s)[3][27] = ss[warp];
+  float (*t)[3][27] = st[warp];
+  float uq[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    uq[c] = v >= 0 ? __ldcg(zf + 3 * int64_t(v) + c) : 0.f;
+    if (active) u[c][q] = uq[c];
+  }
+  if (q < 8) sp[warp][q] = p >= 0 ? __ldcg(zf + nu + p) : 0.f;
+  __syncwarp();
+  // divergence coupling from the tabulated integrals, both ways: the pressure's part of this node's
+  // velocity rows, and this node's part of the eight pressure rows (lane l gets row l & 7)
+  float rp[3], d8[8], d4[4], d2[2];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    rp[c] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) rp[c] = fmaf(dl[8 * c + k], sp[warp][k], rp[c]);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) rp[c] = fmaf(dt[8 * c + k], sp[warp][k], rp[c]);
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    d8[k] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d8[k] = fmaf(dl[8 * c + k], uq[c], d8[k]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d8[k] = fmaf(dt[8 * c + k], uq[c], d8[k]);
+  }
+  const bool h4 = q & 4, h2 = q & 2, h1 = q & 1;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) d4[k] = (h4 ? d8[k + 4] : d8[k]) + __shfl_xor_sync(0xffffffffu, h4 ? d8[k] : d8[k + 4], 4);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) d2[k] = (h2 ? d4[k + 2] : d4[k]) + __shfl_xor_sync(0xffffffffu, h2 ? d4[k] : d4[k + 2], 2);
+  float d = (h1 ? d2[1] : d2[0]) + __shfl_xor_sync(0xffffffffu, h1 ? d2[0] : d2[1], 1);
+  d += __shfl_xor_sync(0xffffffffu, d, 8);
+  d += __shfl_xor_sync(0xffffffffu, d, 16);
+  float gr[3][3] = {};
+  element_gradient<float>(B, q, active, u, s, t, gr, [] { __syncwarp(); });
+  __syncwarp();
+  if (active)
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int l = 0; l < 3; ++l) {
+        const float g = form == GDSW_FORM_SYMMETRIC ? gr[c][l] + gr[l][c] : gr[c][l];
+        s[c][l][q] = fmaf(f.x, g, f.y * g);
+      }
+  __syncwarp();
+  float r[3];
+  element_test<float>(B, q, active, s, t, r, [] { __syncwarp(); });
+  float* o = out + e * ES;
+  if (active)  // through shared memory: the element's 81 values leave as whole lines
+#pragma unroll
+    for (int c = 0; c < 3; ++c) (&u[0][0])[3 * q + c] = r[c] + rp[c];
+  __syncwarp();
+  for (int i = q; i < 81; i += 32) o[i] = (&u[0][0])[i];
+  if (q < 8) o[81 + q] = d;
+}
+
+__global__ void k_scaled_nu(const int32_t* __restrict__ felem, int64_t ne, const double* __restrict__ nu,
+                            const RefTables* __restrict__ T, double sc, float2* __restrict__ f32) {
+  const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (i >= ne * 27) return;
+  const int64_t e = i / 27, q = i - 27 * e;
+  const double f = nu[int64_t(felem[e]) * 27 + q] * T->w[q] * sc;
+  f32[i] = make_float2(float(f), float(f - double(float(f))));
+}
+
+// One warp per patch of a colour: z[d] += omega A_e^{-1} r[d]; lane owns rows lane + 32 k.  The residual
+// comes formed (r), or MF: as b minus the sum of the element residuals of each dof.
+struct ElementSum {
+  const double* b;
+  float* zf;  // FP32 copy of z
+  const float* eres;
+  const int32_t *vptr, *vsrc, *pptr, *psrc;
+  int64_t nu;
+};
+template <typename TM, bool MF>
+__global__ void __launch_bounds__(VT, 16) k_vanka(const int32_t* __restrict__ pdof, const TM* __restrict__ pinv,
                                                int64_t p0, int64_t p1, const double* __restrict__ r,
-                                               double* __restrict__ z, double omega) {
+                                               const ElementSum E, double* __restrict__ z, double omega) {
   const int64_t q = p0 + (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) / 32;
   const int lane = threadIdx.x & 31;
   dep_release();
   if (q < p1)  // the patch inverse is set-up data: its first 4 KB go to L2 before the wait
     prefetch_l2(reinterpret_cast<const char*>(pinv + q * PMAX * PMAX) + 128 * lane);
-  dep_wait();
+  if (!MF) dep_wait();
   if (q >= p1) return;
   const int32_t* d = pdof + q * PMAX;
   const TM* M = pinv + q * PMAX * PMAX;
   int32_t dof[3];
   TM rv[3], y[3] = {TM(0), TM(0), TM(0)};
+  if (MF) {
+    int32_t src[3][8], cnt[3], off[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    dof[k] = d[lane + 32 * k];
-    rv[k] = dof[k] >= 0 ? TM(r[dof[k]]) : TM(0);
+    for (int k = 0; k < 3; ++k) {
+      dof[k] = d[lane + 32 * k];
+      cnt[k] = off[k] = 0;
+      const int32_t* list = E.vsrc;
+      if (dof[k] >= 0) {
+        const bool vel = dof[k] < E.nu;
+        const int32_t n = vel ? dof[k] / 3 : int32_t(dof[k] - E.nu);
+        const int32_t* ptr = (vel ? E.vptr : E.pptr) + n;
+        off[k] = vel ? dof[k] - 3 * n : 0;
+        const int32_t a = ptr[0];
+        cnt[k] = ptr[1] - a;
+        list = (vel ? E.vsrc : E.psrc) + a;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) src[k][i] = i < cnt[k] ? list[i] : 0;
+    }
+    dep_wait();
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      // the elements' parts cancel: their sum keeps its rounding error (two-sum)
+      float x[8], s = 0.f, lost = 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = i < cnt[k] ? __ldcg(E.eres + src[k][i] + off[k]) : 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float t = __fadd_rn(s, x[i]), v = __fsub_rn(t, s);
+        lost += __fadd_rn(__fsub_rn(s, __fsub_rn(t, v)), __fsub_rn(x[i], v));
+        s = t;
+      }
+      rv[k] = dof[k] >= 0 ? TM(E.b[dof[k]] - double(s)) - TM(lost) : TM(0);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      dof[k] = d[lane + 32 * k];
+      rv[k] = dof[k] >= 0 ? TM(r[dof[k]]) : TM(0);
+    }
   }
+  // four partial sums per row: shorter chains, and a smaller rounding error than one of 96 terms
+  TM acc[3][4] = {};
 #pragma unroll
   for (int k = 0; k < 3; ++k)
-#pragma unroll 8
-    for (int jj = 0; jj < 32; ++jj) {
-      const TM rj = __shfl_sync(0xffffffffu, rv[k], jj);
-      const TM* col = M + int64_t(32 * k + jj) * PMAX;
+#pragma unroll 2
+    for (int j0 = 0; j0 < 32; j0 += 4)
 #pragma unroll
-      for (int u = 0; u < 3; ++u) y[u] = fma(__ldcs(col + lane + 32 * u), rj, y[u]);
-    }
+      for (int j = 0; j < 4; ++j) {
+        const TM rj = __shfl_sync(0xffffffffu, rv[k], j0 + j);
+        const TM* col = M + int64_t(32 * k + j0 + j) * PMAX;
+#pragma unroll
+        for (int u = 0; u < 3; ++u) acc[u][j] = fma(__ldcs(col + lane + 32 * u), rj, acc[u][j]);
+      }
+#pragma unroll
+  for (int u = 0; u < 3; ++u) y[u] = (acc[u][0] + acc[u][1]) + (acc[u][2] + acc[u][3]);
 #pragma unroll
   for (int u = 0; u < 3; ++u)
-    if (dof[u] >= 0) z[dof[u]] += omega * double(y[u]);
+    if (dof[u] >= 0) {
+      const double v = z[dof[u]] + omega * double(y[u]);
+      z[dof[u]] = v;
+      if (MF) E.zf[dof[u]] = float(v);
+    }
 }
 
 // r = b - A z on the velocity-node rows of a list, FP32 operator values and products, FP64
@@ -438,7 +672,9 @@ __global__ void __launch_bounds__(256) k_resid_prows(const int32_t* __restrict__
   if (lane == 0) r[nu + P] = b[nu + P] - double(s);
 }
 
-__global__ void k_to_f32(const double* __restrict__ a, float* __restrict__ b, int64_t n) {
+__global__ void k_to_f32(const double* a, float* __restrict__ b, int64_t n) {
+  dep_release();
+  dep_wait();
   const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
   if (i < n) b[i] = float(a[i]);
 }
@@ -465,7 +701,7 @@ static void csr_mv(const int32_t* ptr, const int32_t* col, const double* val, co
 
 // ------------------------------------------------------------------ the cycle
 // r = b - A z where colour c's patches need it: the full FP64 SpMV for FP64 smoothing, the
-// colour's rows in FP32 products otherwise
+// colour's rows in FP32 products for an operator with the Newton term
 static void colour_residual(gdsw_mg* mg, MgGrid& G, int c, const double* b, const double* z, cudaStream_t s) {
   if (mg->opt.smoother_precision == GDSW_FP64) {
     launch_spmv(G.ctx, z, G.d_r, b, s);
@@ -489,19 +725,35 @@ static void colour_residual(gdsw_mg* mg, MgGrid& G, int c, const double* b, cons
 static void smooth(gdsw_mg* mg, int l, const double* b, double* z, int steps, bool reverse = false) {
   MgGrid& G = mg->g[l];
   cudaStream_t s = mg->s;
+  const gdsw_ctx* x = G.ctx;
+  const ElementSum E{b, G.d_zf, G.d_eres, G.d_vptr, G.d_vsrc, G.d_pptr, G.d_psrc, x->mesh.nu};
+  if (G.d_f32 && steps > 0) {
+    launch_chained(k_to_f32, dim3(unsigned((G.n + 255) / 256)), dim3(256), 0, s, z, G.d_zf, G.n);
+    check_launch("k_to_f32");
+  }
   for (int it = 0; it < steps; ++it)
     for (int cc = 0; cc < 8; ++cc) {
       const int c = reverse ? 7 - cc : cc;
       const int64_t p0 = G.colour_off[c], p1 = G.colour_off[c + 1];
       if (p1 == p0) continue;
-      colour_residual(mg, G, c, b, z, s);
-      const int blocks = int((p1 - p0 + 7) / 8);
-      if (mg->opt.smoother_precision == GDSW_FP64)
-        launch_chained(k_vanka<double>, dim3(unsigned(blocks)), dim3(256), 0, s, G.d_pdof,
-                       static_cast<const double*>(G.d_pinv), p0, p1, G.d_r, z, mg->opt.omega);
-      else
-        launch_chained(k_vanka<float>, dim3(unsigned(blocks)), dim3(256), 0, s, G.d_pdof,
-                       static_cast<const float*>(G.d_pinv), p0, p1, G.d_r, z, mg->opt.omega);
+      const dim3 grid(unsigned((p1 - p0 + VT / 32 - 1) / (VT / 32)));
+      if (G.d_f32) {
+        launch_chained(k_element_residuals, dim3(unsigned((G.npatch + 3) / 4)), dim3(128), 0, s, G.d_evel, G.d_epre,
+                       G.d_f32, G.npatch, x->form, G.d_tables, x->mesh.nu, G.d_zf, G.d_eres,
+                       reinterpret_cast<const char*>(static_cast<const float*>(G.d_pinv) + p0 * PMAX * PMAX),
+                       std::min<int64_t>((p1 - p0) * PMAX * PMAX * int64_t(sizeof(float)), kPrefetchBytes));
+        check_launch("k_element_residuals");
+        launch_chained(k_vanka<float, true>, grid, dim3(VT), 0, s, G.d_pdof, static_cast<const float*>(G.d_pinv), p0,
+                       p1, G.d_r, E, z, mg->opt.omega);
+      } else {
+        colour_residual(mg, G, c, b, z, s);
+        if (mg->opt.smoother_precision == GDSW_FP64)
+          launch_chained(k_vanka<double, false>, grid, dim3(VT), 0, s, G.d_pdof,
+                         static_cast<const double*>(G.d_pinv), p0, p1, G.d_r, E, z, mg->opt.omega);
+        else
+          launch_chained(k_vanka<float, false>, grid, dim3(VT), 0, s, G.d_pdof, static_cast<const float*>(G.d_pinv),
+                         p0, p1, G.d_r, E, z, mg->opt.omega);
+      }
       check_launch("k_vanka");
     }
 }
@@ -623,7 +875,37 @@ static void mg_create(gdsw_mg* mg, gdsw_ctx* const* grids, int ngrids, const gds
       throw;
     }
     tmp.free_all();
-    if (opt->smoother_precision == GDSW_FP32) {
+    if (opt->smoother_precision == GDSW_FP32 && !G.ctx->jacobian) {
+      const ElementHost E = element_lists(M, P);
+      const gdsw_ctx* x = G.ctx;
+      G.d_evel = mg->arena.upload(E.vel, s);
+      G.d_epre = mg->arena.upload(E.pre, s);
+      G.d_vptr = mg->arena.upload(E.vptr, s);
+      G.d_vsrc = mg->arena.upload(E.vsrc, s);
+      G.d_pptr = mg->arena.upload(E.pptr, s);
+      G.d_psrc = mg->arena.upload(E.psrc, s);
+      G.d_eres = mg->arena.alloc<float>(size_t(G.npatch) * ES);
+      G.d_f32 = mg->arena.alloc<float2>(size_t(G.npatch) * 27);
+      G.d_zf = mg->arena.alloc<float>(size_t(G.n));
+      RefTables R;
+      host_tables(R);
+      std::vector<ElementTables> H(1);
+      host_grad1d(H[0].B);
+      const double ps = 0.25 * x->mesh.h * x->mesh.h;
+      for (int a = 0; a < 27; ++a)
+        for (int k = 0; k < 8; ++k)
+          for (int c = 0; c < 3; ++c) {
+            const double v = ps * R.div[k][a][c];
+            H[0].div[(8 * c + k) / 4][a][k % 4] = float(v);
+            H[0].divl[(8 * c + k) / 4][a][k % 4] = float(v - double(float(v)));
+          }
+      G.d_tables = mg->arena.upload(H, s);
+      int32_t* fe = mg->arena.upload(P.felem, s);
+      k_scaled_nu<<<unsigned((G.npatch * 27 + 255) / 256), 256, 0, s>>>(
+          fe, G.npatch, x->d_nu, static_cast<RefTables*>(x->d_tables), 0.5 * x->mesh.h, G.d_f32);
+      check_launch("k_scaled_nu");
+      GDSW_CUDA(cudaStreamSynchronize(s));  // the uploads' host arrays end here
+    } else if (opt->smoother_precision == GDSW_FP32) {
       std::vector<int32_t> rows;
       colour_rows(M, P, rows, G.vrow_off, G.prow_off);
       G.d_rows = mg->arena.upload(rows, s);

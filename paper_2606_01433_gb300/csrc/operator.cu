@@ -7,6 +7,7 @@
 // a fluid element (row-major block, 72 bytes); pressure-velocity entries as 3-vectors in
 // both row orientations (B rows per pressure node, B^T rows per velocity node).
 #include "common.h"
+#include "element.h"
 #include "kernels.h"
 
 namespace gdsw {
@@ -74,66 +75,6 @@ __device__ __forceinline__ int shared_range(int a, int b, int n, int& e0) {
   return e1 >= e0 ? e1 - e0 + 1 : 0;
 }
 
-// one-dimensional Q2 basis / derivative a at Gauss point q
-__host__ __device__ constexpr double gauss_x(int q) { return q == 0 ? -0.7745966692414834 : (q == 1 ? 0.0 : 0.7745966692414834); }
-__host__ __device__ constexpr double q2_v(int a, int q) {
-  const double x = gauss_x(q);
-  return a == 0 ? 0.5 * x * (x - 1.0) : (a == 1 ? 1.0 - x * x : 0.5 * x * (x + 1.0));
-}
-__host__ __device__ constexpr double q2_d(int a, int q) {
-  const double x = gauss_x(q);
-  return a == 0 ? x - 0.5 : (a == 1 ? -2.0 * x : x + 0.5);
-}
-
-// ------------------------------------------------------------------ sum factorisation on one element
-// Values of the 27 nodes of an element -> reference gradients at its 27 Gauss points, one axis at a
-// time (the Q2 basis is a tensor product: 72 multiply-adds per point and component triple instead
-// of 243).  Thread q = 0..26 of the element owns node q, then the partial results of index q, then
-// Gauss point q (x fastest throughout); u, s, t are the element's shared arrays [c][27], `sync` is
-// a barrier over the element's threads.
-struct Grad1D {
-  double v[3][3], d[3][3];   // [basis][point]
-};
-__device__ __forceinline__ void fill_grad1d(Grad1D& B, int tid) {
-  if (tid < 9) {
-    B.v[tid / 3][tid % 3] = q2_v(tid / 3, tid % 3);
-    B.d[tid / 3][tid % 3] = q2_d(tid / 3, tid % 3);
-  }
-}
-template <typename Sync>
-__device__ __forceinline__ void element_gradient(const Grad1D& B, int q, bool active, double (*u)[27],
-                                                 double (*s)[3][27], double (*t)[3][27], double gr[3][3],
-                                                 Sync sync) {
-  const int x = q % 3, y = (q / 3) % 3, z = q / 9;
-  if (active)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {  // along x: values s[0], derivatives s[1]
-      const double* p = u[c] + q - x;
-      s[0][c][q] = fma(p[2], B.v[2][x], fma(p[1], B.v[1][x], p[0] * B.v[0][x]));
-      s[1][c][q] = fma(p[2], B.d[2][x], fma(p[1], B.d[1][x], p[0] * B.d[0][x]));
-    }
-  sync();
-  if (active)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {  // along y: dx t[0], dy t[1], no derivative t[2]
-      const double* p = s[0][c] + q - 3 * y;
-      const double* d = s[1][c] + q - 3 * y;
-      t[0][c][q] = fma(d[6], B.v[2][y], fma(d[3], B.v[1][y], d[0] * B.v[0][y]));
-      t[1][c][q] = fma(p[6], B.d[2][y], fma(p[3], B.d[1][y], p[0] * B.d[0][y]));
-      t[2][c][q] = fma(p[6], B.v[2][y], fma(p[3], B.v[1][y], p[0] * B.v[0][y]));
-    }
-  sync();
-  if (active)
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int l = 0; l < 3; ++l) {
-        const double* p = t[l][c] + q - 9 * z;
-        const double(*b)[3] = l == 2 ? B.d : B.v;
-        gr[c][l] = fma(p[18], b[2][z], fma(p[9], b[1][z], p[0] * b[0][z]));
-      }
-}
-
 // ------------------------------------------------------------------ a1: Carreau viscosity
 // dn (optional, Newton linearisation of Section 3): per Gauss point D(u_k) (xx, yy, zz, xy, xz,
 // yz) and N = 4 nu'(gamma_dot) / gamma_dot = 4 (nu0 - nu_inf)(n - 1) lambda^2
@@ -147,7 +88,7 @@ __global__ void __launch_bounds__(256) k_viscosity(const int32_t* __restrict__ f
                                                    const double* __restrict__ uk, Geo G, int form, int has_uk,
                                                    double nu0, double nu_inf, double lam, double ncar,
                                                    double* __restrict__ nu, double* __restrict__ dn) {
-  __shared__ Grad1D B;
+  __shared__ Grad1D<double> B;
   __shared__ double u[kViscElems][3][27], s[kViscElems][2][3][27], w[kViscElems][3][3][27];
   dep_release();
   dep_wait();
@@ -172,7 +113,7 @@ __global__ void __launch_bounds__(256) k_viscosity(const int32_t* __restrict__ f
   __syncthreads();
   double gr[3][3];
   const int se = active ? el : 0;
-  element_gradient(B, q, active, u[se], s[se], w[se], gr, [] { __syncthreads(); });
+  element_gradient<double>(B, q, active, u[se], s[se], w[se], gr, [] { __syncthreads(); });
   if (!active) return;
   const double sc = 2.0 / G.h;
   double dd = 0.0;  // D : D
@@ -526,7 +467,7 @@ __global__ void __launch_bounds__(128) k_lift_elements(const int32_t* __restrict
                                                        const int32_t* __restrict__ fluid, Geo G, int form, int pdisc,
                                                        const double* __restrict__ nu, const RefTables* __restrict__ T,
                                                        const double* __restrict__ g, double* __restrict__ lw) {
-  __shared__ Grad1D B;
+  __shared__ Grad1D<double> B;
   __shared__ double su[4][3][27], ss[4][3][3][27], st[4][3][3][27];
   __shared__ double sdiv[4][27];
   dep_release();
@@ -551,7 +492,7 @@ __global__ void __launch_bounds__(128) k_lift_elements(const int32_t* __restrict
   }
   __syncwarp();
   double gr[3][3];
-  element_gradient(B, q, active, u, s, t, gr, [] { __syncwarp(); });
+  element_gradient<double>(B, q, active, u, s, t, gr, [] { __syncwarp(); });
   __syncwarp();
   const int x = q % 3, y = (q / 3) % 3, z = q / 9;
   if (active) {
@@ -563,40 +504,12 @@ __global__ void __launch_bounds__(128) k_lift_elements(const int32_t* __restrict
       for (int l = 0; l < 3; ++l) s[c][l][q] = f * (form == GDSW_FORM_SYMMETRIC ? gr[c][l] + gr[l][c] : gr[c][l]);
   }
   __syncwarp();
-  if (active)  // test functions along z
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int l = 0; l < 3; ++l) {
-        const double* p = s[c][l] + q - 9 * z;
-        const double* b = l == 2 ? B.d[z] : B.v[z];
-        t[c][l][q] = fma(p[18], b[2], fma(p[9], b[1], p[0] * b[0]));
-      }
-  __syncwarp();
-  if (active)  // along y: s[c][0] still needs the x derivative, s[c][1] the x value
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double *p0 = t[c][0] + q - 3 * y, *p1 = t[c][1] + q - 3 * y, *p2 = t[c][2] + q - 3 * y;
-      double a = 0.0, b = 0.0;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        a = fma(p0[3 * k], B.v[y][k], a);
-        b = fma(p1[3 * k], B.d[y][k], fma(p2[3 * k], B.v[y][k], b));
-      }
-      s[c][0][q] = a;
-      s[c][1][q] = b;
-    }
-  __syncwarp();
   double* o = lw + le * kLiftValues;
+  double f[3];
+  element_test<double>(B, q, active, s, t, f, [] { __syncwarp(); });
   if (active)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double *p0 = s[c][0] + q - x, *p1 = s[c][1] + q - x;
-      double a = 0.0;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) a = fma(p0[k], B.d[x][k], fma(p1[k], B.v[x][k], a));
-      o[3 * q + c] = -a;
-    }
+    for (int c = 0; c < 3; ++c) o[3 * q + c] = -f[c];
   if (q < (pdisc ? 4 : 8)) {
     double a = 0.0;
     for (int k = 0; k < 27; ++k) a = fma(sdiv[warp][k], pdisc ? T->p1[k][q] : T->psi[k][q], a);
@@ -836,6 +749,7 @@ void launch_viscosity(gdsw_ctx* c, cudaStream_t s) {
 }
 
 void launch_assembly(gdsw_ctx* c, cudaStream_t s, bool newton) {
+  c->jacobian = newton;
   const auto* T = static_cast<RefTables*>(c->d_tables);
   const int64_t np = c->mesh.np;
   double* aval = c->d_val;
