@@ -294,7 +294,7 @@ static void build_sweep(gdsw_ctx* c, LevelDev& L, int nslab, int Kmax, const std
   SP.d_items = c->arena.upload(items, c->stream);
   SP.d_tasks = c->arena.upload(all, c->stream);
   SP.d_ctr = c->arena.alloc<unsigned>(nctr);
-  SP.G = L.fwd.rows_per_tile / 32;
+  SP.rows = L.fwd.rows_per_tile;
 }
 
 static void resize_sweep(LevelDev& L, int ctas_per_sm) {
@@ -418,12 +418,13 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
 
 // Tile-shape autotuner for the level-1 local solves, run at the end of the set-up: whole
 // preconditioner applies (level-1 sweeps with the coarse branch running beside them on the
-// second stream) are timed with CUDA events, best of three after a warm-up, with 32, 64 and
+// second stream) are timed with CUDA events, best of three after a warm-up, with 16, 32, 64 and
 // 128 rows per forward tile, each as one launch per slab step and as the persistent launch;
 // the fastest is kept.  Every candidate computes the same numbers bit for bit -- a row's dot
 // product is one warp's in a fixed order and the persistent launch runs the same tiles -- so
-// the choice changes only the schedule.  Small problems (level-1 sweeps under 64 MB) keep
-// the defaults.
+// the choice changes only the schedule.  16 rows pay where a slab step has few tiles and the FP64
+// pipe of the SM with one tile more than the others bounds it (FP64 apply of an 11x9x13 box, 12
+// parts: 325 -> 237 us).  Small problems (level-1 sweeps under 64 MB) keep the defaults.
 static void apply_precond_impl(gdsw_ctx* c, const double* r, double* z, cudaStream_t s);
 
 static void autotune_level1(gdsw_ctx* c) {
@@ -443,13 +444,13 @@ static void autotune_level1(gdsw_ctx* c) {
     GDSW_CUDA(cudaEventCreate(&e0));
     GDSW_CUDA(cudaEventCreate(&e1));
     float best = 1e30f;
-    int bestG = 1, curG = L.fwd.rows_per_tile / 32;
+    int best_rows = 32, rows = L.fwd.rows_per_tile;
     bool bestP = false;
-    for (int G : {1, 2, 4}) {
-      if (G != curG) {
-        L.fwd.rows_per_tile = 32 * G;
+    for (int cand : {16, 32, 64, 128}) {
+      if (cand != rows) {
+        L.fwd.rows_per_tile = cand;
         build_local_plan(c, c->lh[0].loc, L);
-        curG = G;
+        rows = cand;
       }
       for (bool P : {false, true}) {
         L.persistent = P;
@@ -466,13 +467,13 @@ static void autotune_level1(gdsw_ctx* c) {
         }
         if (t < best) {
           best = t;
-          bestG = G;
+          best_rows = cand;
           bestP = P;
         }
       }
     }
-    if (bestG != curG) {
-      L.fwd.rows_per_tile = 32 * bestG;
+    if (best_rows != rows) {
+      L.fwd.rows_per_tile = best_rows;
       build_local_plan(c, c->lh[0].loc, L);
     }
     L.persistent = bestP;

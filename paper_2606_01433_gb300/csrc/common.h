@@ -301,7 +301,7 @@ struct SweepPlan {
   GemvTask* d_tasks = nullptr;   // forward, backward and reduction tasks of the level
   unsigned* d_ctr = nullptr;     // [0] = claim counter, then 4 counters per slab
   int nitems = 0, nctr = 0, xs_elems = 0, grid = 0, ctas_per_sm = 0, max_per_sm = 0;
-  int G = 1;                     // row groups of 32 per forward tile
+  int rows = 32;                 // rows per forward tile
   size_t smem = 0;
 };
 constexpr unsigned long long kSweepWaitLimitNs = 1000000000ull;  // 1 s per wait
