@@ -51,12 +51,19 @@ struct SlabDevice {
 
 static SlabView upload_slabview(DevArena& A, const SlabSet& S, cudaStream_t s, std::vector<int32_t>* owner_out) {
   std::vector<int32_t> owner(S.nvec), pslab(S.nvec), pidx(S.nvec), slab_base(S.nsub + 1);
-  std::vector<int64_t> fS, fG, fW;
-  std::vector<int32_t> ldS, ldG, ldW, m;
+  std::vector<int64_t> fS, fG, fW, fClo, fChi;
+  std::vector<int32_t> ldS, ldG, ldW, m, lo, hi, back;
   int sb = 0;
   for (int i = 0; i < S.nsub; ++i) {
     slab_base[i] = sb;
-    for (int k = 0; k < S.K[i]; ++k) {
+    const int nb = S.K[i] + S.nmid(i);
+    for (int k = 0; k < nb; ++k) {
+      const int q = k - S.K[i];
+      back.push_back(q < 0 && S.condensed() ? S.back[i][k] : 0);
+      lo.push_back(q >= 0 ? S.lo[i][q] : -1);
+      hi.push_back(q >= 0 ? S.hi[i][q] : -1);
+      fClo.push_back(q >= 0 ? S.fClo[i][q] : -1);
+      fChi.push_back(q >= 0 ? S.fChi[i][q] : -1);
       fS.push_back(S.fS[i][k]); fG.push_back(S.fG[i][k]); fW.push_back(S.fW[i][k]);
       ldS.push_back(S.ldS[i][k]); ldG.push_back(S.ldG[i][k]); ldW.push_back(S.ldW[i][k]);
       m.push_back(S.m[i][k]);
@@ -67,7 +74,7 @@ static SlabView upload_slabview(DevArena& A, const SlabSet& S, cudaStream_t s, s
         pidx[p0 + r] = r;
       }
     }
-    sb += S.K[i];
+    sb += nb;
   }
   slab_base[S.nsub] = sb;
   SlabView v;
@@ -81,6 +88,9 @@ static SlabView upload_slabview(DevArena& A, const SlabSet& S, cudaStream_t s, s
   v.fS = A.upload(fS, s); v.fG = A.upload(fG, s); v.fW = A.upload(fW, s);
   v.ldS = A.upload(ldS, s); v.ldG = A.upload(ldG, s); v.ldW = A.upload(ldW, s);
   v.m = A.upload(m, s);
+  v.nslab = A.upload(std::vector<int32_t>(S.K.begin(), S.K.end()), s);
+  v.lo = A.upload(lo, s); v.hi = A.upload(hi, s); v.back = A.upload(back, s);
+  v.fClo = A.upload(fClo, s); v.fChi = A.upload(fChi, s);
   if (owner_out) *owner_out = owner;
   return v;
 }
@@ -108,6 +118,69 @@ static T* ptr_at(void* base, int64_t off) {
 // symmetric, so the block above the diagonal is B_k^T), compute in place
 //   S_0 = A_00, S_k = A_kk - G_k B_k^T,  G_k = B_k S_{k-1}^{-1},  Sinv_k = S_k^{-1},
 // so that A = L D L^T with L_{k,k-1} = G_k and D = diag(S_k).
+// Condensed sets first eliminate every mid layer q (couplings C_lo, C_hi to the slabs below and above):
+//   M_q^{-1} in place, A_lo -= C_lo M_q^{-1} C_lo^T, B_hi -= C_hi M_q^{-1} C_lo^T,
+//   A_hi -= C_hi M_q^{-1} C_hi^T,
+// which leaves a block-tridiagonal system of the slabs alone.
+template <typename T>
+static void condense_mids(const SlabSet& S, T* fac, double& minpiv, cudaStream_t s) {
+  int nmid = 0;
+  int64_t maxP = 1;
+  for (int i = 0; i < S.nsub; ++i) nmid = std::max(nmid, S.nmid(i));
+  for (int q = 0; q < nmid; ++q) {
+    int64_t n = 0;
+    for (int i = 0; i < S.nsub; ++i)
+      if (q < S.nmid(i)) n += (S.lo[i][q] >= 0 ? int64_t(S.s[i][S.lo[i][q]]) : 0) * S.ldS[i][S.K[i] + q] +
+                              (S.hi[i][q] >= 0 ? int64_t(S.back[i][S.hi[i][q]]) : 0) * S.ldS[i][S.K[i] + q];
+    maxP = std::max(maxP, n);
+  }
+  if (nmid == 0) return;
+  DevArena tmp(s);
+  try {
+    T* P = tmp.alloc<T>(maxP);
+    for (int q = 0; q < nmid; ++q) {
+      std::vector<InvTaskP> inv;
+      std::vector<GemmTaskP> mul, lower, upper;
+      int64_t off = 0;
+      for (int i = 0; i < S.nsub; ++i) {
+        if (q >= S.nmid(i)) continue;
+        const int k = S.K[i] + q, n = S.s[i][k], ld = S.ldS[i][k], lo = S.lo[i][q], hi = S.hi[i][q];
+        T* M = fac + S.fS[i][k];
+        inv.push_back({M, n, ld, 0});
+        T* Plo = P + off;
+        if (lo >= 0) {
+          const int r = S.s[i][lo];
+          const T* C = fac + S.fClo[i][q];
+          off += int64_t(r) * ld;
+          mul.push_back({C, M, Plo, r, n, n, ld, ld, ld, 0, 0, 1.0, 0.0});
+          lower.push_back({Plo, C, fac + S.fS[i][lo], r, r, n, ld, ld, S.ldS[i][lo], 0, 1, -1.0, 1.0});
+        }
+        if (hi >= 0 && S.back[i][hi] > 0) {
+          const int r = S.back[i][hi];
+          const T* C = fac + S.fChi[i][q];
+          T* Phi = P + off;
+          off += int64_t(r) * ld;
+          mul.push_back({C, M, Phi, r, n, n, ld, ld, ld, 0, 0, 1.0, 0.0});
+          upper.push_back({Phi, C, fac + S.fS[i][hi], r, r, n, ld, ld, S.ldS[i][hi], 0, 1, -1.0, 1.0});
+          if (lo >= 0 && S.m[i][hi] > 0)
+            lower.push_back({C, Plo, fac + S.fG[i][hi], r, S.s[i][lo], n, ld, ld, S.ldG[i][hi], 0, 1, -1.0, 1.0});
+        }
+      }
+      std::vector<double> mp;
+      run_inverse<T>(tmp, inv, mp, s);
+      for (double v : mp) minpiv = std::min(minpiv, v);
+      run_gemm<T>(tmp, mul, s);
+      run_gemm<T>(tmp, lower, s);
+      run_gemm<T>(tmp, upper, s);
+    }
+    GDSW_CUDA(cudaStreamSynchronize(s));
+  } catch (...) {
+    tmp.free_all();
+    throw;
+  }
+  tmp.free_all();
+}
+
 template <typename T>
 static void factor_slabs(const SlabSet& S, T* fac, double& minpiv, cudaStream_t s) {
   DevArena tmp(s);
@@ -122,6 +195,7 @@ static void factor_slabs(const SlabSet& S, T* fac, double& minpiv, cudaStream_t 
   T* scrB = tmp.alloc<T>(maxB);
   minpiv = 1e300;
   try {
+    condense_mids<T>(S, fac, minpiv, s);
     // symmetric block LDL^T: G_k = B_k S_{k-1}^{-1}, S_k = A_kk - G_k B_k^T
     for (int k = 0; k < S.Kmax; ++k) {
       if (k >= 1) {
@@ -319,11 +393,49 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
   const int64_t nv = S.nvec;
   const int TT = L.sym_T;
   std::vector<int> sb(S.nsub + 1, 0);  // first flattened slab index of each part
-  for (int i = 0; i < S.nsub; ++i) sb[i + 1] = sb[i] + S.K[i];
+  for (int i = 0; i < S.nsub; ++i) sb[i + 1] = sb[i] + S.K[i] + S.nmid(i);
   int64_t part_off = 2 * nv;          // partial sums live behind the two local vectors
   int xs_elems = 8;                   // shared staging of the persistent sweep
-  L.fwd.launch_task_off = {0};
-  L.fwd.launch_tile_off = {0};
+  // w = S_k^{-1} y (k >= K: M^{-1} of a mid layer) of part i; step < 0: no part of the persistent sweep
+  auto inverse_task = [&](int i, int k, int step, int& mld) {
+    const int q = sb[i] + k;
+    int64_t y = S.voff[i] + S.soff[i][k];
+    const int sk = S.s[i][k];
+    if (L.psym[q]) {
+      const int nt = (sk + TT - 1) / TT;
+      GemvTask t{L.pS[q], y, nv + y, -1, sk, nt * TT, nt, 1.0f, 1, 0, part_off};
+      int id = int(tasks.size());
+      tasks.push_back(t);
+      const int t0 = int(tiles.size());
+      for (int I = 0; I < nt; ++I)
+        for (int J = I; J < nt; ++J) tiles.push_back({id, (I << 16) | J});
+      if (step >= 0) recs.push_back({id, q, step, 1, t0, int(tiles.size())});
+      int rid = int(rtasks.size());
+      rtasks.push_back(t);
+      const int r0t = int(rtiles.size());
+      for (int r0 = 0; r0 < sk; r0 += 256) rtiles.push_back({rid, r0});
+      if (step >= 0) recs.push_back({rid, q, step, 3, r0t, int(rtiles.size())});
+      part_off += int64_t(nt) * nt * TT;
+      mld = std::max(mld, 11 * TT);
+    } else {
+      GemvTask t{L.pS[q], y, nv + y, -1, sk, sk, S.ldS[i][k], 1.0f};
+      const int t0 = int(tiles.size());
+      add_task(tasks, tiles, t, rpt);
+      if (step >= 0 && int(tiles.size()) > t0)
+        recs.push_back({int(tasks.size()) - 1, q, step, 0, t0, int(tiles.size())});
+      mld = std::max(mld, S.ldS[i][k]);
+    }
+  };
+  L.mid_ld = 8;
+  for (int i = 0; i < S.nsub; ++i)
+    for (int q = 0; q < S.nmid(i); ++q) inverse_task(i, S.K[i] + q, -1, L.mid_ld);
+  const int mid_tasks = int(tasks.size()), mid_tiles = int(tiles.size());
+  const int mid_rtasks = int(rtasks.size()), mid_rtiles = int(rtiles.size());
+  L.mid.launch_task_off = {0, mid_tasks};
+  L.mid.launch_tile_off = {0, mid_tiles};
+  L.mid.rows_per_tile = rpt;
+  L.fwd.launch_task_off = {mid_tasks};
+  L.fwd.launch_tile_off = {mid_tiles};
   L.fwd_ld.clear();
   for (int k = 0; k < S.Kmax; ++k) {
     int mld = 8;
@@ -332,29 +444,7 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
       const int q = sb[i] + k;
       int64_t y = S.voff[i] + S.soff[i][k];
       const int sk = S.s[i][k];
-      if (L.psym[q]) {
-        const int nt = (sk + TT - 1) / TT;
-        GemvTask t{L.pS[q], y, nv + y, -1, sk, nt * TT, nt, 1.0f, 1, 0, part_off};
-        int id = int(tasks.size());
-        tasks.push_back(t);
-        const int t0 = int(tiles.size());
-        for (int I = 0; I < nt; ++I)
-          for (int J = I; J < nt; ++J) tiles.push_back({id, (I << 16) | J});
-        recs.push_back({id, q, k, 1, t0, int(tiles.size())});
-        int rid = int(rtasks.size());
-        rtasks.push_back(t);
-        const int r0t = int(rtiles.size());
-        for (int r0 = 0; r0 < sk; r0 += 256) rtiles.push_back({rid, r0});
-        recs.push_back({rid, q, k, 3, r0t, int(rtiles.size())});
-        part_off += int64_t(nt) * nt * TT;
-        mld = std::max(mld, 11 * TT);
-      } else {
-        GemvTask t{L.pS[q], y, nv + y, -1, sk, sk, S.ldS[i][k], 1.0f};
-        const int t0 = int(tiles.size());
-        add_task(tasks, tiles, t, rpt);
-        if (int(tiles.size()) > t0) recs.push_back({int(tasks.size()) - 1, q, k, 0, t0, int(tiles.size())});
-        mld = std::max(mld, S.ldS[i][k]);
-      }
+      inverse_task(i, k, k, mld);
       if (k + 1 < S.K[i] && S.m[i][k + 1] > 0) {
         int64_t y1 = S.voff[i] + S.soff[i][k + 1];
         GemvTask g{L.pG[q + 1], y, y1, y1, S.m[i][k + 1], sk, S.ldG[i][k + 1], -1.0f};
@@ -370,11 +460,17 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
     xs_elems = std::max(xs_elems, mld);
   }
   L.npart = part_off - 2 * nv;
-  L.red.launch_task_off = {0, int(rtasks.size())};
-  L.red.launch_tile_off = {0, int(rtiles.size())};
+  L.red.launch_task_off = {mid_rtasks, int(rtasks.size())};
+  L.red.launch_tile_off = {mid_rtiles, int(rtiles.size())};
+  L.midred.launch_task_off = {0, mid_rtasks};
+  L.midred.launch_tile_off = {0, mid_rtiles};
   L.red_bytes = 0;
   for (const GemvTask& t : rtasks) L.red_bytes += (double(t.ld) * t.ld * TT + t.rows) * vsz;
+  for (int t = 0; t < mid_rtasks; ++t)  // the mid layers' partial sums are reduced twice
+    L.red_bytes += (double(rtasks[t].ld) * rtasks[t].ld * TT + rtasks[t].rows) * vsz;
   finish_plan(c->arena, L.red, rtasks, rtiles, c->stream);
+  L.midred.d_tasks = L.red.d_tasks;
+  L.midred.d_tiles = L.red.d_tiles;
   // backward: x_k = w_k - G_{k+1}^T x_{k+1}[0:m_{k+1}], transposed GEMV over column tiles
   L.bwd.transposed = true;
   L.bwd.launch_task_off = {int(tasks.size())};
@@ -406,12 +502,19 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
     L.fwd_bytes.push_back(plan_bytes(tasks, L.fwd.launch_task_off[k], L.fwd.launch_task_off[k + 1], esz, vsz));
   for (int k = 0; k < L.bwd.nlaunch(); ++k)
     L.bwd_bytes.push_back(plan_bytes(tasks, L.bwd.launch_task_off[k], L.bwd.launch_task_off[k + 1], esz, vsz, true));
+  if (mid_tasks > 0) {  // the mid layers before the first forward and after the last backward launch
+    const double mid = plan_bytes(tasks, 0, mid_tasks, esz, vsz);
+    L.fwd_bytes.insert(L.fwd_bytes.begin(), mid + 4.0 * L.to_slabs.ncol + vsz * L.to_slabs.nval);
+    L.bwd_bytes.push_back(mid + 4.0 * L.to_mids.ncol + vsz * L.to_mids.nval);
+  }
   build_sweep(c, L, sb[S.nsub], S.Kmax, tasks, tiles, rtasks, rtiles, recs, xs_elems);
   resize_sweep(L, L.sweep.ctas_per_sm);
   GemvTask* dt = c->arena.upload(tasks, c->stream);
   GemvTile* dl = c->arena.upload(tiles, c->stream);
   L.fwd.d_tasks = dt;
   L.fwd.d_tiles = dl;
+  L.mid.d_tasks = dt;
+  L.mid.d_tiles = dl;
   L.bwd.d_tasks = dt;
   L.bwd.d_tiles = dl;
 }
@@ -637,7 +740,7 @@ static void store_factors(gdsw_ctx* c, const SlabSet& S, const T* fac, LevelDev&
   std::vector<PackTile> tiles;
   int64_t off = 0;
   for (int i = 0; i < S.nsub; ++i)
-    for (int k = 0; k < S.K[i]; ++k) {
+    for (int k = 0; k < S.K[i] + S.nmid(i); ++k) {
       const int sk = S.s[i][k];
       // FP64 stays dense: on GB300 the FP64 sweep is bound by FP64 FMAs, which packing
       // does not reduce (each stored entry then feeds two products)
@@ -656,7 +759,7 @@ static void store_factors(gdsw_ctx* c, const SlabSet& S, const T* fac, LevelDev&
         off += int64_t(sk) * S.ldS[i][k];
       }
       L.pG.push_back(off);
-      if (k > 0) off += int64_t(S.m[i][k]) * S.ldG[i][k];
+      if (k > 0 && k < S.K[i]) off += int64_t(S.m[i][k]) * S.ldG[i][k];
     }
   L.nfac = off;
   T* packed = tmp.alloc<T>(std::max<int64_t>(off, 1));
@@ -664,11 +767,11 @@ static void store_factors(gdsw_ctx* c, const SlabSet& S, const T* fac, LevelDev&
   pack_tiles<T>(tmp, fac, packed, tiles, TT, s);
   size_t q = 0;
   for (int i = 0; i < S.nsub; ++i)
-    for (int k = 0; k < S.K[i]; ++k, ++q) {
+    for (int k = 0; k < S.K[i] + S.nmid(i); ++k, ++q) {
       if (!L.psym[q])
         GDSW_CUDA(cudaMemcpyAsync(packed + L.pS[q], fac + S.fS[i][k], sizeof(T) * S.s[i][k] * S.ldS[i][k],
                                   cudaMemcpyDeviceToDevice, s));
-      if (k > 0)
+      if (k > 0 && k < S.K[i])
         GDSW_CUDA(cudaMemcpyAsync(packed + L.pG[q], fac + S.fG[i][k], sizeof(T) * S.m[i][k] * S.ldG[i][k],
                                   cudaMemcpyDeviceToDevice, s));
     }
@@ -685,6 +788,63 @@ static void store_factors(gdsw_ctx* c, const SlabSet& S, const T* fac, LevelDev&
 }
 
 // ------------------------------------------------------------------ level 1 numeric set-up
+// The couplings of a condensed set, in the apply's compute precision (T: FP64, or FP32 also beside
+// BF16 factors), for the rows of the slabs and for those of the mid layers.
+template <typename T>
+static void build_couplings(gdsw_ctx* c, const SlabSet& S, const MatView& A, const SlabView& SV, int32_t* map,
+                            int batch, LevelDev& L, DevArena& tmp) {
+  cudaStream_t s = c->stream;
+  int32_t* d_count = tmp.alloc<int32_t>(std::max<int64_t>(S.nvec, 1));
+  auto parts = [&](auto f) {  // parts in batches with a private global-to-local map each
+    for (int i0 = 0; i0 < S.nsub; i0 += batch) {
+      const int64_t p0 = S.voff[i0], p1 = S.voff[std::min(S.nsub, i0 + batch)];
+      set_map(SV, p0, p1, i0, A.n, true, map, s);
+      f(p0, p1, i0);
+      set_map(SV, p0, p1, i0, A.n, false, map, s);
+    }
+  };
+  parts([&](int64_t p0, int64_t p1, int i0) { count_coupling(A, SV, p0, p1, i0, map, d_count, s); });
+  std::vector<int32_t> count(S.nvec);
+  GDSW_CUDA(cudaMemcpyAsync(count.data(), d_count, 4 * S.nvec, cudaMemcpyDeviceToHost, s));
+  GDSW_CUDA(cudaStreamSynchronize(s));
+  const int32_t nu = int32_t(A.nu);
+  for (int dir = 0; dir < 2; ++dir) {
+    Coupling& C = dir == 0 ? L.to_slabs : L.to_mids;
+    std::vector<int32_t> row, nrow, blk_of(S.nvec, -1);
+    std::vector<int64_t> off(1, 0), voff(1, 0);
+    for (int i = 0; i < S.nsub; ++i) {
+      const int64_t split = S.voff[i] + (S.nmid(i) > 0 ? S.soff[i][S.K[i]] : S.voff[i + 1] - S.voff[i]);
+      const int64_t p1 = dir == 0 ? split : S.voff[i + 1];
+      for (int64_t p = dir == 0 ? S.voff[i] : split; p < p1;) {
+        const int nr = S.gdof[p] < nu ? 3 : 1;  // the three velocity dofs of a node follow each other
+        if (count[p] > 0) {
+          for (int r = 0; r < nr; ++r) blk_of[p + r] = int32_t(row.size()) * 4 + r;
+          row.push_back(int32_t(p));
+          nrow.push_back(nr);
+          off.push_back(off.back() + count[p]);
+          voff.push_back(voff.back() + int64_t(nr) * count[p]);
+        }
+        p += nr;
+      }
+    }
+    C.nblk = int(row.size());
+    C.ncol = off.back();
+    C.nval = voff.back();
+    C.row = c->arena.upload(row, s);
+    C.nrow = c->arena.upload(nrow, s);
+    C.off = c->arena.upload(off, s);
+    C.voff = c->arena.upload(voff, s);
+    C.col = c->arena.alloc<int32_t>(std::max<int64_t>(C.ncol, 1));
+    T* val = c->arena.alloc<T>(std::max<int64_t>(C.nval, 1));
+    C.val = val;
+    int32_t* d_blk = tmp.upload(blk_of, s);
+    parts([&](int64_t p0, int64_t p1, int i0) {
+      fill_coupling<T>(A, SV, p0, p1, i0, map, d_blk, C.off, C.voff, C.col, val, s);
+    });
+    GDSW_CUDA(cudaStreamSynchronize(s));
+  }
+}
+
 template <typename T>
 static void level1_locals(gdsw_ctx* c, double& minpiv) {
   const SlabSet& S = c->lh[0].loc;
@@ -692,8 +852,8 @@ static void level1_locals(gdsw_ctx* c, double& minpiv) {
   cudaStream_t s = c->stream;
   MatView A = matview(c);
   DevArena tmp(s);
-  T* fac = tmp.alloc<T>(S.nfac);
-  GDSW_CUDA(cudaMemsetAsync(fac, 0, S.nfac * sizeof(T), s));
+  T* fac = tmp.alloc<T>(S.nset);
+  GDSW_CUDA(cudaMemsetAsync(fac, 0, S.nset * sizeof(T), s));
   std::vector<int32_t> owner;
   SlabView SV = upload_slabview(tmp, S, s, &owner);
   int* err = tmp.alloc<int>(1);
@@ -707,6 +867,7 @@ static void level1_locals(gdsw_ctx* c, double& minpiv) {
     int i1 = std::min(S.nsub, i0 + batch);
     extract_slabs<T>(A, SV, S.voff[i0], S.voff[i1], i0, 1, map, fac, err, s);
   }
+  if (S.condensed()) build_couplings<T>(c, S, A, SV, map, batch, L, tmp);
   int herr = 0;
   GDSW_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
   GDSW_CUDA(cudaStreamSynchronize(s));
@@ -938,6 +1099,36 @@ static void coarse_basis(gdsw_ctx* c, int l, double* A0n, double& minpiv) {
 }
 
 // ------------------------------------------------------------------ apply
+// w = M_q^{-1} y of every mid layer of a condensed set (vec: y, w, partial sums)
+template <typename TM, typename TV>
+static void mid_solve(const LevelDev& L, TV* vec, cudaStream_t s) {
+  launch_gemv<TM, TV>(static_cast<const TM*>(L.fac), vec, vec, vec, L.mid, 0, L.mid_ld, s);
+  launch_sym_reduce<TV>(vec, vec, L.midred, L.sym_T, s);
+}
+
+// Condensed sets, around the sweeps of the slabs: before them w_q = M_q^{-1} r_q and the slabs'
+// r -= C w, after them x_q = M_q^{-1} (r_q - C^T x).
+template <typename TM, typename TV>
+static void condense_apply(const LevelDev& L, TV* vec, bool before, cudaStream_t s) {
+  if (before) {
+    mid_solve<TM, TV>(L, vec, s);
+    launch_coupling<TV>(L.to_slabs, vec, L.nvec, s);
+  } else {
+    launch_coupling<TV>(L.to_mids, vec, L.nvec, s);
+    mid_solve<TM, TV>(L, vec, s);
+  }
+}
+
+void condense_apply(const LevelDev& L, void* vec, bool before, cudaStream_t s) {
+  if (L.mid.launch_tile_off.size() < 2 || L.mid.launch_tile_off[1] == 0) return;
+  if (L.prec == GDSW_FP64)
+    condense_apply<double, double>(L, static_cast<double*>(vec), before, s);
+  else if (L.prec == GDSW_FP32)
+    condense_apply<float, float>(L, static_cast<float*>(vec), before, s);
+  else
+    condense_apply<__nv_bfloat16, float>(L, static_cast<float*>(vec), before, s);
+}
+
 static void local_solve(gdsw_ctx* c, int l, const double* r, double* z, cudaStream_t s) {
   LevelDev& L = c->ld[l];
   const LevelHost& H = c->lh[l];
@@ -972,6 +1163,7 @@ static void local_solve(gdsw_ctx* c, int l, const double* r, double* z, cudaStre
     for (double b : L.fwd_bytes) bytes += b;
     for (double b : L.bwd_bytes) bytes += b;
     ProfScope ps(c, group, bytes, s);
+    condense_apply(L, L.vec, true, s);
     if (L.prec == GDSW_FP64)
       launch_sweep<double, double>(static_cast<const double*>(L.fac), static_cast<double*>(L.vec), L.sweep,
                                    c->d_sweep_flag, L.sym_T, s);
@@ -981,12 +1173,14 @@ static void local_solve(gdsw_ctx* c, int l, const double* r, double* z, cudaStre
     else
       launch_sweep<__nv_bfloat16, float>(static_cast<const __nv_bfloat16*>(L.fac), static_cast<float*>(L.vec),
                                          L.sweep, c->d_sweep_flag, L.sym_T, s);
+    condense_apply(L, L.vec, false, s);
   } else {
   // the chained launches are timed as one unit: events between them would break the chain
   double bytes = L.red_bytes;
   for (double b : L.fwd_bytes) bytes += b;
   for (double b : L.bwd_bytes) bytes += b;
   ProfScope ps(c, group, bytes, s);
+  condense_apply(L, L.vec, true, s);
   for (int k = 0; k < L.fwd.nlaunch(); ++k) sweep(L.fwd, k, L.fwd_ld[k]);
   if (L.red.launch_tile_off.size() == 2 && L.red.launch_tile_off[1] > 0) {
     // w_k = S_k^{-1} y_k of the packed symmetric blocks: sum of the partial products
@@ -996,6 +1190,7 @@ static void local_solve(gdsw_ctx* c, int l, const double* r, double* z, cudaStre
       launch_sym_reduce<float>(static_cast<const float*>(L.vec), static_cast<float*>(L.vec), L.red, L.sym_T, s);
   }
   for (int k = 0; k < L.bwd.nlaunch(); ++k) sweep(L.bwd, k, L.bwd_ld[k]);
+  condense_apply(L, L.vec, false, s);
   }
   {
     ProfScope ps(c, l == 0 ? GDSW_K_SCATTER : GDSW_K_COARSE,
@@ -1163,13 +1358,15 @@ void setup_impl(gdsw_ctx* c, const gdsw_mesh* mesh, const gdsw_viscosity* visc, 
     for (int l = 0; l < nlev; ++l) {
       const LevelHost& H = c->lh[l];
       b += double(H.loc.nfac) * elem_size(opt->precision[l]) + 16.0 * H.loc.nvec + 16.0 * H.loc.nvec;
+      // couplings: at most 50 velocity or 50 velocity and 18 pressure neighbours of a row, 100 entries on average
+      if (H.loc.condensed()) b += 100.0 * H.loc.nvec * (opt->precision[l] == GDSW_FP64 ? 9.4 : 5.4);
       for (int J = 0; J < H.cs.nparts; ++J)  // Phi_I^T blocks
         b += double(H.cs.ioff[J + 1] - H.cs.ioff[J]) * double(H.cs.coff[J + 1] - H.cs.coff[J]) *
              elem_size(l == 0 ? opt->phi_precision : GDSW_FP64);
     }
     b += 8.0 * (2.0 * c->opt.restart + 2.0) * M.n;
     // the factorisation works in a temporary copy of the level-1 factors and interiors
-    if (nlev > 0) b += double(c->lh[0].loc.nfac) * (opt->precision[0] == GDSW_FP64 ? 8 : 4);
+    if (nlev > 0) b += double(c->lh[0].loc.nset) * (opt->precision[0] == GDSW_FP64 ? 8 : 4);
     c->est_device_bytes = int64_t(b);
     c->host_ready = true;
   }

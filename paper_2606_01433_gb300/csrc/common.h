@@ -175,12 +175,27 @@ struct InvTask {
   int32_t id;       // index into the status / scratch arrays
 };
 
+// Factors of at least this many bytes are condensed.  Smaller ones run at the latency of their launches,
+// of which condensing adds four to six.  Local solves, plain -> condensed: channel with obstacles
+// 32^3, 64 parts, FP32 (11.6 GB) 1968 -> 1390 us; die, 64 parts, FP32 (1.9 GB) 423 -> 406 us; 20^3 box, 64
+// parts, FP32 (1.7 GB) 342 -> 334 us; the die in BF16 (1.0 GB) 349 -> 385 us; 14^3, 27 parts, FP64 (0.9 GB)
+// 380 -> 389 us; 8^3, 8 parts, FP32 (54 MB) 55 -> 62 us.
+constexpr double kCondenseBytes = 1.5e9;
+
 // ------------------------------------------------------------------ host symbolic structures
 // A batch of block-tridiagonal local problems: dof lists in slab order, slab sizes, the
 // number of back-coupled dofs (those coupled to the previous slab, ordered first) and the
 // offsets of the LDL^T blocks Sinv_k (s_k x s_k) and G_k (m_k x s_{k-1}); the
 // super-diagonal blocks of the symmetric factorisation are the transposes G_{k+1}^T, so no
 // W_k block is stored (fW = -1).
+//
+// Condensed sets (large level-1 factors with slabs one element thick): the node planes in the middle of
+// an element layer hold only velocities and couple to the planes on either side of their layer, so
+// they are eliminated first, each by its own inverse, and the slabs are the planes between the layers.
+// With planes of h dofs a layer stores h^2 / 2 (M_q^{-1}) + h^2 / 2 (S_k^{-1}, both symmetric) + h^2
+// (G_k) instead of 2 h^2 + 2 h^2, and an apply reads 3.5 h^2 entries (M_q^{-1} and G_k twice) and the
+// sparse couplings instead of 6 h^2.  Only well-conditioned blocks are applied twice: FP32 local
+// solves err by 1e-5 of a vector A x instead of 1e-3.
 struct SlabSet {
   int nsub = 0;
   int Kmax = 0;
@@ -193,6 +208,14 @@ struct SlabSet {
   int64_t nvec = 0, nfac = 0;
   std::vector<int32_t> gdof;                 // local position -> global dof of the level
   int64_t max_local = 0;
+  // Mid layers (condensed sets only): block q of part i is entry K[i] + q of s, soff, fS and ldS.
+  // lo, hi: the slabs below and above it (-1: none); back: dofs of each slab coupled downwards (they
+  // come first); fClo, fChi: its dense couplings, s_lo x ldS and back_hi x ldS, behind the factors
+  std::vector<std::vector<int>> lo, hi, back;
+  std::vector<std::vector<int64_t>> fClo, fChi;
+  int64_t nset = 0;                          // entries of the factorisation's work buffer
+  int nmid(int i) const { return lo.empty() ? 0 : int(lo[i].size()); }
+  bool condensed() const { return !lo.empty(); }
   void layout();                             // fills voff/soff/f*/ld*/nvec/nfac from s, m, K
 };
 
@@ -306,6 +329,17 @@ struct SweepPlan {
 };
 constexpr unsigned long long kSweepWaitLimitNs = 1000000000ull;  // 1 s per wait
 
+// Couplings between the mid layers and the slabs of a condensed set, row by row: block b holds
+// nrow[b] (3 velocity, 1 pressure) consecutive rows from position row[b] with common columns
+// col[off[b]], ..., and each row's values one after the other from val[voff[b]].
+struct Coupling {
+  int nblk = 0;
+  int64_t ncol = 0, nval = 0;
+  int32_t *row = nullptr, *nrow = nullptr, *col = nullptr;
+  int64_t *off = nullptr, *voff = nullptr;  // nblk + 1
+  void* val = nullptr;                      // FP64, or FP32 with FP32 and BF16 factors
+};
+
 struct LevelDev {
   int n = 0, N = 0, prec = GDSW_FP64;
   // local problems
@@ -355,6 +389,9 @@ struct LevelDev {
   int sym_T = 128;
   int64_t npart = 0;            // partial-sum entries behind the 2 nvec local vectors
   GemvPlan red;                 // reduction of the symmetric partial sums (one launch)
+  GemvPlan mid, midred;         // condensed sets: M_q^{-1} of every mid layer, and its reduction
+  int mid_ld = 8;
+  Coupling to_slabs, to_mids;   // condensed sets: rows of the slabs, rows of the mid layers
   double red_bytes = 0;
   double minpiv = 0;            // smallest pivot magnitude met by the local factorisation
   double local_bytes = 0;       // algorithmic bytes of one local-solve sweep pair

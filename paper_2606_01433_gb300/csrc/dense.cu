@@ -420,6 +420,53 @@ void launch_sym_reduce(const TV* vec, TV* y, const GemvPlan& P, int T, cudaStrea
 template void launch_sym_reduce<double>(const double*, double*, const GemvPlan&, int, cudaStream_t);
 template void launch_sym_reduce<float>(const float*, float*, const GemvPlan&, int, cudaStream_t);
 
+// ------------------------------------------------------------------ couplings of a condensed set
+// y[rows] -= C w for the couplings between mid layers and slabs (y, w: the two local vectors): eight
+// lanes per block of rows, whose rows share their columns (5.3 bytes an entry instead of 8).  A
+// block has about 110 columns: whole warps spent as long on the butterflies as on the products in
+// FP64, and eight lanes still read whole 32-byte sectors in FP32.
+template <typename TV>
+__global__ void __launch_bounds__(256) k_coupling(int nblk, const int32_t* __restrict__ row,
+                                                  const int32_t* __restrict__ nrow, const int64_t* __restrict__ off,
+                                                  const int64_t* __restrict__ voff, const int32_t* __restrict__ col,
+                                                  const TV* __restrict__ val, TV* y, const TV* w) {
+  const int64_t b = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) / 8;
+  const int lane = threadIdx.x & 7;
+  dep_release();
+  const bool in = b < nblk;
+  const int64_t o = in ? off[b] : 0;
+  const int n = in ? int(off[b + 1] - o) : 0, nr = in ? nrow[b] : 0, r0 = in ? row[b] : 0;
+  const TV* v = val + (in ? voff[b] : 0);
+  dep_wait();
+  TV acc[3] = {TV(0), TV(0), TV(0)};
+  if (nr == 3) {
+#pragma unroll 4
+    for (int j = lane; j < n; j += 8) {
+      const TV x = __ldcg(w + col[o + j]);
+#pragma unroll
+      for (int r = 0; r < 3; ++r) acc[r] = fma(v[r * n + j], x, acc[r]);
+    }
+  } else {
+#pragma unroll 4
+    for (int j = lane; j < n; j += 8) acc[0] = fma(v[j], __ldcg(w + col[o + j]), acc[0]);
+  }
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], d);
+  if (lane < nr) y[r0 + lane] -= lane == 0 ? acc[0] : (lane == 1 ? acc[1] : acc[2]);
+}
+
+template <typename TV>
+void launch_coupling(const Coupling& C, TV* vec, int64_t nvec, cudaStream_t s) {
+  if (C.nblk == 0) return;
+  launch_chained(k_coupling<TV>, dim3(unsigned((int64_t(C.nblk) * 8 + 255) / 256)), dim3(256), 0, s, C.nblk, C.row,
+                 C.nrow, C.off, C.voff, C.col, static_cast<const TV*>(C.val), vec, vec + nvec);
+  check_launch("k_coupling");
+}
+template void launch_coupling<double>(const Coupling&, double*, int64_t, cudaStream_t);
+template void launch_coupling<float>(const Coupling&, float*, int64_t, cudaStream_t);
+
 // ------------------------------------------------------------------ persistent level sweep
 // One launch runs every tile of a level's local solves -- forward row tiles and packed
 // symmetric tiles, the partial-sum reductions, the transposed backward tiles -- from a work

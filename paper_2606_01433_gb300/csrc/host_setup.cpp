@@ -520,29 +520,41 @@ void SlabSet::layout() {
   for (int i = 0; i < nsub; ++i) {
     Kmax = std::max(Kmax, K[i]);
     int64_t off = 0;
-    for (int k = 0; k < K[i]; ++k) {
+    const int nb = K[i] + nmid(i);
+    for (int k = 0; k < nb; ++k) {
       soff[i].push_back(off);
       off += s[i][k];
     }
     voff[i + 1] = voff[i] + off;
     max_local = std::max(max_local, off);
-    for (int k = 0; k < K[i]; ++k) {
+    for (int k = 0; k < nb; ++k) {
       int sk = s[i][k];
       int ld = int(pad8(sk));
       ldS[i].push_back(ld);
       fS[i].push_back(nfac);
       nfac += int64_t(sk) * ld;
       // G_k: m_k x s_{k-1}
-      int ldg = k > 0 ? int(pad8(s[i][k - 1])) : 8;
+      int ldg = k > 0 && k < K[i] ? int(pad8(s[i][k - 1])) : 8;
       ldG[i].push_back(ldg);
       fG[i].push_back(nfac);
-      if (k > 0) nfac += int64_t(m[i][k]) * ldg;
+      if (k > 0 && k < K[i]) nfac += int64_t(m[i][k]) * ldg;
       // W_k = S_k^{-1} C_k is not stored: the operator is symmetric, so W_k = G_{k+1}^T
       ldW[i].push_back(8);
       fW[i].push_back(-1);
     }
   }
   nvec = voff[nsub];
+  nset = nfac;
+  fClo.assign(nsub, {});
+  fChi.assign(nsub, {});
+  for (int i = 0; i < nsub; ++i)
+    for (int q = 0; q < nmid(i); ++q) {
+      const int64_t ld = ldS[i][K[i] + q];
+      fClo[i].push_back(nset);
+      if (lo[i][q] >= 0) nset += s[i][lo[i][q]] * ld;
+      fChi[i].push_back(nset);
+      if (hi[i][q] >= 0) nset += back[i][hi[i][q]] * ld;
+    }
 }
 
 // P1-disc pressure dofs that an element adds to a dof set (they belong to no node).  high:
@@ -677,6 +689,112 @@ static void slab_order(const MeshHost& M, std::vector<int64_t> nodes, int t, Sla
   S.K.push_back(int(s2.size()));
   S.s.push_back(s2);
   S.m.push_back(m2);
+}
+
+// Order the free dofs of a node set for the condensed factorisation (one part per call): slabs are the
+// node planes at even distance across the longest axis, the planes between them -- velocity nodes
+// in the middle of an element layer, coupled to the two slabs beside them only -- are mid blocks
+// behind the slabs.  Element pressure dofs join the plane after their element (see ElemDofs), else
+// the one before it.
+static void condensed_order(const MeshHost& M, std::vector<int64_t> nodes, SlabSet& S,
+                            const std::vector<ElemDofs>* edofs) {
+  std::sort(nodes.begin(), nodes.end());
+  S.K.push_back(0);
+  S.s.push_back({});
+  S.m.push_back({});
+  S.lo.push_back({});
+  S.hi.push_back({});
+  S.back.push_back({});
+  if (nodes.empty()) return;
+  int lo[3] = {1 << 30, 1 << 30, 1 << 30}, hi[3] = {-1, -1, -1};
+  for (int64_t v : nodes) {
+    int c[3];
+    M.coords(v, c[0], c[1], c[2]);
+    for (int d = 0; d < 3; ++d) {
+      lo[d] = std::min(lo[d], c[d]);
+      hi[d] = std::max(hi[d], c[d]);
+    }
+  }
+  int ax = 0;
+  for (int d = 1; d < 3; ++d)
+    if (hi[d] - lo[d] > hi[ax] - lo[ax]) ax = d;
+  const int c0 = lo[ax] - (lo[ax] % 2), nplane = hi[ax] - c0 + 2;
+  std::vector<uint8_t> box(int64_t(hi[0] - lo[0] + 1) * (hi[1] - lo[1] + 1) * (hi[2] - lo[2] + 1), 0);
+  auto member = [&](int i, int j, int k) -> uint8_t* {
+    if (i < lo[0] || i > hi[0] || j < lo[1] || j > hi[1] || k < lo[2] || k > hi[2]) return nullptr;
+    return &box[(i - lo[0]) + int64_t(hi[0] - lo[0] + 1) * ((j - lo[1]) + int64_t(hi[1] - lo[1] + 1) * (k - lo[2]))];
+  };
+  for (int64_t v : nodes) {
+    int c[3];
+    M.coords(v, c[0], c[1], c[2]);
+    *member(c[0], c[1], c[2]) = 1;
+  }
+  // per plane: dofs coupled to a lower plane, the others
+  std::vector<std::vector<int32_t>> A(nplane), B(nplane);
+  std::vector<uint8_t> has_node(nplane, 0);
+  for (int64_t v : nodes) {
+    int c[3];
+    M.coords(v, c[0], c[1], c[2]);
+    const int plane = c[ax] - c0;
+    has_node[plane] = 1;
+    bool back = false;
+    if (plane % 2 == 0)
+      for (int dk = -2; dk <= 2 && !back; ++dk)
+        for (int dj = -2; dj <= 2 && !back; ++dj)
+          for (int di = -2; di <= 2 && !back; ++di) {
+            const int d[3] = {di, dj, dk};
+            if (d[ax] >= 0) continue;
+            const uint8_t* w = member(c[0] + di, c[1] + dj, c[2] + dk);
+            if (!w || !*w) continue;
+            back = M.shares_element(v, (c[0] + di) + int64_t(M.NX) * ((c[1] + dj) + int64_t(M.NY) * (c[2] + dk)));
+          }
+    auto& dst = back ? A[plane] : B[plane];
+    if (M.vidx[v] >= 0)
+      for (int q = 0; q < 3; ++q) dst.push_back(int32_t(3 * M.vidx[v] + q));
+    if (M.pidx[v] >= 0) dst.push_back(int32_t(M.nu + M.pidx[v]));
+  }
+  if (edofs)
+    for (const ElemDofs& x : *edofs) {
+      const int ec[3] = {int(x.e % M.nx), int((x.e / M.nx) % M.ny), int(x.e / (int64_t(M.nx) * M.ny))};
+      const int centre = 2 * ec[ax] + 1 - c0;
+      int plane = -1;
+      for (int p : {centre + 1, centre - 1, centre})
+        if (plane < 0 && p >= 0 && p < nplane && has_node[p]) plane = p;
+      GDSW_CHECK(plane >= 0, GDSW_ERR_INVALID_ARG, "element pressure dofs without their element's nodes");
+      bool back = false;
+      if (plane % 2 == 0)
+        for (int z = 0; z < 3; ++z)
+          for (int y = 0; y < 3; ++y)
+            for (int w = 0; w < 3; ++w) {
+              const int c[3] = {2 * ec[0] + w, 2 * ec[1] + y, 2 * ec[2] + z};
+              const uint8_t* q = member(c[0], c[1], c[2]);
+              back |= q && *q && c[ax] - c0 < plane;
+            }
+      auto& dst = back ? A[plane] : B[plane];
+      for (int c = 0; c < x.n; ++c) dst.push_back(x.d[c]);
+    }
+  std::vector<int> slab(nplane + 1, -1);  // plane -> slab (planes without dofs are dropped)
+  for (int p = 0; p < nplane; p += 2) {
+    std::sort(A[p].begin(), A[p].end());
+    std::sort(B[p].begin(), B[p].end());
+    if (A[p].empty() && B[p].empty()) continue;
+    slab[p] = S.K[0]++;
+    S.s[0].push_back(int(A[p].size() + B[p].size()));
+    S.back[0].push_back(int(A[p].size()));
+    // coupled to the previous slab (directly and through the mid layer) only if that is two planes below
+    S.m[0].push_back(p >= 2 && slab[p - 2] >= 0 ? int(A[p].size()) : 0);
+    S.gdof.insert(S.gdof.end(), A[p].begin(), A[p].end());
+    S.gdof.insert(S.gdof.end(), B[p].begin(), B[p].end());
+  }
+  for (int p = 1; p < nplane; p += 2) {
+    std::sort(B[p].begin(), B[p].end());
+    if (B[p].empty()) continue;
+    S.s[0].push_back(int(B[p].size()));
+    S.m[0].push_back(0);
+    S.lo[0].push_back(slab[p - 1]);
+    S.hi[0].push_back(p + 1 < nplane ? slab[p + 1] : -1);
+    S.gdof.insert(S.gdof.end(), B[p].begin(), B[p].end());
+  }
 }
 
 // One dense block holding sorted dofs (coarse levels).
@@ -903,25 +1021,36 @@ void build_level1(gdsw_ctx* ctx, const gdsw_partition* part, int overlap, int sl
           }
   });
   {
-    std::vector<SlabSet> parts(N);
-    parallel_tasks(N, [&](int64_t i) {
-      std::vector<ElemDofs> ed;
-      for (int32_t f : oelems[i]) {
-        ElemDofs x{M.fluid[f], 4, {}, true};
-        for (int k = 0; k < 4; ++k) x.d[k] = int32_t(M.nu + 4 * int64_t(f) + k);
-        ed.push_back(x);
-      }
-      slab_order(M, onodes[i], slab_elems, parts[i], M.pdisc ? &ed : nullptr);
-    });
     SlabSet& S = L.loc;
-    S = SlabSet();
-    for (int i = 0; i < N; ++i) {
-      S.K.push_back(parts[i].K[0]);
-      S.s.push_back(parts[i].s[0]);
-      S.m.push_back(parts[i].m[0]);
-      S.gdof.insert(S.gdof.end(), parts[i].gdof.begin(), parts[i].gdof.end());
+    for (bool condensed : {false, true}) {
+      if (condensed && (slab_elems != 1 || double(S.nfac) * elem_size(ctx->opt.precision[0]) < kCondenseBytes)) break;
+      std::vector<SlabSet> parts(N);
+      parallel_tasks(N, [&](int64_t i) {
+        std::vector<ElemDofs> ed;
+        for (int32_t f : oelems[i]) {
+          ElemDofs x{M.fluid[f], 4, {}, true};
+          for (int k = 0; k < 4; ++k) x.d[k] = int32_t(M.nu + 4 * int64_t(f) + k);
+          ed.push_back(x);
+        }
+        if (condensed)
+          condensed_order(M, onodes[i], parts[i], M.pdisc ? &ed : nullptr);
+        else
+          slab_order(M, onodes[i], slab_elems, parts[i], M.pdisc ? &ed : nullptr);
+      });
+      S = SlabSet();
+      for (int i = 0; i < N; ++i) {
+        S.K.push_back(parts[i].K[0]);
+        S.s.push_back(parts[i].s[0]);
+        S.m.push_back(parts[i].m[0]);
+        if (condensed) {
+          S.lo.push_back(parts[i].lo[0]);
+          S.hi.push_back(parts[i].hi[0]);
+          S.back.push_back(parts[i].back[0]);
+        }
+        S.gdof.insert(S.gdof.end(), parts[i].gdof.begin(), parts[i].gdof.end());
+      }
+      S.layout();
     }
-    S.layout();
   }
   scatter_lists(L, ctx->opt.weighting);
 

@@ -43,6 +43,8 @@ template <typename TM, typename TV>
 void launch_sweep(const TM* M, TV* vec, const SweepPlan& P, unsigned* flag, int T, cudaStream_t s);
 template <typename TV>
 void launch_sym_reduce(const TV* vec, TV* y, const GemvPlan& P, int T, cudaStream_t s);
+template <typename TV>
+void launch_coupling(const Coupling& C, TV* vec, int64_t nvec, cudaStream_t s);
 struct PackTile {
   int64_t src, dst;
   int32_t ld, rows, cols, pad;  // rows/cols valid inside the tile

@@ -12,6 +12,7 @@
 
 #include "common.h"
 #include "kernels.h"
+#include "setup.h"
 
 namespace gdsw {
 
@@ -52,15 +53,18 @@ static void local_solve_into(gdsw_ctx* c, int l, const double* r, double* z, voi
   if (L.prec == GDSW_FP64) {
     double* v = static_cast<double*>(vec);
     launch_gather<double>(r, L.gdof, v, nv, s);
+    condense_apply(L, vec, true, s);
     for (int k = 0; k < L.fwd.nlaunch(); ++k)
       launch_gemv<double, double>(static_cast<const double*>(L.fac), v, v, v, L.fwd, k, L.fwd_ld[k], s);
     if (L.red.launch_tile_off.size() == 2) launch_sym_reduce<double>(v, v, L.red, L.sym_T, s);
     for (int k = 0; k < L.bwd.nlaunch(); ++k)
       launch_gemv<double, double>(static_cast<const double*>(L.fac), v, v, v, L.bwd, k, L.bwd_ld[k], s);
+    condense_apply(L, vec, false, s);
     launch_scatter<double>(v + nv, L.sc_ptr, L.sc_pos, L.sc_w, z, L.n, 0, s);
   } else {
     float* v = static_cast<float*>(vec);
     launch_gather<float>(r, L.gdof, v, nv, s);
+    condense_apply(L, vec, true, s);
     for (int k = 0; k < L.fwd.nlaunch(); ++k) {
       if (L.prec == GDSW_FP32)
         launch_gemv<float, float>(static_cast<const float*>(L.fac), v, v, v, L.fwd, k, L.fwd_ld[k], s);
@@ -74,6 +78,7 @@ static void local_solve_into(gdsw_ctx* c, int l, const double* r, double* z, voi
       else
         launch_gemv<__nv_bfloat16, float>(static_cast<const __nv_bfloat16*>(L.fac), v, v, v, L.bwd, k, L.bwd_ld[k], s);
     }
+    condense_apply(L, vec, false, s);
     launch_scatter<float>(v + nv, L.sc_ptr, L.sc_pos, L.sc_w, z, L.n, 0, s);
   }
 }

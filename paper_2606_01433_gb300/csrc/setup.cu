@@ -71,8 +71,15 @@ __global__ void k_extract(MatView A, SlabView S, int64_t p0, int64_t p1, int i0,
     int32_t q = map[slot + col];
     if (q < 0 || S.owner[q] != i) return;
     const int kc = S.pslab[q], c = S.pidx[q];
+    const int K = S.nslab[i];
     if (kc == kr) {
       fac[S.fS[sb + kr] + int64_t(r) * S.ldS[sb + kr] + c] = T(v);
+    } else if (kr >= K || kc >= K) {  // a mid layer: its couplings are kept with the slab's rows
+      const int mid = sb + (kc >= K ? kc : kr), k = kc >= K ? kr : kc;
+      if (k >= K || (k != S.lo[mid] && (k != S.hi[mid] || (kc >= K ? r : c) >= S.back[sb + k])))
+        atomicExch(err, 1);
+      else if (kc >= K)
+        fac[(k == S.lo[mid] ? S.fClo[mid] : S.fChi[mid]) + int64_t(r) * S.ldS[mid] + c] = T(v);
     } else if (kc == kr - 1 && r < S.m[sb + kr]) {
       fac[S.fG[sb + kr] + int64_t(r) * S.ldG[sb + kr] + c] = T(v);
     } else if (kc == kr + 1 && c < S.m[sb + kc]) {
@@ -83,6 +90,74 @@ __global__ void k_extract(MatView A, SlabView S, int64_t p0, int64_t p1, int i0,
     }
   });
 }
+
+// Couplings of a condensed set for the apply: one thread per row, columns of the other class (mid
+// layer or slab) in the operator's order
+template <typename F>
+__device__ __forceinline__ void coupling_visit(const MatView& A, const SlabView& S, int64_t p, int i0,
+                                               const int32_t* map, F f) {
+  const int i = S.owner[p];
+  const int64_t slot = int64_t(i - i0) * A.n;
+  const bool mid = S.pslab[p] >= S.nslab[i];
+  row_visit(A, S.gdof[p], [&](int64_t col, double v) {
+    const int32_t q = map[slot + col];
+    if (q >= 0 && S.owner[q] == i && (S.pslab[q] >= S.nslab[i]) != mid) f(q, v);
+  });
+}
+
+__global__ void k_coupling_count(MatView A, SlabView S, int64_t p0, int64_t p1, int i0, const int32_t* __restrict__ map,
+                                 int32_t* __restrict__ count) {
+  const int64_t p = p0 + blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (p >= p1) return;
+  int n = 0;
+  coupling_visit(A, S, p, i0, map, [&](int32_t, double) { ++n; });
+  count[p] = n;
+}
+
+template <typename T>
+__global__ void k_coupling_fill(MatView A, SlabView S, int64_t p0, int64_t p1, int i0, const int32_t* __restrict__ map,
+                                const int32_t* __restrict__ blk_of, const int64_t* __restrict__ off,
+                                const int64_t* __restrict__ voff, int32_t* __restrict__ col, T* __restrict__ val) {
+  const int64_t p = p0 + blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (p >= p1) return;
+  const int32_t w = blk_of[p];  // 4 block + row inside it
+  if (w < 0) return;
+  const int64_t o = off[w >> 2], nc = off[(w >> 2) + 1] - o;
+  T* v0 = val + voff[w >> 2] + (w & 3) * nc;
+  int n = 0;
+  coupling_visit(A, S, p, i0, map, [&](int32_t q, double v) {
+    if ((w & 3) == 0) col[o + n] = q;
+    v0[n++] = T(v);
+  });
+}
+
+void set_map(const SlabView& S, int64_t p0, int64_t p1, int i0, int64_t n, bool set, int32_t* map, cudaStream_t s) {
+  if (p1 <= p0) return;
+  const int blocks = int((p1 - p0 + 127) / 128);
+  if (set)
+    k_map_set<<<blocks, 128, 0, s>>>(S.gdof, S.owner, p0, p1, i0, 1, n, map);
+  else
+    k_map_reset<<<blocks, 128, 0, s>>>(S.gdof, S.owner, p0, p1, i0, 1, n, map);
+  check_launch("set_map");
+}
+void count_coupling(const MatView& A, const SlabView& S, int64_t p0, int64_t p1, int i0, const int32_t* map,
+                    int32_t* count, cudaStream_t s) {
+  if (p1 <= p0) return;
+  k_coupling_count<<<unsigned((p1 - p0 + 127) / 128), 128, 0, s>>>(A, S, p0, p1, i0, map, count);
+  check_launch("k_coupling_count");
+}
+template <typename T>
+void fill_coupling(const MatView& A, const SlabView& S, int64_t p0, int64_t p1, int i0, const int32_t* map,
+                   const int32_t* blk_of, const int64_t* off, const int64_t* voff, int32_t* col, T* val,
+                   cudaStream_t s) {
+  if (p1 <= p0) return;
+  k_coupling_fill<T><<<unsigned((p1 - p0 + 127) / 128), 128, 0, s>>>(A, S, p0, p1, i0, map, blk_of, off, voff, col, val);
+  check_launch("k_coupling_fill");
+}
+template void fill_coupling<double>(const MatView&, const SlabView&, int64_t, int64_t, int, const int32_t*,
+                                    const int32_t*, const int64_t*, const int64_t*, int32_t*, double*, cudaStream_t);
+template void fill_coupling<float>(const MatView&, const SlabView&, int64_t, int64_t, int, const int32_t*,
+                                   const int32_t*, const int64_t*, const int64_t*, int32_t*, float*, cudaStream_t);
 
 template <typename T>
 void extract_slabs(const MatView& A, const SlabView& S, int64_t p0, int64_t p1, int i0, int separate,

@@ -23,7 +23,20 @@ struct SlabView {
   const int32_t* slab_base;  // part -> index of its first slab in the per-slab arrays
   const int64_t *fS, *fG, *fW;
   const int32_t *ldS, *ldG, *ldW, *m;
+  // condensed sets: slabs per part; per block slab below, slab above, rows
+  // coupled downwards and the offsets of the couplings
+  const int32_t *nslab, *lo, *hi, *back;
+  const int64_t *fClo, *fChi;
 };
+
+// rows of the couplings between slabs and mid layers (blk: first row of a block), columns and values
+template <typename T>
+void fill_coupling(const MatView& A, const SlabView& S, int64_t p0, int64_t p1, int i0, const int32_t* map,
+                   const int32_t* blk_of, const int64_t* off, const int64_t* voff, int32_t* col, T* val,
+                   cudaStream_t s);
+void count_coupling(const MatView& A, const SlabView& S, int64_t p0, int64_t p1, int i0, const int32_t* map,
+                    int32_t* count, cudaStream_t s);
+void set_map(const SlabView& S, int64_t p0, int64_t p1, int i0, int64_t n, bool set, int32_t* map, cudaStream_t s);
 
 template <typename T>
 void extract_slabs(const MatView& A, const SlabView& S, int64_t p0, int64_t p1, int i0, int separate,
@@ -50,6 +63,8 @@ void launch_tneg(const MatView& A, const SlabView& S, const int32_t* gamma_ptr, 
 void launch_yint(const MatView& A, const SlabView& S, const int32_t* ilocal, const int64_t* coff, const int64_t* toff,
                  const int32_t* ldt, const double* X, const double* Tn, double* Y, cudaStream_t s);
 
+// mid layers of a condensed set before (true) or after the sweeps over its slabs
+void condense_apply(const LevelDev& L, void* vec, bool before, cudaStream_t s);
 // whole set-up: host symbolic phase unless already done, then (unless host_only) the device phase
 void setup_impl(gdsw_ctx* c, const gdsw_mesh* mesh, const gdsw_viscosity* visc, const gdsw_partition* part,
                 const gdsw_levels* lv, const gdsw_options* opt);
