@@ -51,22 +51,24 @@ struct SlabDevice {
 
 static SlabView upload_slabview(DevArena& A, const SlabSet& S, cudaStream_t s, std::vector<int32_t>* owner_out) {
   std::vector<int32_t> owner(S.nvec), pslab(S.nvec), pidx(S.nvec), slab_base(S.nsub + 1);
-  std::vector<int64_t> fS, fG, fW, fClo, fChi;
-  std::vector<int32_t> ldS, ldG, ldW, m, lo, hi, back;
+  std::vector<int64_t> fS, fG, fClo, fChi;
+  std::vector<int32_t> ldS, ldG, m, next, lo, hi, nlo, nhi;
   int sb = 0;
   for (int i = 0; i < S.nsub; ++i) {
     slab_base[i] = sb;
     const int nb = S.K[i] + S.nmid(i);
     for (int k = 0; k < nb; ++k) {
       const int q = k - S.K[i];
-      back.push_back(q < 0 && S.condensed() ? S.back[i][k] : 0);
       lo.push_back(q >= 0 ? S.lo[i][q] : -1);
       hi.push_back(q >= 0 ? S.hi[i][q] : -1);
+      nlo.push_back(q >= 0 ? S.rows_lo(i, q) : 0);
+      nhi.push_back(q >= 0 ? S.rows_hi(i, q) : 0);
       fClo.push_back(q >= 0 ? S.fClo[i][q] : -1);
       fChi.push_back(q >= 0 ? S.fChi[i][q] : -1);
-      fS.push_back(S.fS[i][k]); fG.push_back(S.fG[i][k]); fW.push_back(S.fW[i][k]);
-      ldS.push_back(S.ldS[i][k]); ldG.push_back(S.ldG[i][k]); ldW.push_back(S.ldW[i][k]);
-      m.push_back(S.m[i][k]);
+      fS.push_back(S.fS[i][k]); fG.push_back(S.fG[i][k]);
+      ldS.push_back(S.ldS[i][k]); ldG.push_back(S.ldG[i][k]);
+      m.push_back(q < 0 ? S.m[i][k] : 0);
+      next.push_back(q < 0 ? S.next[i][k] : -1);
       int64_t p0 = S.voff[i] + S.soff[i][k];
       for (int r = 0; r < S.s[i][k]; ++r) {
         owner[p0 + r] = i;
@@ -85,11 +87,12 @@ static SlabView upload_slabview(DevArena& A, const SlabSet& S, cudaStream_t s, s
   v.pidx = A.upload(pidx, s);
   v.voff = A.upload(S.voff, s);
   v.slab_base = A.upload(slab_base, s);
-  v.fS = A.upload(fS, s); v.fG = A.upload(fG, s); v.fW = A.upload(fW, s);
-  v.ldS = A.upload(ldS, s); v.ldG = A.upload(ldG, s); v.ldW = A.upload(ldW, s);
-  v.m = A.upload(m, s);
+  v.fS = A.upload(fS, s); v.fG = A.upload(fG, s);
+  v.ldS = A.upload(ldS, s); v.ldG = A.upload(ldG, s);
+  v.m = A.upload(m, s); v.next = A.upload(next, s);
   v.nslab = A.upload(std::vector<int32_t>(S.K.begin(), S.K.end()), s);
-  v.lo = A.upload(lo, s); v.hi = A.upload(hi, s); v.back = A.upload(back, s);
+  v.lo = A.upload(lo, s); v.hi = A.upload(hi, s);
+  v.nlo = A.upload(nlo, s); v.nhi = A.upload(nhi, s);
   v.fClo = A.upload(fClo, s); v.fChi = A.upload(fChi, s);
   if (owner_out) *owner_out = owner;
   return v;
@@ -119,8 +122,8 @@ static T* ptr_at(void* base, int64_t off) {
 //   S_0 = A_00, S_k = A_kk - G_k B_k^T,  G_k = B_k S_{k-1}^{-1},  Sinv_k = S_k^{-1},
 // so that A = L D L^T with L_{k,k-1} = G_k and D = diag(S_k).
 // Condensed sets first eliminate every mid layer q (couplings C_lo, C_hi to the slabs below and above):
-//   M_q^{-1} in place, A_lo -= C_lo M_q^{-1} C_lo^T, B_hi -= C_hi M_q^{-1} C_lo^T,
-//   A_hi -= C_hi M_q^{-1} C_hi^T,
+//   M_q^{-1} in place, A_lo -= C_lo M_q^{-1} C_lo^T, A_hi -= C_hi M_q^{-1} C_hi^T, and the update
+//   between the two slabs -= C_hi M_q^{-1} C_lo^T (or its transpose),
 // which leaves a block-tridiagonal system of the slabs alone.
 template <typename T>
 static void condense_mids(const SlabSet& S, T* fac, double& minpiv, cudaStream_t s) {
@@ -130,8 +133,7 @@ static void condense_mids(const SlabSet& S, T* fac, double& minpiv, cudaStream_t
   for (int q = 0; q < nmid; ++q) {
     int64_t n = 0;
     for (int i = 0; i < S.nsub; ++i)
-      if (q < S.nmid(i)) n += (S.lo[i][q] >= 0 ? int64_t(S.s[i][S.lo[i][q]]) : 0) * S.ldS[i][S.K[i] + q] +
-                              (S.hi[i][q] >= 0 ? int64_t(S.back[i][S.hi[i][q]]) : 0) * S.ldS[i][S.K[i] + q];
+      if (q < S.nmid(i)) n += int64_t(S.rows_lo(i, q) + S.rows_hi(i, q)) * S.ldS[i][S.K[i] + q];
     maxP = std::max(maxP, n);
   }
   if (nmid == 0) return;
@@ -145,26 +147,24 @@ static void condense_mids(const SlabSet& S, T* fac, double& minpiv, cudaStream_t
       for (int i = 0; i < S.nsub; ++i) {
         if (q >= S.nmid(i)) continue;
         const int k = S.K[i] + q, n = S.s[i][k], ld = S.ldS[i][k], lo = S.lo[i][q], hi = S.hi[i][q];
+        const int rlo = S.rows_lo(i, q), rhi = S.rows_hi(i, q);
         T* M = fac + S.fS[i][k];
+        const T *Clo = fac + S.fClo[i][q], *Chi = fac + S.fChi[i][q];
+        T *Plo = P + off, *Phi = Plo + int64_t(rlo) * ld;
+        off += int64_t(rlo + rhi) * ld;
         inv.push_back({M, n, ld, 0});
-        T* Plo = P + off;
-        if (lo >= 0) {
-          const int r = S.s[i][lo];
-          const T* C = fac + S.fClo[i][q];
-          off += int64_t(r) * ld;
-          mul.push_back({C, M, Plo, r, n, n, ld, ld, ld, 0, 0, 1.0, 0.0});
-          lower.push_back({Plo, C, fac + S.fS[i][lo], r, r, n, ld, ld, S.ldS[i][lo], 0, 1, -1.0, 1.0});
+        if (rlo > 0) {
+          mul.push_back({Clo, M, Plo, rlo, n, n, ld, ld, ld, 0, 0, 1.0, 0.0});
+          lower.push_back({Plo, Clo, fac + S.fS[i][lo], rlo, rlo, n, ld, ld, S.ldS[i][lo], 0, 1, -1.0, 1.0});
         }
-        if (hi >= 0 && S.back[i][hi] > 0) {
-          const int r = S.back[i][hi];
-          const T* C = fac + S.fChi[i][q];
-          T* Phi = P + off;
-          off += int64_t(r) * ld;
-          mul.push_back({C, M, Phi, r, n, n, ld, ld, ld, 0, 0, 1.0, 0.0});
-          upper.push_back({Phi, C, fac + S.fS[i][hi], r, r, n, ld, ld, S.ldS[i][hi], 0, 1, -1.0, 1.0});
-          if (lo >= 0 && S.m[i][hi] > 0)
-            lower.push_back({C, Plo, fac + S.fG[i][hi], r, S.s[i][lo], n, ld, ld, S.ldG[i][hi], 0, 1, -1.0, 1.0});
+        if (rhi > 0) {
+          mul.push_back({Chi, M, Phi, rhi, n, n, ld, ld, ld, 0, 0, 1.0, 0.0});
+          upper.push_back({Phi, Chi, fac + S.fS[i][hi], rhi, rhi, n, ld, ld, S.ldS[i][hi], 0, 1, -1.0, 1.0});
         }
+        if (rlo > 0 && rhi > 0 && S.next[i][lo] == hi)
+          lower.push_back({Chi, Plo, fac + S.fG[i][lo], rhi, rlo, n, ld, ld, S.ldG[i][lo], 0, 1, -1.0, 1.0});
+        if (rlo > 0 && rhi > 0 && S.next[i][hi] == lo)
+          lower.push_back({Clo, Phi, fac + S.fG[i][hi], rlo, rhi, n, ld, ld, S.ldG[i][hi], 0, 1, -1.0, 1.0});
       }
       std::vector<double> mp;
       run_inverse<T>(tmp, inv, mp, s);
@@ -181,46 +181,46 @@ static void condense_mids(const SlabSet& S, T* fac, double& minpiv, cudaStream_t
   tmp.free_all();
 }
 
+// Block LDL^T of the slabs, step by step: S_k^{-1} in place of S_k, then with the rows B_k of the next
+// slab j that are coupled to k: G_k = B_k S_k^{-1}, S_j -= G_k B_k^T.
 template <typename T>
 static void factor_slabs(const SlabSet& S, T* fac, double& minpiv, cudaStream_t s) {
   DevArena tmp(s);
-  int64_t maxB = 1, maxC = 1;
-  for (int k = 0; k < S.Kmax; ++k) {
-    int64_t sb = 0, sc = 0;
+  int64_t maxB = 1;
+  for (int t = 0; t < S.max_steps; ++t) {
+    int64_t n = 0;
     for (int i = 0; i < S.nsub; ++i)
-      if (k >= 1 && k < S.K[i]) sb += int64_t(S.m[i][k]) * S.ldG[i][k];
-    maxB = std::max(maxB, sb);
-    (void)sc;
+      for (int k = 0; k < S.K[i]; ++k)
+        if (S.step[i][k] == t) n += int64_t(S.m[i][k]) * S.ldG[i][k];
+    maxB = std::max(maxB, n);
   }
   T* scrB = tmp.alloc<T>(maxB);
   minpiv = 1e300;
   try {
     condense_mids<T>(S, fac, minpiv, s);
-    // symmetric block LDL^T: G_k = B_k S_{k-1}^{-1}, S_k = A_kk - G_k B_k^T
-    for (int k = 0; k < S.Kmax; ++k) {
-      if (k >= 1) {
-        std::vector<GemmTaskP> tg, tu;
-        int64_t off = 0;
-        for (int i = 0; i < S.nsub; ++i) {
-          if (k >= S.K[i] || S.m[i][k] == 0) continue;
-          int m = S.m[i][k], sp = S.s[i][k - 1];
-          int64_t cnt = int64_t(m) * S.ldG[i][k];
+    for (int t = 0; t < S.max_steps; ++t) {
+      std::vector<InvTaskP> inv;
+      std::vector<GemmTaskP> tg, tu;
+      int64_t off = 0;
+      for (int i = 0; i < S.nsub; ++i)
+        for (int k = 0; k < S.K[i]; ++k) {
+          if (S.step[i][k] != t) continue;
+          inv.push_back({fac + S.fS[i][k], S.s[i][k], S.ldS[i][k], 0});
+          const int m = S.m[i][k], sk = S.s[i][k], j = S.next[i][k];
+          if (j < 0) continue;
+          const int64_t cnt = int64_t(m) * S.ldG[i][k];
           GDSW_CUDA(cudaMemcpyAsync(scrB + off, fac + S.fG[i][k], cnt * sizeof(T), cudaMemcpyDeviceToDevice, s));
-          tg.push_back({scrB + off, fac + S.fS[i][k - 1], fac + S.fG[i][k], m, sp, sp, S.ldG[i][k], S.ldS[i][k - 1],
+          tg.push_back({scrB + off, fac + S.fS[i][k], fac + S.fG[i][k], m, sk, sk, S.ldG[i][k], S.ldS[i][k],
                         S.ldG[i][k], 0, 0, 1.0, 0.0});
-          tu.push_back({fac + S.fG[i][k], scrB + off, fac + S.fS[i][k], m, m, sp, S.ldG[i][k], S.ldG[i][k],
-                        S.ldS[i][k], 0, 1, -1.0, 1.0});
+          tu.push_back({fac + S.fG[i][k], scrB + off, fac + S.fS[i][j], m, m, sk, S.ldG[i][k], S.ldG[i][k],
+                        S.ldS[i][j], 0, 1, -1.0, 1.0});
           off += cnt;
         }
-        run_gemm<T>(tmp, tg, s);
-        run_gemm<T>(tmp, tu, s);
-      }
-      std::vector<InvTaskP> inv;
-      for (int i = 0; i < S.nsub; ++i)
-        if (k < S.K[i]) inv.push_back({fac + S.fS[i][k], S.s[i][k], S.ldS[i][k], 0});
       std::vector<double> mp;
       run_inverse<T>(tmp, inv, mp, s);
       for (double v : mp) minpiv = std::min(minpiv, v);
+      run_gemm<T>(tmp, tg, s);
+      run_gemm<T>(tmp, tu, s);
     }
     GDSW_CUDA(cudaStreamSynchronize(s));
   } catch (...) {
@@ -238,29 +238,30 @@ static void sweep_multi(const SlabSet& S, const T* fac, T* R, T* W, const std::v
                         const std::vector<int>& ldt, const std::vector<int>& nc, cudaStream_t s) {
   DevArena tmp(s);
   try {
-    for (int k = 0; k < S.Kmax; ++k) {
-      std::vector<GemmTaskP> g, d;
-      for (int i = 0; i < S.nsub; ++i) {
-        if (k >= S.K[i] || nc[i] == 0) continue;
-        T* Rk = R + toff[i] + S.soff[i][k] * ldt[i];
-        if (k >= 1 && S.m[i][k] > 0)
-          g.push_back({fac + S.fG[i][k], R + toff[i] + S.soff[i][k - 1] * ldt[i], Rk, S.m[i][k], nc[i], S.s[i][k - 1],
-                       S.ldG[i][k], ldt[i], ldt[i], 0, 0, -1.0, 1.0});
-        d.push_back({fac + S.fS[i][k], Rk, W + toff[i] + S.soff[i][k] * ldt[i], S.s[i][k], nc[i], S.s[i][k],
-                     S.ldS[i][k], ldt[i], ldt[i], 0, 0, 1.0, 0.0});
-      }
+    for (int t = 0; t < S.max_steps; ++t) {
+      std::vector<GemmTaskP> g;  // W_k = S_k^{-1} R_k and the next slab's R_j -= G_k R_k
+      for (int i = 0; i < S.nsub; ++i)
+        for (int k = 0; k < S.K[i]; ++k) {
+          if (S.step[i][k] != t || nc[i] == 0) continue;
+          T* Rk = R + toff[i] + S.soff[i][k] * ldt[i];
+          if (S.next[i][k] >= 0)
+            g.push_back({fac + S.fG[i][k], Rk, R + toff[i] + S.soff[i][S.next[i][k]] * ldt[i], S.m[i][k], nc[i],
+                         S.s[i][k], S.ldG[i][k], ldt[i], ldt[i], 0, 0, -1.0, 1.0});
+          g.push_back({fac + S.fS[i][k], Rk, W + toff[i] + S.soff[i][k] * ldt[i], S.s[i][k], nc[i], S.s[i][k],
+                       S.ldS[i][k], ldt[i], ldt[i], 0, 0, 1.0, 0.0});
+        }
       run_gemm<T>(tmp, g, s);
-      run_gemm<T>(tmp, d, s);
     }
-    for (int j = 0; j + 1 < S.Kmax; ++j) {
+    for (int t = S.max_steps - 2; t >= 0; --t) {
       std::vector<GemmTaskP> b;
-      for (int i = 0; i < S.nsub; ++i) {
-        int k = S.K[i] - 2 - j;
-        if (k < 0 || nc[i] == 0 || S.m[i][k + 1] == 0) continue;
-        // X_k -= G_{k+1}^T X_{k+1}[0:m_{k+1}]  (the super-diagonal block of the symmetric LDL^T)
-        b.push_back({fac + S.fG[i][k + 1], W + toff[i] + S.soff[i][k + 1] * ldt[i], W + toff[i] + S.soff[i][k] * ldt[i],
-                     S.s[i][k], nc[i], S.m[i][k + 1], S.ldG[i][k + 1], ldt[i], ldt[i], 1, 0, -1.0, 1.0});
-      }
+      for (int i = 0; i < S.nsub; ++i)
+        for (int k = 0; k < S.K[i]; ++k) {
+          const int j = S.next[i][k];
+          if (S.step[i][k] != t || j < 0 || nc[i] == 0) continue;
+          // X_k -= G_k^T X_j[0:m_k]  (the block above the diagonal of the symmetric LDL^T)
+          b.push_back({fac + S.fG[i][k], W + toff[i] + S.soff[i][j] * ldt[i], W + toff[i] + S.soff[i][k] * ldt[i],
+                       S.s[i][k], nc[i], S.m[i][k], S.ldG[i][k], ldt[i], ldt[i], 1, 0, -1.0, 1.0});
+        }
       run_gemm<T>(tmp, b, s);
     }
     GDSW_CUDA(cudaStreamSynchronize(s));
@@ -308,7 +309,7 @@ static double plan_bytes(const std::vector<GemvTask>& tasks, int t0, int t1, siz
 // tiles of S_q^{-1}), W (tiles that write w_q: dense S_q^{-1} rows or reductions), X
 // (backward tiles that write x_q).  Every item is listed after all producers it waits for.
 struct TaskRec {
-  int task, q, step, role, t0, t1;  // role: 0 dense S^{-1}, 1 symmetric S^{-1}, 2 G, 3 reduction, 4 backward
+  int task, q, to, step, role, t0, t1;  // to: the next slab; role: 0 dense S^{-1}, 1 symmetric S^{-1}, 2 G, 3 reduction, 4 backward
 };
 
 static void build_sweep(gdsw_ctx* c, LevelDev& L, int nslab, int Kmax, const std::vector<GemvTask>& tasks,
@@ -347,16 +348,23 @@ static void build_sweep(gdsw_ctx* c, LevelDev& L, int nslab, int Kmax, const std
   for (int k = 0; k < Kmax; ++k) {
     for (const TaskRec& r : recs) {
       if (r.step != k || r.role > 2) continue;
-      const int wy = k > 0 ? ctr(r.q, Y) : -1;  // y_q is final once the G task of step k-1 is done
-      const int sig = r.role == 0 ? ctr(r.q, W) : (r.role == 1 ? ctr(r.q, P) : ctr(r.q + 1, Y));
-      for (int t = r.t0; t < r.t1; ++t) emit(r.role == 1 ? SWEEP_SYM : SWEEP_ROWS, r.task, tiles[t].row0, sig, wy, -1);
+      const int wy = ctr(r.q, Y);  // y_q is final once the updates of the slabs before it are done
+      const int sig = r.role == 0 ? ctr(r.q, W) : (r.role == 1 ? ctr(r.q, P) : ctr(r.to, Y));
+      const int before = nsig[sig];  // an update of a slab follows the earlier one of the same rows
+      for (int t = r.t0; t < r.t1; ++t) {
+        emit(r.role == 1 ? SWEEP_SYM : SWEEP_ROWS, r.task, tiles[t].row0, sig, wy, -1);
+        if (r.role == 2 && before > 0) {
+          items.back().wait1 = sig;
+          items.back().need1 = before;
+        }
+      }
     }
     if (k > 0) emit_reduce(k - 1);  // one step behind, so that the partials are mostly done
   }
   if (Kmax > 0) emit_reduce(Kmax - 1);
-  for (const TaskRec& r : recs) {  // backward, in step order: x_k = w_k - G_{k+1}^T x_{k+1}
+  for (const TaskRec& r : recs) {  // backward, in step order: x_k = w_k - G_k^T x_j
     if (r.role != 4) continue;
-    const int wx = nsig[ctr(r.q + 1, X)] > 0 ? ctr(r.q + 1, X) : ctr(r.q + 1, W);
+    const int wx = nsig[ctr(r.to, X)] > 0 ? ctr(r.to, X) : ctr(r.to, W);
     for (int t = r.t0; t < r.t1; ++t) emit(SWEEP_COLS, r.task, tiles[t].row0, ctr(r.q, X), ctr(r.q, W), wx);
   }
   std::vector<GemvTask> all = tasks;
@@ -409,12 +417,12 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
       const int t0 = int(tiles.size());
       for (int I = 0; I < nt; ++I)
         for (int J = I; J < nt; ++J) tiles.push_back({id, (I << 16) | J});
-      if (step >= 0) recs.push_back({id, q, step, 1, t0, int(tiles.size())});
+      if (step >= 0) recs.push_back({id, q, -1, step, 1, t0, int(tiles.size())});
       int rid = int(rtasks.size());
       rtasks.push_back(t);
       const int r0t = int(rtiles.size());
       for (int r0 = 0; r0 < sk; r0 += 256) rtiles.push_back({rid, r0});
-      if (step >= 0) recs.push_back({rid, q, step, 3, r0t, int(rtiles.size())});
+      if (step >= 0) recs.push_back({rid, q, -1, step, 3, r0t, int(rtiles.size())});
       part_off += int64_t(nt) * nt * TT;
       mld = std::max(mld, 11 * TT);
     } else {
@@ -422,7 +430,7 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
       const int t0 = int(tiles.size());
       add_task(tasks, tiles, t, rpt);
       if (step >= 0 && int(tiles.size()) > t0)
-        recs.push_back({int(tasks.size()) - 1, q, step, 0, t0, int(tiles.size())});
+        recs.push_back({int(tasks.size()) - 1, q, -1, step, 0, t0, int(tiles.size())});
       mld = std::max(mld, S.ldS[i][k]);
     }
   };
@@ -437,23 +445,22 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
   L.fwd.launch_task_off = {mid_tasks};
   L.fwd.launch_tile_off = {mid_tiles};
   L.fwd_ld.clear();
-  for (int k = 0; k < S.Kmax; ++k) {
+  for (int st = 0; st < S.max_steps; ++st) {
     int mld = 8;
-    for (int i = 0; i < S.nsub; ++i) {
-      if (k >= S.K[i]) continue;
-      const int q = sb[i] + k;
-      int64_t y = S.voff[i] + S.soff[i][k];
-      const int sk = S.s[i][k];
-      inverse_task(i, k, k, mld);
-      if (k + 1 < S.K[i] && S.m[i][k + 1] > 0) {
-        int64_t y1 = S.voff[i] + S.soff[i][k + 1];
-        GemvTask g{L.pG[q + 1], y, y1, y1, S.m[i][k + 1], sk, S.ldG[i][k + 1], -1.0f};
+    for (int i = 0; i < S.nsub; ++i)
+      for (int k = 0; k < S.K[i]; ++k) {
+        if (S.step[i][k] != st) continue;
+        const int j = S.next[i][k];
+        inverse_task(i, k, st, mld);
+        if (j < 0) continue;
+        const int64_t y = S.voff[i] + S.soff[i][k], y1 = S.voff[i] + S.soff[i][j];
+        GemvTask g{L.pG[sb[i] + k], y, y1, y1, S.m[i][k], S.s[i][k], S.ldG[i][k], -1.0f};
         const int t0 = int(tiles.size());
         add_task(tasks, tiles, g, rpt);
-        if (int(tiles.size()) > t0) recs.push_back({int(tasks.size()) - 1, q, k, 2, t0, int(tiles.size())});
-        mld = std::max(mld, S.ldG[i][k + 1]);
+        if (int(tiles.size()) > t0)
+          recs.push_back({int(tasks.size()) - 1, sb[i] + k, sb[i] + j, st, 2, t0, int(tiles.size())});
+        mld = std::max(mld, S.ldG[i][k]);
       }
-    }
     L.fwd.launch_task_off.push_back(int(tasks.size()));
     L.fwd.launch_tile_off.push_back(int(tiles.size()));
     L.fwd_ld.push_back(mld);
@@ -471,26 +478,26 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
   finish_plan(c->arena, L.red, rtasks, rtiles, c->stream);
   L.midred.d_tasks = L.red.d_tasks;
   L.midred.d_tiles = L.red.d_tiles;
-  // backward: x_k = w_k - G_{k+1}^T x_{k+1}[0:m_{k+1}], transposed GEMV over column tiles
+  // backward: x_k = w_k - G_k^T x_j[0:m_k] with the next slab j, transposed GEMV over column tiles
   L.bwd.transposed = true;
   L.bwd.launch_task_off = {int(tasks.size())};
   L.bwd.launch_tile_off = {int(tiles.size())};
   L.bwd_ld.clear();
-  for (int j = 0; j + 1 < S.Kmax; ++j) {
+  for (int st = S.max_steps - 2; st >= 0; --st) {
     int mrows = 8;
-    for (int i = 0; i < S.nsub; ++i) {
-      int k = S.K[i] - 2 - j;
-      if (k < 0 || S.m[i][k + 1] == 0) continue;
-      int64_t y = nv + S.voff[i] + S.soff[i][k];
-      int64_t x = nv + S.voff[i] + S.soff[i][k + 1];
-      GemvTask t{L.pG[sb[i] + k + 1], x, y, y, S.m[i][k + 1], S.s[i][k], S.ldG[i][k + 1], -1.0f};
-      int id = int(tasks.size());
-      tasks.push_back(t);
-      const int t0 = int(tiles.size());
-      for (int c0 = 0; c0 < t.cols; c0 += gemvt_tile_cols(L.prec)) tiles.push_back({id, c0});
-      recs.push_back({id, sb[i] + k, S.Kmax + j, 4, t0, int(tiles.size())});
-      mrows = std::max(mrows, t.rows);
-    }
+    for (int i = 0; i < S.nsub; ++i)
+      for (int k = 0; k < S.K[i]; ++k) {
+        const int j = S.next[i][k];
+        if (S.step[i][k] != st || j < 0) continue;
+        const int64_t y = nv + S.voff[i] + S.soff[i][k], x = nv + S.voff[i] + S.soff[i][j];
+        GemvTask t{L.pG[sb[i] + k], x, y, y, S.m[i][k], S.s[i][k], S.ldG[i][k], -1.0f};
+        int id = int(tasks.size());
+        tasks.push_back(t);
+        const int t0 = int(tiles.size());
+        for (int c0 = 0; c0 < t.cols; c0 += gemvt_tile_cols(L.prec)) tiles.push_back({id, c0});
+        recs.push_back({id, sb[i] + k, sb[i] + j, S.max_steps + (S.max_steps - 2 - st), 4, t0, int(tiles.size())});
+        mrows = std::max(mrows, t.rows);
+      }
     L.bwd.launch_task_off.push_back(int(tasks.size()));
     L.bwd.launch_tile_off.push_back(int(tiles.size()));
     L.bwd_ld.push_back(mrows);
@@ -507,7 +514,7 @@ static void build_local_plan(gdsw_ctx* c, const SlabSet& S, LevelDev& L) {
     L.fwd_bytes.insert(L.fwd_bytes.begin(), mid + 4.0 * L.to_slabs.ncol + vsz * L.to_slabs.nval);
     L.bwd_bytes.push_back(mid + 4.0 * L.to_mids.ncol + vsz * L.to_mids.nval);
   }
-  build_sweep(c, L, sb[S.nsub], S.Kmax, tasks, tiles, rtasks, rtiles, recs, xs_elems);
+  build_sweep(c, L, sb[S.nsub], S.max_steps, tasks, tiles, rtasks, rtiles, recs, xs_elems);
   resize_sweep(L, L.sweep.ctas_per_sm);
   GemvTask* dt = c->arena.upload(tasks, c->stream);
   GemvTile* dl = c->arena.upload(tiles, c->stream);
@@ -759,7 +766,7 @@ static void store_factors(gdsw_ctx* c, const SlabSet& S, const T* fac, LevelDev&
         off += int64_t(sk) * S.ldS[i][k];
       }
       L.pG.push_back(off);
-      if (k > 0 && k < S.K[i]) off += int64_t(S.m[i][k]) * S.ldG[i][k];
+      if (k < S.K[i]) off += int64_t(S.m[i][k]) * S.ldG[i][k];
     }
   L.nfac = off;
   T* packed = tmp.alloc<T>(std::max<int64_t>(off, 1));
@@ -771,7 +778,7 @@ static void store_factors(gdsw_ctx* c, const SlabSet& S, const T* fac, LevelDev&
       if (!L.psym[q])
         GDSW_CUDA(cudaMemcpyAsync(packed + L.pS[q], fac + S.fS[i][k], sizeof(T) * S.s[i][k] * S.ldS[i][k],
                                   cudaMemcpyDeviceToDevice, s));
-      if (k > 0 && k < S.K[i])
+      if (k < S.K[i] && S.m[i][k] > 0)
         GDSW_CUDA(cudaMemcpyAsync(packed + L.pG[q], fac + S.fG[i][k], sizeof(T) * S.m[i][k] * S.ldG[i][k],
                                   cudaMemcpyDeviceToDevice, s));
     }

@@ -183,11 +183,11 @@ struct InvTask {
 constexpr double kCondenseBytes = 1.5e9;
 
 // ------------------------------------------------------------------ host symbolic structures
-// A batch of block-tridiagonal local problems: dof lists in slab order, slab sizes, the
-// number of back-coupled dofs (those coupled to the previous slab, ordered first) and the
-// offsets of the LDL^T blocks Sinv_k (s_k x s_k) and G_k (m_k x s_{k-1}); the
-// super-diagonal blocks of the symmetric factorisation are the transposes G_{k+1}^T, so no
-// W_k block is stored (fW = -1).
+// A batch of block-tridiagonal local problems: dof lists by slab, slab sizes and the offsets of the LDL^T
+// blocks Sinv_k (s_k x s_k) and G_k (m_k x s_k), the update of slab next[k] by slab k: its first m_k
+// rows are those coupled to k.  Slabs are eliminated from both ends of the axis towards a middle slab,
+// which halves the chain of dependent steps: step[k] says when.  The middle slab's two updates fall into
+// different steps, so that no two blocks add to the same rows at once.
 //
 // Condensed sets (large level-1 factors with slabs one element thick): the node planes in the middle of
 // an element layer hold only velocities and couple to the planes on either side of their layer, so
@@ -201,21 +201,34 @@ struct SlabSet {
   int Kmax = 0;
   std::vector<int> K;
   std::vector<std::vector<int>> s, m;
+  std::vector<std::vector<int>> next, step;  // slab that k updates (-1: none), its elimination step
+  std::vector<std::vector<int>> na, side;    // rows coupled to the slabs it is updated by; -1, 0, 1: before, at, behind the middle
+  std::vector<int> steps;                    // steps per part
+  int max_steps = 0;
   std::vector<int64_t> voff;                 // subdomain offset in the concatenated local vector
   std::vector<std::vector<int64_t>> soff;    // slab offset relative to voff
-  std::vector<std::vector<int64_t>> fS, fG, fW;
-  std::vector<std::vector<int>> ldS, ldG, ldW;
+  std::vector<std::vector<int64_t>> fS, fG;
+  std::vector<std::vector<int>> ldS, ldG;
   int64_t nvec = 0, nfac = 0;
   std::vector<int32_t> gdof;                 // local position -> global dof of the level
   int64_t max_local = 0;
   // Mid layers (condensed sets only): block q of part i is entry K[i] + q of s, soff, fS and ldS.
-  // lo, hi: the slabs below and above it (-1: none); back: dofs of each slab coupled downwards (they
-  // come first); fClo, fChi: its dense couplings, s_lo x ldS and back_hi x ldS, behind the factors
-  std::vector<std::vector<int>> lo, hi, back;
+  // lo, hi: the slabs below and above it (-1: none); fClo, fChi: its dense couplings to their first
+  // rows_lo and rows_hi rows, behind the factors
+  std::vector<std::vector<int>> lo, hi;
   std::vector<std::vector<int64_t>> fClo, fChi;
   int64_t nset = 0;                          // entries of the factorisation's work buffer
   int nmid(int i) const { return lo.empty() ? 0 : int(lo[i].size()); }
   bool condensed() const { return !lo.empty(); }
+  int rows_lo(int i, int q) const {
+    const int k = lo[i][q];
+    return k < 0 ? 0 : (side[i][k] < 0 ? s[i][k] : na[i][k]);
+  }
+  int rows_hi(int i, int q) const {
+    const int k = hi[i][q];
+    return k < 0 ? 0 : (side[i][k] > 0 ? s[i][k] : na[i][k]);
+  }
+  void append(const SlabSet& part);          // one more part
   void layout();                             // fills voff/soff/f*/ld*/nvec/nfac from s, m, K
 };
 

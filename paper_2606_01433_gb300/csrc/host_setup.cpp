@@ -508,14 +508,30 @@ void build_mesh(MeshHost& M, const gdsw_mesh* m) {
 }
 
 // ------------------------------------------------------------------ slab layout
+void SlabSet::append(const SlabSet& p) {
+  K.push_back(p.K[0]);
+  s.push_back(p.s[0]);
+  m.push_back(p.m[0]);
+  next.push_back(p.next[0]);
+  step.push_back(p.step[0]);
+  na.push_back(p.na[0]);
+  side.push_back(p.side[0]);
+  if (p.condensed()) {
+    lo.push_back(p.lo[0]);
+    hi.push_back(p.hi[0]);
+  }
+  gdof.insert(gdof.end(), p.gdof.begin(), p.gdof.end());
+}
+
 void SlabSet::layout() {
   nsub = int(K.size());
   voff.assign(nsub + 1, 0);
   soff.assign(nsub, {});
-  fS.assign(nsub, {}); fG.assign(nsub, {}); fW.assign(nsub, {});
-  ldS.assign(nsub, {}); ldG.assign(nsub, {}); ldW.assign(nsub, {});
+  fS.assign(nsub, {}); fG.assign(nsub, {});
+  ldS.assign(nsub, {}); ldG.assign(nsub, {});
+  steps.assign(nsub, 0);
   nfac = 0;
-  Kmax = 0;
+  Kmax = max_steps = 0;
   max_local = 0;
   for (int i = 0; i < nsub; ++i) {
     Kmax = std::max(Kmax, K[i]);
@@ -528,20 +544,18 @@ void SlabSet::layout() {
     voff[i + 1] = voff[i] + off;
     max_local = std::max(max_local, off);
     for (int k = 0; k < nb; ++k) {
-      int sk = s[i][k];
-      int ld = int(pad8(sk));
+      const int ld = int(pad8(s[i][k]));
       ldS[i].push_back(ld);
       fS[i].push_back(nfac);
-      nfac += int64_t(sk) * ld;
-      // G_k: m_k x s_{k-1}
-      int ldg = k > 0 && k < K[i] ? int(pad8(s[i][k - 1])) : 8;
-      ldG[i].push_back(ldg);
+      nfac += int64_t(s[i][k]) * ld;
+      ldG[i].push_back(ld);  // G_k: m_k x s_k
       fG[i].push_back(nfac);
-      if (k > 0 && k < K[i]) nfac += int64_t(m[i][k]) * ldg;
-      // W_k = S_k^{-1} C_k is not stored: the operator is symmetric, so W_k = G_{k+1}^T
-      ldW[i].push_back(8);
-      fW[i].push_back(-1);
+      if (k < K[i]) {
+        nfac += int64_t(m[i][k]) * ld;
+        steps[i] = std::max(steps[i], step[i][k] + 1);
+      }
     }
+    max_steps = std::max(max_steps, steps[i]);
   }
   nvec = voff[nsub];
   nset = nfac;
@@ -551,10 +565,67 @@ void SlabSet::layout() {
     for (int q = 0; q < nmid(i); ++q) {
       const int64_t ld = ldS[i][K[i] + q];
       fClo[i].push_back(nset);
-      if (lo[i][q] >= 0) nset += s[i][lo[i][q]] * ld;
+      nset += rows_lo(i, q) * ld;
       fChi[i].push_back(nset);
-      if (hi[i][q] >= 0) nset += back[i][hi[i][q]] * ld;
+      nset += rows_hi(i, q) * ld;
     }
+}
+
+// The slabs of one part from the dofs of each slab along the axis (A: coupled to the slabs that update
+// it, which come first; B: the others; slabs without dofs are dropped), middle slab c: appended as the
+// slabs before the middle, those behind it from the far end, the middle.  Returns the index of each.
+static std::vector<int> append_slabs(SlabSet& S, std::vector<std::vector<int32_t>>& A,
+                                     std::vector<std::vector<int32_t>>& B, int c) {
+  const int n = int(A.size());
+  std::vector<int> order, idx(n, -1);
+  for (int k = 0; k < c; ++k) order.push_back(k);
+  for (int k = n - 1; k > c; --k) order.push_back(k);
+  if (c < n) order.push_back(c);
+  int K = 0, nl = 0, nr = 0;
+  for (int k : order) {
+    if (A[k].empty() && B[k].empty()) continue;
+    idx[k] = K++;
+    if (k < c) ++nl;
+    if (k > c) ++nr;
+  }
+  const int shift = nl == nr && nl > 0 ? 1 : 0;  // both ends would update the middle in the same step
+  std::vector<int> s, m, next, step, na, side;
+  for (int k : order) {
+    if (idx[k] < 0) continue;
+    std::sort(A[k].begin(), A[k].end());
+    std::sort(B[k].begin(), B[k].end());
+    S.gdof.insert(S.gdof.end(), A[k].begin(), A[k].end());
+    S.gdof.insert(S.gdof.end(), B[k].begin(), B[k].end());
+    s.push_back(int(A[k].size() + B[k].size()));
+    na.push_back(int(A[k].size()));
+    side.push_back(k < c ? -1 : (k > c ? 1 : 0));
+    const int to = k < c ? k + 1 : (k > c ? k - 1 : -1);
+    const bool up = to >= 0 && to < n && idx[to] >= 0 && !A[to].empty();
+    next.push_back(up ? idx[to] : -1);
+    m.push_back(up ? int(A[to].size()) : 0);
+    step.push_back(k < c ? idx[k] + shift : (k > c ? idx[k] - nl : std::max(nl + shift, nr)));
+  }
+  S.K.push_back(K);
+  S.s.push_back(s);
+  S.m.push_back(m);
+  S.next.push_back(next);
+  S.step.push_back(step);
+  S.na.push_back(na);
+  S.side.push_back(side);
+  return idx;
+}
+
+static void append_empty(SlabSet& S) {
+  std::vector<std::vector<int32_t>> none;
+  append_slabs(S, none, none, 0);
+}
+
+// Middle slab: the first with fewer slabs behind it than before it.  behind(c): slabs behind slab c.
+template <typename F>
+static int middle_slab(F behind) {
+  int c = 0;
+  while (behind(c) > 0 && behind(c) >= c) ++c;
+  return c;
 }
 
 // P1-disc pressure dofs that an element adds to a dof set (they belong to no node).  high:
@@ -562,7 +633,8 @@ void SlabSet::layout() {
 // of its centre.  A set of whole elements (an overlapping subdomain, whose element constants
 // are free) needs `high`: a leading block of the block-tridiagonal factorisation then holds an
 // element's constant only together with every one of its velocity nodes, so the constant
-// pressure on the elements of the leading slabs is never a kernel of the leading block.  The
+// pressure on the elements of the leading slabs is never a kernel of the leading block (behind the
+// middle slab, where the elimination comes from the other end, it is the first node plane).  The
 // linear dofs of an interior set are controlled by the element's centre (bubble) node alone.
 struct ElemDofs {
   int64_t e;
@@ -571,18 +643,14 @@ struct ElemDofs {
   bool high;
 };
 
-// Order the free dofs of a node set for a block-tridiagonal factorisation: slabs of
-// `t` element layers across the longest axis of the set (t = 0: one slab); inside each
-// slab the dofs of nodes coupled to the previous slab come first.  Appends to `S`.
+// Order the free dofs of a node set for a block-tridiagonal factorisation: slabs of `t` element
+// layers across the longest axis of the set (t = 0: one slab), each with its first node plane before
+// the middle slab (a single plane) and with its last one behind it; inside each slab the dofs of
+// nodes coupled to a slab that updates it come first.  Appends to `S`.
 static void slab_order(const MeshHost& M, std::vector<int64_t> nodes, int t, SlabSet& S,
                        const std::vector<ElemDofs>* edofs = nullptr) {
   std::sort(nodes.begin(), nodes.end());
-  if (nodes.empty()) {
-    S.K.push_back(0);
-    S.s.push_back({});
-    S.m.push_back({});
-    return;
-  }
+  if (nodes.empty()) return append_empty(S);
   int lo[3] = {1 << 30, 1 << 30, 1 << 30}, hi[3] = {-1, -1, -1};
   for (int64_t v : nodes) {
     int c[3];
@@ -596,27 +664,30 @@ static void slab_order(const MeshHost& M, std::vector<int64_t> nodes, int t, Sla
   for (int d = 1; d < 3; ++d)
     if (hi[d] - lo[d] > hi[ax] - lo[ax]) ax = d;
   int c0 = lo[ax] - (lo[ax] % 2);
+  const int omax = hi[ax] - c0;
+  auto behind = [&](int c) { return t > 0 ? std::max(0, (omax - 2 * t * c + 2 * t - 1) / (2 * t)) : 0; };
+  const int mid = middle_slab(behind), K = mid + 1 + behind(mid);
+  auto slab_of = [&](int off) {
+    if (t == 0) return 0;
+    return off <= 2 * t * mid ? off / (2 * t) : mid + (off - 2 * t * mid + 2 * t - 1) / (2 * t);
+  };
   // membership lookup over the bounding box
   int bx = hi[0] - lo[0] + 1, by = hi[1] - lo[1] + 1, bz = hi[2] - lo[2] + 1;
   std::vector<int32_t> box(int64_t(bx) * by * bz, -1);
   auto bidx = [&](int i, int j, int k) { return (i - lo[0]) + int64_t(bx) * ((j - lo[1]) + int64_t(by) * (k - lo[2])); };
-  std::vector<int> raw(nodes.size());
+  std::vector<int> slab(nodes.size());
+  std::vector<uint8_t> has_node(K, 0);
   for (size_t q = 0; q < nodes.size(); ++q) {
     int c[3];
     M.coords(nodes[q], c[0], c[1], c[2]);
     box[bidx(c[0], c[1], c[2])] = int32_t(q);
-    raw[q] = t > 0 ? (c[ax] - c0) / (2 * t) : 0;
+    slab[q] = slab_of(c[ax] - c0);
+    has_node[slab[q]] = 1;
   }
-  std::vector<int> uniq(raw);
-  std::sort(uniq.begin(), uniq.end());
-  uniq.erase(std::unique(uniq.begin(), uniq.end()), uniq.end());
-  std::vector<int> slab(nodes.size());
-  for (size_t q = 0; q < nodes.size(); ++q)
-    slab[q] = int(std::lower_bound(uniq.begin(), uniq.end(), raw[q]) - uniq.begin());
-  int K = int(uniq.size());
+  // slab w updates slab k
+  auto updates = [&](int w, int k) { return (w == k - 1 && k <= mid) || (w == k + 1 && k >= mid); };
   std::vector<uint8_t> back(nodes.size(), 0);
   for (size_t q = 0; q < nodes.size(); ++q) {
-    if (slab[q] == 0) continue;
     int c[3];
     M.coords(nodes[q], c[0], c[1], c[2]);
     bool found = false;
@@ -626,7 +697,7 @@ static void slab_order(const MeshHost& M, std::vector<int64_t> nodes, int t, Sla
           int i = c[0] + di, j = c[1] + dj, k = c[2] + dk;
           if (i < lo[0] || i > hi[0] || j < lo[1] || j > hi[1] || k < lo[2] || k > hi[2]) continue;
           int32_t w = box[bidx(i, j, k)];
-          if (w < 0 || slab[w] != slab[q] - 1) continue;
+          if (w < 0 || !updates(slab[w], slab[q])) continue;
           if (M.shares_element(nodes[q], nodes[w])) found = true;
         }
     back[q] = found;
@@ -644,51 +715,26 @@ static void slab_order(const MeshHost& M, std::vector<int64_t> nodes, int t, Sla
       if (i < lo[0] || i > hi[0] || j < lo[1] || j > hi[1] || k < lo[2] || k > hi[2]) return -1;
       return box[bidx(i, j, k)];
     };
-    auto slab_of_raw = [&](int r) {
-      auto it = std::lower_bound(uniq.begin(), uniq.end(), r);
-      return (it != uniq.end() && *it == r) ? int(it - uniq.begin()) : -1;
-    };
     for (const ElemDofs& x : *edofs) {
       const int ec[3] = {int(x.e % M.nx), int((x.e / M.nx) % M.ny), int(x.e / (int64_t(M.nx) * M.ny))};
-      const int centre = 2 * ec[ax] + 1;
-      const int rc = t > 0 ? (centre - c0) / (2 * t) : 0;
+      const int centre = 2 * ec[ax] + 1 - c0;
       int sl = -1;
-      if (x.high) sl = slab_of_raw(t > 0 ? (centre + 1 - c0) / (2 * t) : 0);
-      if (sl < 0) sl = slab_of_raw(rc);
+      if (x.high) sl = slab_of(centre < 2 * t * mid || t == 0 ? centre + 1 : centre - 1);
+      if (sl < 0 || sl >= K || !has_node[sl]) sl = slab_of(centre);
+      if (sl >= K || !has_node[sl]) sl = -1;
       GDSW_CHECK(sl >= 0, GDSW_ERR_INVALID_ARG, "element pressure dofs without their element's nodes");
       bool bk = false;
       for (int z = 0; z < 3 && !bk; ++z)
         for (int y = 0; y < 3 && !bk; ++y)
           for (int w = 0; w < 3 && !bk; ++w) {
             const int32_t q = member(2 * ec[0] + w, 2 * ec[1] + y, 2 * ec[2] + z);
-            if (q >= 0 && slab[q] == sl - 1) bk = true;
+            if (q >= 0 && updates(slab[q], sl)) bk = true;
           }
       auto& dst = bk ? A[sl] : B[sl];
       for (int c = 0; c < x.n; ++c) dst.push_back(x.d[c]);
     }
   }
-  std::vector<int> s, m;
-  for (int k = 0; k < K; ++k) {
-    std::sort(A[k].begin(), A[k].end());
-    std::sort(B[k].begin(), B[k].end());
-    s.push_back(int(A[k].size() + B[k].size()));
-    m.push_back(int(A[k].size()));
-    S.gdof.insert(S.gdof.end(), A[k].begin(), A[k].end());
-    S.gdof.insert(S.gdof.end(), B[k].begin(), B[k].end());
-  }
-  // drop empty slabs (a slab can be empty of dofs if all its nodes are Dirichlet-only)
-  std::vector<int> s2, m2;
-  for (int k = 0; k < K; ++k)
-    if (s[k] > 0) {
-      s2.push_back(s[k]);
-      m2.push_back(m[k]);
-    } else if (k + 1 < K) {
-      m[k + 1] = 0;
-    }
-  if (!s2.empty()) m2[0] = 0;
-  S.K.push_back(int(s2.size()));
-  S.s.push_back(s2);
-  S.m.push_back(m2);
+  append_slabs(S, A, B, mid);
 }
 
 // Order the free dofs of a node set for the condensed factorisation (one part per call): slabs are the
@@ -699,13 +745,9 @@ static void slab_order(const MeshHost& M, std::vector<int64_t> nodes, int t, Sla
 static void condensed_order(const MeshHost& M, std::vector<int64_t> nodes, SlabSet& S,
                             const std::vector<ElemDofs>* edofs) {
   std::sort(nodes.begin(), nodes.end());
-  S.K.push_back(0);
-  S.s.push_back({});
-  S.m.push_back({});
   S.lo.push_back({});
   S.hi.push_back({});
-  S.back.push_back({});
-  if (nodes.empty()) return;
+  if (nodes.empty()) return append_empty(S);
   int lo[3] = {1 << 30, 1 << 30, 1 << 30}, hi[3] = {-1, -1, -1};
   for (int64_t v : nodes) {
     int c[3];
@@ -718,7 +760,10 @@ static void condensed_order(const MeshHost& M, std::vector<int64_t> nodes, SlabS
   int ax = 0;
   for (int d = 1; d < 3; ++d)
     if (hi[d] - lo[d] > hi[ax] - lo[ax]) ax = d;
-  const int c0 = lo[ax] - (lo[ax] % 2), nplane = hi[ax] - c0 + 2;
+  const int c0 = lo[ax] - (lo[ax] % 2), nplane = hi[ax] - c0 + 1, nslab = (nplane + 1) / 2;
+  const int mid = middle_slab([&](int c) { return nslab - 1 - c; });
+  // the planes on the side from which slab p / 2 is updated
+  auto updates = [&](int w, int p) { return (w < p && p <= 2 * mid) || (w > p && p >= 2 * mid); };
   std::vector<uint8_t> box(int64_t(hi[0] - lo[0] + 1) * (hi[1] - lo[1] + 1) * (hi[2] - lo[2] + 1), 0);
   auto member = [&](int i, int j, int k) -> uint8_t* {
     if (i < lo[0] || i > hi[0] || j < lo[1] || j > hi[1] || k < lo[2] || k > hi[2]) return nullptr;
@@ -729,7 +774,7 @@ static void condensed_order(const MeshHost& M, std::vector<int64_t> nodes, SlabS
     M.coords(v, c[0], c[1], c[2]);
     *member(c[0], c[1], c[2]) = 1;
   }
-  // per plane: dofs coupled to a lower plane, the others
+  // per plane: dofs coupled to a plane on that side, the others
   std::vector<std::vector<int32_t>> A(nplane), B(nplane);
   std::vector<uint8_t> has_node(nplane, 0);
   for (int64_t v : nodes) {
@@ -743,7 +788,7 @@ static void condensed_order(const MeshHost& M, std::vector<int64_t> nodes, SlabS
         for (int dj = -2; dj <= 2 && !back; ++dj)
           for (int di = -2; di <= 2 && !back; ++di) {
             const int d[3] = {di, dj, dk};
-            if (d[ax] >= 0) continue;
+            if (!updates(plane + d[ax], plane)) continue;
             const uint8_t* w = member(c[0] + di, c[1] + dj, c[2] + dk);
             if (!w || !*w) continue;
             back = M.shares_element(v, (c[0] + di) + int64_t(M.NX) * ((c[1] + dj) + int64_t(M.NY) * (c[2] + dk)));
@@ -758,7 +803,8 @@ static void condensed_order(const MeshHost& M, std::vector<int64_t> nodes, SlabS
       const int ec[3] = {int(x.e % M.nx), int((x.e / M.nx) % M.ny), int(x.e / (int64_t(M.nx) * M.ny))};
       const int centre = 2 * ec[ax] + 1 - c0;
       int plane = -1;
-      for (int p : {centre + 1, centre - 1, centre})
+      const int first = centre < 2 * mid ? centre + 1 : centre - 1;
+      for (int p : {first, 2 * centre - first, centre})
         if (plane < 0 && p >= 0 && p < nplane && has_node[p]) plane = p;
       GDSW_CHECK(plane >= 0, GDSW_ERR_INVALID_ARG, "element pressure dofs without their element's nodes");
       bool back = false;
@@ -768,49 +814,31 @@ static void condensed_order(const MeshHost& M, std::vector<int64_t> nodes, SlabS
             for (int w = 0; w < 3; ++w) {
               const int c[3] = {2 * ec[0] + w, 2 * ec[1] + y, 2 * ec[2] + z};
               const uint8_t* q = member(c[0], c[1], c[2]);
-              back |= q && *q && c[ax] - c0 < plane;
+              back |= q && *q && updates(c[ax] - c0, plane);
             }
       auto& dst = back ? A[plane] : B[plane];
       for (int c = 0; c < x.n; ++c) dst.push_back(x.d[c]);
     }
-  std::vector<int> slab(nplane + 1, -1);  // plane -> slab (planes without dofs are dropped)
-  for (int p = 0; p < nplane; p += 2) {
-    std::sort(A[p].begin(), A[p].end());
-    std::sort(B[p].begin(), B[p].end());
-    if (A[p].empty() && B[p].empty()) continue;
-    slab[p] = S.K[0]++;
-    S.s[0].push_back(int(A[p].size() + B[p].size()));
-    S.back[0].push_back(int(A[p].size()));
-    // coupled to the previous slab (directly and through the mid layer) only if that is two planes below
-    S.m[0].push_back(p >= 2 && slab[p - 2] >= 0 ? int(A[p].size()) : 0);
-    S.gdof.insert(S.gdof.end(), A[p].begin(), A[p].end());
-    S.gdof.insert(S.gdof.end(), B[p].begin(), B[p].end());
+  std::vector<std::vector<int32_t>> SA(nslab), SB(nslab);
+  for (int k = 0; k < nslab; ++k) {
+    SA[k].swap(A[2 * k]);
+    SB[k].swap(B[2 * k]);
   }
+  const std::vector<int> slab = append_slabs(S, SA, SB, mid);
   for (int p = 1; p < nplane; p += 2) {
-    std::sort(B[p].begin(), B[p].end());
     if (B[p].empty()) continue;
+    std::sort(B[p].begin(), B[p].end());
     S.s[0].push_back(int(B[p].size()));
-    S.m[0].push_back(0);
-    S.lo[0].push_back(slab[p - 1]);
-    S.hi[0].push_back(p + 1 < nplane ? slab[p + 1] : -1);
+    S.lo[0].push_back(slab[p / 2]);
+    S.hi[0].push_back(p / 2 + 1 < nslab ? slab[p / 2 + 1] : -1);
     S.gdof.insert(S.gdof.end(), B[p].begin(), B[p].end());
   }
 }
 
 // One dense block holding sorted dofs (coarse levels).
 static void dense_order(const std::vector<int32_t>& dofs, SlabSet& S) {
-  std::vector<int32_t> d(dofs);
-  std::sort(d.begin(), d.end());
-  if (d.empty()) {
-    S.K.push_back(0);
-    S.s.push_back({});
-    S.m.push_back({});
-    return;
-  }
-  S.K.push_back(1);
-  S.s.push_back({int(d.size())});
-  S.m.push_back({0});
-  S.gdof.insert(S.gdof.end(), d.begin(), d.end());
+  std::vector<std::vector<int32_t>> none(1), all(1, dofs);
+  append_slabs(S, none, all, 0);
 }
 
 static void scatter_lists(LevelHost& L, int weighting) {
@@ -1038,17 +1066,7 @@ void build_level1(gdsw_ctx* ctx, const gdsw_partition* part, int overlap, int sl
           slab_order(M, onodes[i], slab_elems, parts[i], M.pdisc ? &ed : nullptr);
       });
       S = SlabSet();
-      for (int i = 0; i < N; ++i) {
-        S.K.push_back(parts[i].K[0]);
-        S.s.push_back(parts[i].s[0]);
-        S.m.push_back(parts[i].m[0]);
-        if (condensed) {
-          S.lo.push_back(parts[i].lo[0]);
-          S.hi.push_back(parts[i].hi[0]);
-          S.back.push_back(parts[i].back[0]);
-        }
-        S.gdof.insert(S.gdof.end(), parts[i].gdof.begin(), parts[i].gdof.end());
-      }
+      for (int i = 0; i < N; ++i) S.append(parts[i]);
       S.layout();
     }
   }
@@ -1220,12 +1238,7 @@ void build_level1(gdsw_ctx* ctx, const gdsw_partition* part, int overlap, int sl
     parallel_tasks(N, [&](int64_t i) { slab_order(M, inodes[i], slab_elems, parts[i], M.pdisc ? &ied[i] : nullptr); });
     SlabSet& S = L.inter;
     S = SlabSet();
-    for (int i = 0; i < N; ++i) {
-      S.K.push_back(parts[i].K[0]);
-      S.s.push_back(parts[i].s[0]);
-      S.m.push_back(parts[i].m[0]);
-      S.gdof.insert(S.gdof.end(), parts[i].gdof.begin(), parts[i].gdof.end());
-    }
+    for (int i = 0; i < N; ++i) S.append(parts[i]);
     S.layout();
     C.idofs = S.gdof;
     C.ioff = S.voff;

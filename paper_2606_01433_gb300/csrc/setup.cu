@@ -55,9 +55,9 @@ __global__ void k_map_reset(const int32_t* __restrict__ gdof, const int32_t* __r
   map[slot + gdof[p]] = -1;
 }
 
-// Write A restricted to a slab set into its blocks: diagonal S_k, sub-diagonal B_k (rows
-// = back-coupled dofs of slab k) and super-diagonal C_k (columns = back-coupled dofs of
-// slab k+1).  Any other coupling means the ordering is wrong: flagged in *err.
+// Write A restricted to a slab set into its blocks: diagonal S_k, the updates B_k (rows = dofs of the
+// next slab coupled to slab k), couplings of mid layers.  Any other coupling means the ordering is
+// wrong: flagged in *err.
 template <typename T>
 __global__ void k_extract(MatView A, SlabView S, int64_t p0, int64_t p1, int i0, int separate,
                           const int32_t* __restrict__ map, T* __restrict__ fac, int* __restrict__ err) {
@@ -75,17 +75,15 @@ __global__ void k_extract(MatView A, SlabView S, int64_t p0, int64_t p1, int i0,
     if (kc == kr) {
       fac[S.fS[sb + kr] + int64_t(r) * S.ldS[sb + kr] + c] = T(v);
     } else if (kr >= K || kc >= K) {  // a mid layer: its couplings are kept with the slab's rows
-      const int mid = sb + (kc >= K ? kc : kr), k = kc >= K ? kr : kc;
-      if (k >= K || (k != S.lo[mid] && (k != S.hi[mid] || (kc >= K ? r : c) >= S.back[sb + k])))
+      const int mid = sb + (kc >= K ? kc : kr), k = kc >= K ? kr : kc, row = kc >= K ? r : c;
+      const bool lo = k == S.lo[mid] && row < S.nlo[mid], hi = k == S.hi[mid] && row < S.nhi[mid];
+      if (k >= K || !(lo || hi))
         atomicExch(err, 1);
       else if (kc >= K)
-        fac[(k == S.lo[mid] ? S.fClo[mid] : S.fChi[mid]) + int64_t(r) * S.ldS[mid] + c] = T(v);
-    } else if (kc == kr - 1 && r < S.m[sb + kr]) {
-      fac[S.fG[sb + kr] + int64_t(r) * S.ldG[sb + kr] + c] = T(v);
-    } else if (kc == kr + 1 && c < S.m[sb + kc]) {
-      // super-diagonal coupling: the transpose of the next slab's sub-diagonal block
-      if (S.fW[sb + kr] >= 0) fac[S.fW[sb + kr] + int64_t(r) * S.ldW[sb + kr] + c] = T(v);
-    } else {
+        fac[(lo ? S.fClo[mid] : S.fChi[mid]) + int64_t(r) * S.ldS[mid] + c] = T(v);
+    } else if (S.next[sb + kc] == kr && r < S.m[sb + kc]) {
+      fac[S.fG[sb + kc] + int64_t(r) * S.ldG[sb + kc] + c] = T(v);
+    } else if (S.next[sb + kr] != kc || c >= S.m[sb + kr]) {  // else the transpose of an update
       atomicExch(err, 1);
     }
   });

@@ -21,11 +21,10 @@ struct SlabView {
   const int32_t* pidx;       // position -> index within its slab
   const int64_t* voff;       // part -> first position
   const int32_t* slab_base;  // part -> index of its first slab in the per-slab arrays
-  const int64_t *fS, *fG, *fW;
-  const int32_t *ldS, *ldG, *ldW, *m;
-  // condensed sets: slabs per part; per block slab below, slab above, rows
-  // coupled downwards and the offsets of the couplings
-  const int32_t *nslab, *lo, *hi, *back;
+  const int64_t *fS, *fG;
+  const int32_t *ldS, *ldG, *m, *next;
+  // slabs per part; mid layers of condensed sets: slabs below and above, rows and offsets of the couplings
+  const int32_t *nslab, *lo, *hi, *nlo, *nhi;
   const int64_t *fClo, *fChi;
 };
 
