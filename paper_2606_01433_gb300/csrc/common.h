@@ -176,11 +176,12 @@ struct InvTask {
 };
 
 // Factors of at least this many bytes are condensed.  Smaller ones run at the latency of their launches,
-// of which condensing adds four to six.  Local solves, plain -> condensed: channel with obstacles
-// 32^3, 64 parts, FP32 (11.6 GB) 1968 -> 1390 us; die, 64 parts, FP32 (1.9 GB) 423 -> 406 us; 20^3 box, 64
-// parts, FP32 (1.7 GB) 342 -> 334 us; the die in BF16 (1.0 GB) 349 -> 385 us; 14^3, 27 parts, FP64 (0.9 GB)
-// 380 -> 389 us; 8^3, 8 parts, FP32 (54 MB) 55 -> 62 us.
-constexpr double kCondenseBytes = 1.5e9;
+// of which condensing adds four to six.  Local solves, plain -> condensed.  FP32: channel with obstacles
+// 32^3, 64 parts (11.4 GB) 1937 -> 1380 us, die, 64 parts (1.9 GB) 424 -> 393, 20^3 box, 64 parts (1.7 GB)
+// 343 -> 325.  FP64: 17x14x12 box, 36 parts, discontinuous pressure (0.99 GB) 398 -> 366, 14^3, 27 parts (0.91
+// GB) 354 -> 351.  BF16, whose smaller blocks are stored in full: die (0.95 GB) 328 -> 371, 20^3 (0.84 GB)
+// 271 -> 292.
+inline double condense_bytes(int prec) { return prec == GDSW_BF16 ? 1.5e9 : 0.9e9; }
 
 // ------------------------------------------------------------------ host symbolic structures
 // A batch of block-tridiagonal local problems: dof lists by slab, slab sizes and the offsets of the LDL^T

@@ -1050,8 +1050,9 @@ void build_level1(gdsw_ctx* ctx, const gdsw_partition* part, int overlap, int sl
   });
   {
     SlabSet& S = L.loc;
+    const int prec = ctx->opt.precision[0];
     for (bool condensed : {false, true}) {
-      if (condensed && (slab_elems != 1 || double(S.nfac) * elem_size(ctx->opt.precision[0]) < kCondenseBytes)) break;
+      if (condensed && (slab_elems != 1 || double(S.nfac) * elem_size(prec) < condense_bytes(prec))) break;
       std::vector<SlabSet> parts(N);
       parallel_tasks(N, [&](int64_t i) {
         std::vector<ElemDofs> ed;
