@@ -1666,6 +1666,7 @@ void gdsw_destroy(gdsw_ctx* c) {
     c->ev_pool.push_back(p.b);
   }
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
+  if (c->h_est) cudaFreeHost(c->h_est);
   c->arena.free_all();
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);

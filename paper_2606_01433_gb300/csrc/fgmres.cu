@@ -401,6 +401,7 @@ static void ensure_workspace(gdsw_ctx* c, int m) {
   c->d_count = c->arena.alloc<unsigned>(1 + groups);
   GDSW_CUDA(cudaMemsetAsync(c->d_count, 0, sizeof(unsigned) * (1 + groups), c->stream));
   c->d_scal = c->arena.alloc<double>(8);
+  if (!c->h_est) GDSW_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&c->h_est), 2 * sizeof(double), cudaHostAllocDefault));
   c->m_alloc = m;
 }
 
@@ -443,6 +444,22 @@ static void arnoldi_step(gdsw_ctx* c, int j, double* w, cudaStream_t s) {
   check_launch("k_scale_givens");
 }
 
+// Two iterations may be in flight: the estimate of one is read while the next runs, so that the device
+// does not wait for the host (10 us of the 117 us of an iteration on an 8^3 box).  An iteration whose
+// predecessor turns out to have converged is dropped -- its column of H, its vectors and its
+// entries of the rotated right-hand side are not read -- and the margin keeps that rare.
+constexpr double kAheadMargin = 0.3;
+struct EventPair {
+  cudaEvent_t e[2] = {nullptr, nullptr};
+  EventPair() {
+    for (cudaEvent_t& v : e) GDSW_CUDA(cudaEventCreateWithFlags(&v, cudaEventDisableTiming));
+  }
+  ~EventPair() {
+    for (cudaEvent_t v : e)
+      if (v) cudaEventDestroy(v);
+  }
+};
+
 void fgmres_solve(gdsw_ctx* c, const double* b, double* x, gdsw_solve_info* info) {
   cudaStream_t s = c->stream;
   const int64_t n = c->mesh.n;
@@ -472,6 +489,8 @@ void fgmres_solve(gdsw_ctx* c, const double* b, double* x, gdsw_solve_info* info
     return;
   }
   const double tol = c->opt.tol;
+  const bool may_run_ahead = !c->ext_precond;  // a V-cycle waits for its coarse solve anyway
+  EventPair copied;
   int it = 0;
   double est = 0.0, beta = 0.0;
   const double spmv_b = c->spmv_bytes();
@@ -486,6 +505,18 @@ void fgmres_solve(gdsw_ctx* c, const double* b, double* x, gdsw_solve_info* info
     check_launch("k_norm_finish");
     GDSW_CUDA(cudaMemcpyAsync(&beta, c->d_scal, 8, cudaMemcpyDeviceToHost, s));
     GDSW_CUDA(cudaStreamSynchronize(s));
+  };
+  auto iteration = [&](int j) {
+    double* zj = c->d_Z + int64_t(j) * n;
+    double* w = c->d_V + int64_t(j + 1) * n;
+    apply_precond(c, c->d_V + int64_t(j) * n, zj, s);
+    {
+      ProfScope ps(c, GDSW_K_SPMV, spmv_b, s);
+      launch_spmv(c, zj, w, nullptr, s);
+    }
+    arnoldi_step(c, j, w, s);
+    GDSW_CUDA(cudaMemcpyAsync(c->h_est + (j & 1), c->d_scal + 2, 8, cudaMemcpyDeviceToHost, s));
+    GDSW_CUDA(cudaEventRecord(copied.e[j & 1], s));
   };
   true_residual();
   int status = GDSW_OK;
@@ -504,19 +535,19 @@ void fgmres_solve(gdsw_ctx* c, const double* b, double* x, gdsw_solve_info* info
     k_cycle_start<<<(m + 1 + 127) / 128, 128, 0, s>>>(c->d_gvec, m + 1, c->d_scal);
     check_launch("k_cycle_start");
     int jd = 0;
+    bool ahead = false;
+    double last = 0.0;  // the estimate before est
+    est = beta;
     for (int j = 0; j < m && it < c->opt.max_it; ++j) {
-      double* vj = c->d_V + int64_t(j) * n;
-      double* zj = c->d_Z + int64_t(j) * n;
-      double* w = c->d_V + int64_t(j + 1) * n;
-      apply_precond(c, vj, zj, s);
-      {
-        ProfScope ps(c, GDSW_K_SPMV, spmv_b, s);
-        launch_spmv(c, zj, w, nullptr, s);
-      }
-      arnoldi_step(c, j, w, s);
-      GDSW_CUDA(cudaMemcpyAsync(c->h_scal, c->d_scal + 2, 8, cudaMemcpyDeviceToHost, s));
-      GDSW_CUDA(cudaStreamSynchronize(s));
-      est = c->h_scal[0];
+      if (!ahead) iteration(j);
+      // the next iteration is queued before this one's estimate is here, unless one more step at the
+      // last rate could reach the tolerance
+      ahead = may_run_ahead && j >= 2 && j + 1 < m && it + 1 < c->opt.max_it &&
+              kAheadMargin * est * std::min(1.0, est / last) > tol * bnorm;
+      if (ahead) iteration(j + 1);
+      GDSW_CUDA(cudaEventSynchronize(copied.e[j & 1]));
+      last = est;
+      est = c->h_est[j & 1];
       ++it;
       jd = j + 1;
       if (!std::isfinite(est)) {
