@@ -14,6 +14,7 @@
 namespace gdsw {
 
 void fgmres_solve(gdsw_ctx* c, const double* b, double* x, gdsw_solve_info* info);
+void give_estimates(double* p);
 
 static thread_local std::string g_setup_error;
 
@@ -1666,7 +1667,7 @@ void gdsw_destroy(gdsw_ctx* c) {
     c->ev_pool.push_back(p.b);
   }
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
-  if (c->h_est) cudaFreeHost(c->h_est);
+  give_estimates(c->h_est);
   c->arena.free_all();
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);

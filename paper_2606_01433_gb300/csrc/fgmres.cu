@@ -7,6 +7,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <mutex>
+#include <vector>
 
 #include "common.h"
 #include "kernels.h"
@@ -386,6 +388,48 @@ static int arnoldi_ctas(int64_t n) {
   return int(waves * kWave);
 }
 
+// Pinned pairs of estimates for the contexts of the process.  Freeing pinned memory waits for the whole
+// device, so a context gives its pair back instead; the page goes with the last context that holds a
+// pair.  Contexts beyond the page's pairs allocate their own.
+static std::mutex g_est_mu;
+static double* g_est_page = nullptr;
+static std::vector<int> g_est_free;
+constexpr int kEstPairs = 256;
+
+static double* pinned(int n) {
+  void* p = nullptr;
+  GDSW_CUDA(cudaHostAlloc(&p, n * sizeof(double), cudaHostAllocPortable));
+  return static_cast<double*>(p);
+}
+
+static double* take_estimates() {
+  std::lock_guard<std::mutex> lock(g_est_mu);
+  if (!g_est_page) {
+    g_est_free.resize(kEstPairs);
+    for (int i = 0; i < kEstPairs; ++i) g_est_free[i] = i;
+    g_est_page = pinned(2 * kEstPairs);
+  }
+  if (g_est_free.empty()) return pinned(2);
+  const int i = g_est_free.back();
+  g_est_free.pop_back();
+  return g_est_page + 2 * i;
+}
+
+void give_estimates(double* p) {
+  if (!p) return;
+  std::lock_guard<std::mutex> lock(g_est_mu);
+  if (!g_est_page || p < g_est_page || p >= g_est_page + 2 * kEstPairs) {
+    cudaFreeHost(p);
+    return;
+  }
+  g_est_free.push_back(int((p - g_est_page) / 2));
+  if (int(g_est_free.size()) == kEstPairs) {
+    cudaFreeHost(g_est_page);
+    g_est_page = nullptr;
+    g_est_free.clear();
+  }
+}
+
 static void ensure_workspace(gdsw_ctx* c, int m) {
   if (c->m_alloc >= m) return;
   const int64_t n = c->mesh.n;
@@ -401,7 +445,7 @@ static void ensure_workspace(gdsw_ctx* c, int m) {
   c->d_count = c->arena.alloc<unsigned>(1 + groups);
   GDSW_CUDA(cudaMemsetAsync(c->d_count, 0, sizeof(unsigned) * (1 + groups), c->stream));
   c->d_scal = c->arena.alloc<double>(8);
-  if (!c->h_est) GDSW_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&c->h_est), 2 * sizeof(double), cudaHostAllocDefault));
+  if (!c->h_est) c->h_est = take_estimates();
   c->m_alloc = m;
 }
 

@@ -41,3 +41,20 @@ def test_counted_iterations(lib, max_it, restart, tol):
     assert abs(true - info.relres) <= 1e-10 * (1 + true)
     assert abs(info.est_relres - info.relres) <= 1e-3 * info.est_relres
     ctx.close()
+
+
+def test_many_contexts(lib):
+    """More contexts alive at once than the shared page has estimate pairs (256); pairs given back are
+    used again."""
+    p = I.box_problem(3, 3, 3, (1, 1, 1), levels=2, form="symmetric", uk_seed=3, lam=1.0, n=0.5, nu_inf=1e-2)
+    ref = None
+    for count in (258, 2):
+        ctxs = [lib.Context(p, tol=1e-10) for _ in range(count)]
+        b = torch.from_numpy(np.random.default_rng(5).standard_normal(ctxs[0].n)).cuda()
+        for c in ctxs:
+            x = torch.zeros_like(b)
+            assert c.gdsw_solve(b, x).relres <= 1e-10
+            ref = x if ref is None else ref
+            assert torch.equal(x, ref)
+        for c in ctxs:
+            c.close()
