@@ -20,30 +20,16 @@ __host__ __device__ constexpr double q2_d(int a, int q) {
 // time (the Q2 basis is a tensor product: 72 multiply-adds per point and component triple instead
 // of 243).  Thread q = 0..26 of the element owns node q, then the partial results of index q, then
 // Gauss point q (x fastest throughout); u, s, t are the element's shared arrays [c][27], `sync` is
-// a barrier over the element's threads.  In FP32 the basis values keep a second word (hi + lo): their
-// rounding, the same at every element, would otherwise be half of the error of an operator product.
+// a barrier over the element's threads.
 template <typename T>
 struct Grad1D {
   T v[3][3], d[3][3];   // [basis][point]
-};
-template <>
-struct Grad1D<float> {
-  float v[3][3], d[3][3], vl[3][3], dl[3][3];
 };
 __device__ __forceinline__ void fill_grad1d(Grad1D<double>& B, int tid) {
   if (tid < 9) {
     B.v[tid / 3][tid % 3] = q2_v(tid / 3, tid % 3);
     B.d[tid / 3][tid % 3] = q2_d(tid / 3, tid % 3);
   }
-}
-inline void host_grad1d(Grad1D<float>& B) {
-  for (int a = 0; a < 3; ++a)
-    for (int q = 0; q < 3; ++q) {
-      B.v[a][q] = float(q2_v(a, q));
-      B.vl[a][q] = float(q2_v(a, q) - double(B.v[a][q]));
-      B.d[a][q] = float(q2_d(a, q));
-      B.dl[a][q] = float(q2_d(a, q) - double(B.d[a][q]));
-    }
 }
 // acc + sum over k of p[k step] times the values (DER: derivatives) of basis k at point i, or (TEST) of
 // basis i at point k
@@ -53,15 +39,6 @@ __device__ __forceinline__ double line(const Grad1D<double>& B, int i, const dou
   return fma(p[2 * step], TEST ? b[i][2] : b[2][i],
              fma(p[step], TEST ? b[i][1] : b[1][i], fma(p[0], TEST ? b[i][0] : b[0][i], acc)));
 }
-template <bool DER, bool TEST>
-__device__ __forceinline__ float line(const Grad1D<float>& B, int i, const float* p, int step, float acc) {
-  const float(*h)[3] = DER ? B.d : B.v;
-  const float(*l)[3] = DER ? B.dl : B.vl;
-  const float p0 = p[0], p1 = p[step], p2 = p[2 * step];
-  acc = fmaf(p2, TEST ? l[i][2] : l[2][i], fmaf(p1, TEST ? l[i][1] : l[1][i], fmaf(p0, TEST ? l[i][0] : l[0][i], acc)));
-  return fmaf(p2, TEST ? h[i][2] : h[2][i], fmaf(p1, TEST ? h[i][1] : h[1][i], fmaf(p0, TEST ? h[i][0] : h[0][i], acc)));
-}
-
 template <typename T, typename Sync>
 __device__ __forceinline__ void element_gradient(const Grad1D<T>& B, int q, bool active, const T (*u)[27],
                                                  T (*s)[3][27], T (*t)[3][27], T gr[3][3], Sync sync) {
@@ -115,6 +92,39 @@ __device__ __forceinline__ void element_test(const Grad1D<T>& B, int q, bool act
 #pragma unroll
     for (int c = 0; c < 3; ++c)
       f[c] = line<true, true>(B, x, s[c][0] + q - x, 1, line<false, true>(B, x, s[c][1] + q - x, 1, T(0)));
+}
+
+// ------------------------------------------------------------------ the same in FP32, a line per thread
+// A thread that owns a whole line of three nodes (or points) of one component reads each value once for
+// all three results, and the basis values are constants in the instructions, those of the middle point
+// (0, 1, 0 and -1/2, 0, 1/2) left out.  Every constant keeps a second word (hi + lo): its rounding,
+// the same at every element, would otherwise be half of the error of an operator product.
+// acc + sum over k of p_k times the value (DER: derivative) of basis k at point I, or (TEST) of basis I at
+// point k
+template <bool DER, bool TEST, int I>
+__device__ __forceinline__ float line_at(const float (&p)[3], float acc) {
+  constexpr double c0 = DER ? (TEST ? q2_d(I, 0) : q2_d(0, I)) : (TEST ? q2_v(I, 0) : q2_v(0, I));
+  constexpr double c1 = DER ? (TEST ? q2_d(I, 1) : q2_d(1, I)) : (TEST ? q2_v(I, 1) : q2_v(1, I));
+  constexpr double c2 = DER ? (TEST ? q2_d(I, 2) : q2_d(2, I)) : (TEST ? q2_v(I, 2) : q2_v(2, I));
+  constexpr float h0 = float(c0), h1 = float(c1), h2 = float(c2);
+  constexpr float l0 = float(c0 - double(h0)), l1 = float(c1 - double(h1)), l2 = float(c2 - double(h2));
+  if constexpr (l0 != 0.f) acc = fmaf(p[0], l0, acc);
+  if constexpr (l1 != 0.f) acc = fmaf(p[1], l1, acc);
+  if constexpr (l2 != 0.f) acc = fmaf(p[2], l2, acc);
+  if constexpr (h0 != 0.f) acc = fmaf(p[0], h0, acc);
+  if constexpr (h1 != 0.f) acc = fmaf(p[1], h1, acc);
+  if constexpr (h2 != 0.f) acc = fmaf(p[2], h2, acc);
+  return acc;
+}
+// out[i step] for the three i of a line
+template <bool DER, bool TEST>
+__device__ __forceinline__ void line_all(const float (&p)[3], float* out, int step) {
+  out[0] = line_at<DER, TEST, 0>(p, 0.f);
+  out[step] = line_at<DER, TEST, 1>(p, 0.f);
+  out[2 * step] = line_at<DER, TEST, 2>(p, 0.f);
+}
+__device__ __forceinline__ void load_line(const float* p, int step, float (&v)[3]) {
+  v[0] = p[0], v[1] = p[step], v[2] = p[2 * step];
 }
 
 }  // namespace gdsw

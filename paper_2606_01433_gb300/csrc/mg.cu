@@ -402,30 +402,29 @@ __global__ void k_patch_store(const double* __restrict__ inv, const int32_t* __r
 struct ElementTables {
   alignas(16) float div[6][32][4];
   float divl[6][32][4];
-  Grad1D<float> B;
 };
 
-// A_e z_e of every element in FP32, matrix-free: one warp per element, lane = node, then Gauss point,
-// then node; gradient, stress and test integrals by sum factorisation, the divergence from
-// tabulated integrals (ten thousand products per element: FP32 is cheap here, while any FP64
-// instruction, conversions included, holds the pipe for 16 cycles -- hence z in FP32, zf, kept beside
-// z by the smoother).  With the assembled rows each colour of a sweep read the 36-byte blocks of the rows its patches touch, 425 MB of a
-// 32^3 grid; the elements read z and 27 viscosities each and write 12 MB, which stays in L2.
-// Measured per colour (both launches): 32^3 grid ~145 -> 73 us, 16^3 ~30 -> 17 us; several elements
-// per warp, with the tables kept in registers, were slower (84 and 21 us: half the warps).  Against FP64
-// smoothing the error of a V-cycle is 2.7e-7 (3.2e-7 with assembled rows), of one sweep from random
-// data 2.1e-7 (2.1e-7).
+// A_e z_e of every element in FP32, matrix-free: one warp per element; gradient and test integrals by sum
+// factorisation with a line of one component per lane, stress with a Gauss point per lane, the
+// divergence from tabulated integrals (ten thousand products per element: FP32 is cheap here, while any
+// FP64 instruction, conversions included, holds the pipe for 16 cycles -- hence z in FP32, zf, kept
+// beside z by the smoother).  With the assembled rows each colour of a sweep read the 36-byte blocks of
+// the rows its patches touch, 425 MB of a 32^3 grid; the elements read z and 27 viscosities each and
+// write 12 MB, which stays in L2.  What bounds it is the issue of its instructions, half of them
+// shared-memory accesses while a lane held one point of all components (a table value and three inputs for each
+// result); a lane with a line reads three inputs for three results and has the table in its
+// instructions.  Measured per colour (both launches): 32^3 grid ~145 -> 73 us with a point per lane, 16^3
+// ~30 -> 17 us; solve on 32^3 with V(2,2) 401 -> 214 ms, and 191 ms with a line per lane.  Several elements
+// per warp were slower (84 and 21 us: half the warps).  Against FP64 smoothing the error of a V-cycle is
+// 2.7e-7 (3.2e-7 with assembled rows), of one sweep from random data 2.1e-7 (2.1e-7).
 __global__ void __launch_bounds__(128) k_element_residuals(const int32_t* __restrict__ evel,
                                                            const int32_t* __restrict__ epre,
                                                            const float2* __restrict__ f32, int64_t ne, int form,
                                                            const ElementTables* __restrict__ T, int64_t nu,
                                                            const float* zf, float* __restrict__ out,
                                                            const char* __restrict__ next, int64_t next_bytes) {
-  __shared__ Grad1D<float> B;
   __shared__ float su[4][3][27], ss[4][3][3][27], st[4][3][3][27], sp[4][8];
   dep_release();
-  if (threadIdx.x < sizeof(Grad1D<float>) / 4)
-    reinterpret_cast<float*>(&B)[threadIdx.x] = reinterpret_cast<const float*>(&T->B)[threadIdx.x];
   const int warp = threadIdx.x >> 5, q = threadIdx.x & 31;
   const int64_t e = int64_t(blockIdx.x) * 4 + warp;
   const bool here = e < ne, active = here && q < 27;
@@ -443,7 +442,6 @@ __global__ void __launch_bounds__(128) k_element_residuals(const int32_t* __rest
   // this colour's patch inverses, which the next launch streams: DRAM is idle here
   for (int64_t b = (int64_t(blockIdx.x) * 128 + threadIdx.x) * 128; b < next_bytes; b += int64_t(gridDim.x) * 128 * 128)
     prefetch_l2(next + b);
-  __syncthreads();
   dep_wait();
   if (!here) return;
   float (*u)[27] = su[warp];
@@ -484,10 +482,38 @@ __global__ void __launch_bounds__(128) k_element_residuals(const int32_t* __rest
   float d = (h1 ? d2[1] : d2[0]) + __shfl_xor_sync(0xffffffffu, h1 ? d2[0] : d2[1], 1);
   d += __shfl_xor_sync(0xffffffffu, d, 8);
   d += __shfl_xor_sync(0xffffffffu, d, 16);
-  float gr[3][3] = {};
-  element_gradient<float>(B, q, active, u, s, t, gr, [] { __syncwarp(); });
+  // a line of component lc per lane: x lines start at node 3 r, y lines at x + 9 z, z lines at r
+  const int lc = q / 9, r = q % 9, yz = r % 3 + 9 * (r / 3);
+  float p0[3], p1[3], p2[3];
+  if (active) {
+    load_line(u[lc] + 3 * r, 1, p0);
+    line_all<false, false>(p0, s[0][lc] + 3 * r, 1);  // values
+    line_all<true, false>(p0, s[1][lc] + 3 * r, 1);   // x derivatives
+  }
   __syncwarp();
-  if (active)
+  if (active) {
+    load_line(s[0][lc] + yz, 3, p0);
+    load_line(s[1][lc] + yz, 3, p1);
+    line_all<false, false>(p1, t[0][lc] + yz, 3);  // x derivatives
+    line_all<true, false>(p0, t[1][lc] + yz, 3);   // y derivatives
+    line_all<false, false>(p0, t[2][lc] + yz, 3);  // values
+  }
+  __syncwarp();
+  if (active) {
+    load_line(t[0][lc] + r, 9, p0);
+    load_line(t[1][lc] + r, 9, p1);
+    load_line(t[2][lc] + r, 9, p2);
+    line_all<false, false>(p0, s[lc][0] + r, 9);
+    line_all<false, false>(p1, s[lc][1] + r, 9);
+    line_all<true, false>(p2, s[lc][2] + r, 9);
+  }
+  __syncwarp();
+  if (active) {  // gradient -> stress at point q
+    float gr[3][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int l = 0; l < 3; ++l) gr[c][l] = s[c][l][q];
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -495,15 +521,41 @@ __global__ void __launch_bounds__(128) k_element_residuals(const int32_t* __rest
         const float g = form == GDSW_FORM_SYMMETRIC ? gr[c][l] + gr[l][c] : gr[c][l];
         s[c][l][q] = fmaf(f.x, g, f.y * g);
       }
+  }
   __syncwarp();
-  float r[3];
-  element_test<float>(B, q, active, s, t, r, [] { __syncwarp(); });
-  float* o = out + e * ES;
-  if (active)  // through shared memory: the element's 81 values leave as whole lines
+  if (active) {  // the transposed steps
+    load_line(s[lc][0] + r, 9, p0);
+    load_line(s[lc][1] + r, 9, p1);
+    load_line(s[lc][2] + r, 9, p2);
+    line_all<false, true>(p0, t[lc][0] + r, 9);
+    line_all<false, true>(p1, t[lc][1] + r, 9);
+    line_all<true, true>(p2, t[lc][2] + r, 9);
+  }
+  __syncwarp();
+  if (active) {
+    load_line(t[lc][0] + yz, 3, p0);
+    load_line(t[lc][1] + yz, 3, p1);
+    load_line(t[lc][2] + yz, 3, p2);
+    line_all<false, true>(p0, s[lc][0] + yz, 3);
+    s[lc][1][yz] = line_at<true, true, 0>(p1, line_at<false, true, 0>(p2, 0.f));
+    s[lc][1][yz + 3] = line_at<true, true, 1>(p1, line_at<false, true, 1>(p2, 0.f));
+    s[lc][1][yz + 6] = line_at<true, true, 2>(p1, line_at<false, true, 2>(p2, 0.f));
+  }
+  __syncwarp();
+  float* w = &u[0][0];
+  float* wp = &t[0][0][0];
+  if (active) {
+    load_line(s[lc][0] + 3 * r, 1, p0);
+    load_line(s[lc][1] + 3 * r, 1, p1);
+    w[9 * r + lc] = line_at<true, true, 0>(p0, line_at<false, true, 0>(p1, 0.f));
+    w[9 * r + 3 + lc] = line_at<true, true, 1>(p0, line_at<false, true, 1>(p1, 0.f));
+    w[9 * r + 6 + lc] = line_at<true, true, 2>(p0, line_at<false, true, 2>(p1, 0.f));
 #pragma unroll
-    for (int c = 0; c < 3; ++c) (&u[0][0])[3 * q + c] = r[c] + rp[c];
+    for (int c = 0; c < 3; ++c) wp[3 * q + c] = rp[c];
+  }
   __syncwarp();
-  for (int i = q; i < 81; i += 32) o[i] = (&u[0][0])[i];
+  float* o = out + e * ES;
+  for (int i = q; i < 81; i += 32) o[i] = w[i] + wp[i];  // whole lines
   if (q < 8) o[81 + q] = d;
 }
 
@@ -890,7 +942,6 @@ static void mg_create(gdsw_mg* mg, gdsw_ctx* const* grids, int ngrids, const gds
       RefTables R;
       host_tables(R);
       std::vector<ElementTables> H(1);
-      host_grad1d(H[0].B);
       const double ps = 0.25 * x->mesh.h * x->mesh.h;
       for (int a = 0; a < 27; ++a)
         for (int k = 0; k < 8; ++k)
