@@ -357,8 +357,9 @@ int gdsw_set_launch_overlap(int32_t on);
 int gdsw_probe_fma(int32_t precision, double* tflops);
 
 /* Algorithmic bytes of one launch of the level-l local-solve sweeps: direction 0 = forward
- * launches (k = 0 .. K-1), 1 = backward launches (k = 0 .. K-2), in launch order, 2 = the
- * partial-sum reduction of the packed symmetric blocks (k = 0; 0 bytes when none).  Used to
+ * launches, 1 = backward launches, in launch order from k = 0 (of a condensed level the first
+ * forward and the last backward entry are the mid planes with their couplings), 2 = the
+ * partial-sum reductions of the packed symmetric blocks (k = 0; 0 bytes when none).  Used to
  * put the DRAM traffic of a profiled launch beside the bytes the method must move. */
 int gdsw_plan_bytes(const gdsw_ctx* ctx, int32_t level, int32_t direction, int32_t k, double* bytes);
 

@@ -187,8 +187,11 @@ inline double condense_bytes(int prec) { return prec == GDSW_BF16 ? 1.5e9 : 0.9e
 // A batch of block-tridiagonal local problems: dof lists by slab, slab sizes and the offsets of the LDL^T
 // blocks Sinv_k (s_k x s_k) and G_k (m_k x s_k), the update of slab next[k] by slab k: its first m_k
 // rows are those coupled to k.  Slabs are eliminated from both ends of the axis towards a middle slab,
-// which halves the chain of dependent steps: step[k] says when.  The middle slab's two updates fall into
-// different steps, so that no two blocks add to the same rows at once.
+// which halves the chain of dependent steps (launches, or waits of the persistent sweep) that small and
+// medium sets are bound by: step[k] says when.  The middle slab's two updates fall into different
+// steps, so that no two blocks add to the same rows at once.  From one end -> from both: 8^3 box, 8 parts,
+// FP64 apply 137 -> 108 us, FP32 65 -> 48; 11x9x13, 12 parts, FP64 255 -> 224; die, 64 parts, BF16 396 -> 383;
+// large sets, bound by reading the factors, 2 % (channel 32^3, plain slabs, 1968 -> 1937).
 //
 // Condensed sets (large level-1 factors with slabs one element thick): the node planes in the middle of
 // an element layer hold only velocities and couple to the planes on either side of their layer, so

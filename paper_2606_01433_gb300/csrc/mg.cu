@@ -414,8 +414,8 @@ struct ElementTables {
 // shared-memory accesses while a lane held one point of all components (a table value and three inputs for each
 // result); a lane with a line reads three inputs for three results and has the table in its
 // instructions.  Measured per colour (both launches): 32^3 grid ~145 -> 73 us with a point per lane, 16^3
-// ~30 -> 17 us; solve on 32^3 with V(2,2) 401 -> 214 ms, and 191 ms with a line per lane.  Several elements
-// per warp were slower (84 and 21 us: half the warps).  Against FP64 smoothing the error of a V-cycle is
+// ~30 -> 17 us; solve on 32^3 with V(2,2) 401 -> 214 ms, with a line per lane 419 -> 211 (another device).  Several
+// elements per warp were slower (84 and 21 us: half the warps).  Against FP64 smoothing the error of a V-cycle is
 // 2.7e-7 (3.2e-7 with assembled rows), of one sweep from random data 2.1e-7 (2.1e-7).
 __global__ void __launch_bounds__(128) k_element_residuals(const int32_t* __restrict__ evel,
                                                            const int32_t* __restrict__ epre,
