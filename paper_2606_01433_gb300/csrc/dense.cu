@@ -425,7 +425,7 @@ template void launch_sym_reduce<float>(const float*, float*, const GemvPlan&, in
 // lanes per block of rows, whose rows share their columns (5.3 bytes an entry instead of 8).  A
 // block has about 110 columns: whole warps spent as long on the butterflies as on the products in
 // FP64, and eight lanes still read whole 32-byte sectors in FP32.  FP32: 24 us on a 20^3 box in 64 parts
-// (70 MB), 28 us on the die; FP64: 29 us on 135 thousand local dofs.
+// (70 MB), 28 us on the die, 60 us on the 32^3 channel; FP64: 29 us on 135 thousand local dofs.
 template <typename TV>
 __global__ void __launch_bounds__(256) k_coupling(int nblk, const int32_t* __restrict__ row,
                                                   const int32_t* __restrict__ nrow, const int64_t* __restrict__ off,
