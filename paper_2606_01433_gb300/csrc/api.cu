@@ -1150,8 +1150,8 @@ static void local_solve(gdsw_ctx* c, int l, const double* r, double* z, cudaStre
     else
       launch_gather<float>(r, L.gdof, static_cast<float*>(L.vec), nv, s);
   }
-  // block-LDL^T sweeps: forward launches (S_k^{-1} y_k and the G_{k+1} update), then backward
-  // launches (G_{k+1}^T), every one a ragged batched GEMV over all parts of the level
+  // block-LDL^T sweeps: forward launches (S_k^{-1} y_k and the update by G_k), then backward
+  // launches (G_k^T), every one a ragged batched GEMV over all parts of the level
   const int group = l == 0 ? GDSW_K_LOCAL : GDSW_K_COARSE;
   auto sweep = [&](const GemvPlan& P, int k, int ld) {
     if (L.prec == GDSW_FP64) {

@@ -1,7 +1,7 @@
 // Device kernels of the numeric set-up (arXiv 2606.01433, Section 2.1 and 2.2):
 //  - extraction of the local saddle-point matrices A_i = R_i A R_i^T into the blocks of a
 //    block-tridiagonal (slab) ordering: diagonal blocks, and the sub/super-diagonal
-//    couplings restricted to the back-coupled dofs;
+//    couplings restricted to the dofs coupled to the next slab;
 //  - the right-hand sides -A_IGamma Phi_Gamma of the coarse-basis extension, and the
 //    pieces of the Galerkin product A_0 = Phi^T A Phi;
 //  - dense gathers and basis assembly on the coarse levels.
