@@ -489,7 +489,7 @@ struct gdsw_ctx {
   int m_alloc = 0;
   double *d_V = nullptr, *d_Z = nullptr, *d_w = nullptr, *d_H = nullptr, *d_gvec = nullptr;
   double *d_cs = nullptr, *d_sn = nullptr, *d_part = nullptr, *d_scal = nullptr, *d_y = nullptr;
-  double* h_est = nullptr;          // pinned: residual estimates of the two iterations in flight
+  double* h_est = nullptr;          // host: residual estimates of the two iterations in flight
   unsigned* d_count = nullptr;      // CTAs done in an Arnoldi launch, in all and per group (0 between launches)
   int* d_status = nullptr;          // device error word
   // CUDA graph of the apply

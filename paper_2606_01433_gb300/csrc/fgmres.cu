@@ -388,46 +388,43 @@ static int arnoldi_ctas(int64_t n) {
   return int(waves * kWave);
 }
 
-// Pinned pairs of estimates for the contexts of the process.  Freeing pinned memory waits for the whole
-// device, so a context gives its pair back instead; the page goes with the last context that holds a
-// pair.  Contexts beyond the page's pairs allocate their own.
+// Pairs of estimates for the contexts of the process, in host memory that is page-locked once, by the first
+// solve, and stays so: page-locking memory per context, and freeing it, would wait for the whole device
+// (gdsw_destroy waited out a 0.4 s kernel on another stream).  Contexts beyond the pairs take pageable
+// memory, where a copy holds the host until it is done: nothing runs ahead, and the results are the same.
+// So it is if the page-locking fails, or after a reset of the device, which undoes it.
+constexpr int kEstPairs = 4096;
+alignas(65536) static double g_est[2 * kEstPairs];
 static std::mutex g_est_mu;
-static double* g_est_page = nullptr;
 static std::vector<int> g_est_free;
-constexpr int kEstPairs = 256;
-
-static double* pinned(int n) {
-  void* p = nullptr;
-  GDSW_CUDA(cudaHostAlloc(&p, n * sizeof(double), cudaHostAllocPortable));
-  return static_cast<double*>(p);
-}
+static bool g_est_ready = false;
 
 static double* take_estimates() {
-  std::lock_guard<std::mutex> lock(g_est_mu);
-  if (!g_est_page) {
-    g_est_free.resize(kEstPairs);
-    for (int i = 0; i < kEstPairs; ++i) g_est_free[i] = i;
-    g_est_page = pinned(2 * kEstPairs);
+  {
+    std::lock_guard<std::mutex> lock(g_est_mu);
+    if (!g_est_ready) {
+      g_est_free.resize(kEstPairs);
+      for (int i = 0; i < kEstPairs; ++i) g_est_free[i] = kEstPairs - 1 - i;
+      if (cudaHostRegister(g_est, sizeof(g_est), cudaHostRegisterPortable) != cudaSuccess) cudaGetLastError();
+      g_est_ready = true;
+    }
+    if (!g_est_free.empty()) {
+      const int i = g_est_free.back();
+      g_est_free.pop_back();
+      return g_est + 2 * i;
+    }
   }
-  if (g_est_free.empty()) return pinned(2);
-  const int i = g_est_free.back();
-  g_est_free.pop_back();
-  return g_est_page + 2 * i;
+  return new double[2];
 }
 
 void give_estimates(double* p) {
   if (!p) return;
-  std::lock_guard<std::mutex> lock(g_est_mu);
-  if (!g_est_page || p < g_est_page || p >= g_est_page + 2 * kEstPairs) {
-    cudaFreeHost(p);
+  if (p < g_est || p >= g_est + 2 * kEstPairs) {
+    delete[] p;
     return;
   }
-  g_est_free.push_back(int((p - g_est_page) / 2));
-  if (int(g_est_free.size()) == kEstPairs) {
-    cudaFreeHost(g_est_page);
-    g_est_page = nullptr;
-    g_est_free.clear();
-  }
+  std::lock_guard<std::mutex> lock(g_est_mu);
+  g_est_free.push_back(int((p - g_est) / 2));
 }
 
 static void ensure_workspace(gdsw_ctx* c, int m) {
