@@ -588,6 +588,7 @@ static void autotune_level1(gdsw_ctx* c) {
       build_local_plan(c, c->lh[0].loc, L);
     }
     L.persistent = bestP;
+    L.chosen_rows = best_rows;
     L.tuned_ms = best;
   } catch (...) {
     if (e0) cudaEventDestroy(e0);
@@ -1967,7 +1968,10 @@ int gdsw_sweep_wait_selftest(gdsw_ctx* c) {
 
 int gdsw_set_local_sweep(gdsw_ctx* c, int32_t persistent, int32_t ctas_per_sm, int32_t tile_rows) {
   if (!c || c->host_only || ctas_per_sm < 0) return GDSW_ERR_INVALID_ARG;
-  if (tile_rows != 0 && tile_rows != 32 && tile_rows != 64 && tile_rows != 128) return GDSW_ERR_INVALID_ARG;
+  // the shapes open to callers, and any that the context has (gdsw_sizes), as 16 rows of its set-up's choice
+  bool known = tile_rows == 0 || tile_rows == -1 || tile_rows == 32 || tile_rows == 64 || tile_rows == 128;
+  for (const LevelDev& L : c->ld) known = known || tile_rows == L.fwd.rows_per_tile;
+  if (!known) return GDSW_ERR_INVALID_ARG;
   if (c->apply_graph) {
     c->err = "gdsw_set_local_sweep: the apply is already captured in a CUDA graph (use_graph)";
     return GDSW_ERR_INVALID_ARG;
@@ -1976,8 +1980,9 @@ int gdsw_set_local_sweep(gdsw_ctx* c, int32_t persistent, int32_t ctas_per_sm, i
     for (size_t l = 0; l < c->ld.size(); ++l) {
       LevelDev& L = c->ld[l];
       L.persistent = persistent != 0;
-      if (tile_rows != 0 && tile_rows != L.fwd.rows_per_tile) {
-        L.fwd.rows_per_tile = tile_rows;
+      const int rows = tile_rows > 0 ? tile_rows : (tile_rows < 0 ? L.chosen_rows : L.fwd.rows_per_tile);
+      if (rows != L.fwd.rows_per_tile) {
+        L.fwd.rows_per_tile = rows;
         build_local_plan(c, c->lh[l].loc, L);
       }
       resize_sweep(L, ctas_per_sm);

@@ -367,6 +367,7 @@ struct LevelDev {
   SweepPlan sweep;              // the same tiles as one persistent launch
   bool persistent = false;      // local solve as the persistent launch (else one launch per slab step)
   double tuned_ms = 0;          // autotuned local-solve time (0: not tuned)
+  int chosen_rows = 32;         // rows per forward tile that the set-up chose
   void* vec = nullptr;          // local vector workspace (2 * nvec, compute precision)
   int32_t *sc_ptr = nullptr, *sc_pos = nullptr;
   double* sc_w = nullptr;

@@ -403,7 +403,8 @@ class Context:
 
     def gdsw_set_local_sweep(self, persistent=True, ctas_per_sm=0, tile_rows=0):
         """Override the set-up autotuner: local solves as one persistent launch per level or one
-        launch per slab step, and rows per forward tile (32/64/128; 0 keeps the current)."""
+        launch per slab step, and rows per forward tile (32/64/128 or what sizes.tile_rows reports
+        for a level; 0 keeps the current, -1 goes back to the set-up's choice)."""
         return self._check(self.lib.gdsw_set_local_sweep(self.h, 1 if persistent else 0, int(ctas_per_sm),
                                                          int(tile_rows)))
 
