@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 #include <cstdio>
@@ -134,7 +135,9 @@ struct DevArena {
 
 inline size_t elem_size(int prec) { return prec == GDSW_FP64 ? 8 : (prec == GDSW_FP32 ? 4 : 2); }
 // assembly workspace: the 405 blocks (9 values) of each fluid element of a chunk.  9120 elements
-// are five full waves of the element kernel (152 SMs, 6 CTAs of 2 elements) and 266 MB.
+// are five full waves of the element kernel (152 SMs, 6 CTAs of 2 elements) and 266 MB, which is no more
+// than the sliced copy of that many elements where most nodes are free: they take turns in one buffer
+// (MeshHost::sell_values).
 constexpr int64_t kAsmChunk = 9120;
 constexpr int64_t kAsmElemValues = 405 * 9;
 // velocity nodes up to which the SpMV uses slices of 8 rows (build_sell)
@@ -311,6 +314,10 @@ struct MeshHost {
   std::vector<int64_t> sell_aoff, sell_boff;  // nslices + 1: first block / B^T slot of each slice
   std::vector<int32_t> sell_acol, sell_asrc;  // per block slot: column node, source block (-1: pad)
   std::vector<int32_t> sell_bcol, sell_bsrc;  // per B^T slot: pressure column, source entry (-1: pad)
+  // values of the buffer that holds the sliced blocks, and during an assembly the element blocks
+  int64_t sell_values() const {
+    return std::max(9 * int64_t(sell_acol.size()), std::min(kAsmChunk, int64_t(fluid.size())) * kAsmElemValues);
+  }
   bool shares_element(int64_t a, int64_t b) const;
   void coords(int64_t node, int& i, int& j, int& k) const {
     i = int(node % NX);
@@ -459,7 +466,6 @@ struct gdsw_ctx {
   int32_t *d_a_diag = nullptr, *d_a_tpos = nullptr;  // diagonal block of each row, transpose map
   int32_t *d_asm_cta = nullptr, *d_asm_uoff = nullptr;  // assembly work units (see MeshHost)
   uint32_t* d_asm_unit = nullptr;
-  double* d_asm_ws = nullptr;       // element blocks of one chunk (asm_ws_bytes)
   int32_t *d_sell_row = nullptr, *d_sell_acol = nullptr, *d_sell_asrc = nullptr;  // sliced SpMV copy
   int32_t *d_sell_bcol = nullptr, *d_sell_bsrc = nullptr;
   int64_t *d_sell_aoff = nullptr, *d_sell_boff = nullptr;

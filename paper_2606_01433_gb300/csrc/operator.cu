@@ -199,7 +199,8 @@ __device__ void divergence_entry_p1(int64_t P, int64_t J, const Geo& G, const in
 //
 // Workspace: unit (a, b) of element e at ws[((a_z 3 + b_z) NT + 45 e + P(A, B)) 9 .. + 9], so a
 // warp's 32 blocks are 2304 contiguous bytes.  It holds kAsmChunk elements (266 MB); larger
-// meshes run chunk by chunk and the gather adds onto the blocks of the chunks before.
+// meshes run chunk by chunk and the gather adds onto the blocks of the chunks before.  It lies in the
+// buffer of the sliced copy, which is filled from the gathered blocks afterwards.
 constexpr int kAsmPairs = 45;
 
 // derivative pattern t of a one-dimensional pair: 0 value-value, 1 value-derivative (of b), 2
@@ -755,6 +756,7 @@ void launch_assembly(gdsw_ctx* c, cudaStream_t s, bool newton) {
   double* aval = c->d_val;
   double* btval = c->d_val + 9 * c->nnzb;
   double* bval = btval + 3 * c->nbt;
+  double* ws = c->d_sell_aval;  // of use again once launch_sell_fill has refreshed it below
   for (size_t q = 0; q + 1 < c->mesh.asm_chunk.size(); ++q) {
     const int64_t f0 = c->mesh.asm_chunk[q], f1 = c->mesh.asm_chunk[q + 1];
     const int cta0 = c->mesh.asm_chunk_cta[2 * q], cta1 = c->mesh.asm_chunk_cta[2 * q + 1];
@@ -762,11 +764,11 @@ void launch_assembly(gdsw_ctx* c, cudaStream_t s, bool newton) {
                    : newton                       ? k_element_blocks<true, true>
                                                   : k_element_blocks<true, false>;
     launch_chained(element, dim3(unsigned((f1 - f0 + 1) / 2)), dim3(96), 0, s, c->d_nu, T, 0.5 * c->mesh.h,
-                   c->d_dn, f0, f1 - f0, c->d_asm_ws);
+                   c->d_dn, f0, f1 - f0, ws);
     check_launch("k_element_blocks");
     if (cta1 > cta0) {
       launch_chained(k_gather_blocks, dim3(unsigned(cta1 - cta0)), dim3(256), 0, s, c->d_asm_cta, cta0,
-                     c->d_asm_uoff, c->d_asm_unit, c->d_a_tpos, c->d_asm_ws, f0, f1, aval);
+                     c->d_asm_uoff, c->d_asm_unit, c->d_a_tpos, ws, f0, f1, aval);
       check_launch("k_gather_blocks");
     }
   }
