@@ -258,8 +258,8 @@ void segsum(const int64_t* key, const int64_t* ptr, const int64_t* pos, int64_t 
   check_launch("k_segsum");
 }
 
-// Phi_Gamma^T A_GammaGamma Phi_Gamma: a warp runs over one of gridDim.y shares of the interface dofs
-// that carry coarse column k = blockIdx.x (value w_a) and over the nonzeros of their rows; a nonzero of
+// Rows k0 ... of Phi_Gamma^T A_GammaGamma Phi_Gamma: a warp runs over one of gridDim.y shares of the interface
+// dofs that carry coarse column k = k0 + blockIdx.x (value w_a) and over the nonzeros of their rows; a nonzero of
 // column b adds w_a w_b A_ab to entry (k, l) of the share's matrix for every Phi_Gamma entry
 // (b, l, w_b).  Lanes that meet in one l are summed in lane order by the lowest of them, so every
 // entry is one sum in list order, without atomics.  Bound by the latency of those additions (one
@@ -270,9 +270,9 @@ __global__ void __launch_bounds__(32) k_gamma_gamma(MatView A, const int32_t* __
                                                     const double* __restrict__ rg_val,
                                                     const int32_t* __restrict__ gamma_ptr,
                                                     const int32_t* __restrict__ gcol, const double* __restrict__ gval,
-                                                    int64_t n0, double* A0) {
-  const int k = blockIdx.x, lane = threadIdx.x;
-  double* row = A0 + (int64_t(blockIdx.y) * n0 + k) * n0;
+                                                    int64_t n0, int k0, double* part) {
+  const int k = k0 + int(blockIdx.x), lane = threadIdx.x;
+  double* row = part + (int64_t(blockIdx.y) * gridDim.x + blockIdx.x) * n0;
   auto add = [&](int64_t b, double v, bool on) {  // every lane of the warp
     int32_t e = on ? gamma_ptr[b] : 0;
     const int32_t e1 = on ? gamma_ptr[b + 1] : 0;
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(32) k_gamma_gamma(MatView A, const int32_t* __
   }
 }
 
-// A0 += the sum of the shares, in order
+// rows of A0 += the sum of their shares, in order
 __global__ void __launch_bounds__(256) k_add_shares(const double* __restrict__ part, int shares, int64_t n,
                                                     double* __restrict__ A0) {
   const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
@@ -339,20 +339,25 @@ __global__ void __launch_bounds__(256) k_add_shares(const double* __restrict__ p
   A0[i] += s;
 }
 
-// A0 += Phi_Gamma^T A_GammaGamma Phi_Gamma; eight shares per coarse column (fewer if their matrices
-// would exceed 1 GB)
+// A0 += Phi_Gamma^T A_GammaGamma Phi_Gamma, eight shares per coarse column, fewer from 4097 columns on (enough
+// warps without).  Rows are taken in blocks whose shares fill 128 MB at most: A_0 itself has 4 GB on the die
+// (22 thousand columns), and its shares would have as much again.
 void gamma_gamma(DevArena& tmp, const MatView& A, const int32_t* rg_ptr, const int32_t* rg_dof, const double* rg_val,
                  const int32_t* gamma_ptr, const int32_t* gcol, const double* gval, int64_t n0, double* A0,
                  cudaStream_t s) {
   if (n0 == 0) return;
-  const int shares = int(std::max<int64_t>(1, std::min<int64_t>(8, (int64_t(1) << 27) / (n0 * n0))));
-  double* part = tmp.alloc<double>(size_t(shares) * n0 * n0);
-  GDSW_CUDA(cudaMemsetAsync(part, 0, size_t(shares) * n0 * n0 * sizeof(double), s));
-  k_gamma_gamma<<<dim3(unsigned(n0), unsigned(shares)), 32, 0, s>>>(A, rg_ptr, rg_dof, rg_val, gamma_ptr, gcol, gval,
-                                                                    n0, part);
-  check_launch("k_gamma_gamma");
-  k_add_shares<<<unsigned((n0 * n0 + 255) / 256), 256, 0, s>>>(part, shares, n0 * n0, A0);
-  check_launch("k_add_shares");
+  const int64_t shares = std::max<int64_t>(1, std::min<int64_t>(8, (int64_t(1) << 27) / (n0 * n0)));
+  const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(n0, (int64_t(1) << 24) / (shares * n0)));
+  double* part = tmp.alloc<double>(size_t(shares * rows * n0));
+  for (int64_t k0 = 0; k0 < n0; k0 += rows) {
+    const int64_t nk = std::min<int64_t>(rows, n0 - k0);
+    GDSW_CUDA(cudaMemsetAsync(part, 0, size_t(shares * nk * n0) * sizeof(double), s));
+    k_gamma_gamma<<<dim3(unsigned(nk), unsigned(shares)), 32, 0, s>>>(A, rg_ptr, rg_dof, rg_val, gamma_ptr, gcol, gval,
+                                                                      n0, int(k0), part);
+    check_launch("k_gamma_gamma");
+    k_add_shares<<<unsigned((nk * n0 + 255) / 256), 256, 0, s>>>(part, int(shares), nk * n0, A0 + k0 * n0);
+    check_launch("k_add_shares");
+  }
   tmp.release(part);
 }
 
