@@ -696,9 +696,10 @@ def run_gdsw(args, rank, world, local):
         "setup_breakdown_ms": dict(zip(["host_symbolic", "viscosity_assembly", "level1_factors", "phi_and_A0",
                                         "coarse_levels", "total"], [float(v) for v in sizes.setup_ms])),
         "factor_gb": sizes.factor_entries[0] * (4 if args.mixed == "fp32" else 2) / 1e9,
-        "roofline": {"kernel": ("k_sweep (level-1 persistent block-LDL^T sweep, one launch per apply)" if persistent
+        "roofline": {"kernel": ("k_sweep (level-1 persistent block-LDL^T sweep" if persistent
                                 else "k_gemv/k_sym_reduce/k_gemvt (level-1 block-LDL^T sweep: one chained launch "
-                                     "per slab step, the chain of one apply timed as one unit)"),
+                                     "per slab step") + "; of a condensed set with its mid-plane k_gemv and "
+                               "k_coupling launches; the local solves of one apply timed as one unit)",
                      "bound": "hbm", "achieved": gemv_gbs,
                      "peak": peak, "unit": "GB/s", "frac": (gemv_gbs / peak) if gemv_gbs else None,
                      "peak_kind": peak_kind, "avg_launch_ms": gemv_avg_ms, "avg_launch_bytes": gemv_avg_bytes,

@@ -181,7 +181,7 @@ struct InvTask {
 // Factors of at least this many bytes are condensed.  Smaller ones run at the latency of their launches,
 // of which condensing adds four to six.  Local solves, plain -> condensed.  FP32: channel with obstacles
 // 32^3, 64 parts (11.4 GB) 1937 -> 1380 us, die, 64 parts (1.9 GB) 424 -> 393, 20^3 box, 64 parts (1.7 GB)
-// 343 -> 325.  FP64: 17x14x12 box, 36 parts, discontinuous pressure (0.99 GB) 398 -> 366, 14^3, 27 parts (0.91
+// 343 -> 325; 17x14x12 box, 36 parts (0.49 GB) 147 -> 144, even.  FP64: 17x14x12 box, 36 parts, discontinuous pressure (0.99 GB) 398 -> 366, 14^3, 27 parts (0.91
 // GB) 354 -> 351.  BF16, whose smaller blocks are stored in full: die (0.95 GB) 328 -> 371, 20^3 (0.84 GB)
 // 271 -> 292.
 inline double condense_bytes(int prec) { return prec == GDSW_BF16 ? 1.5e9 : 0.9e9; }
@@ -460,7 +460,6 @@ struct gdsw_ctx {
   double* d_newton_work = nullptr;  // Newton step: lifted b, residual, increment (3 n)
   uint8_t* d_mask = nullptr;
   int32_t* d_fluid = nullptr;       // fluid index -> element
-  int32_t* d_felem = nullptr;
   int32_t *d_vnode = nullptr, *d_pnode = nullptr, *d_vidx = nullptr;
   int32_t *d_a_ptr = nullptr, *d_a_col = nullptr, *d_bt_ptr = nullptr, *d_bt_col = nullptr;
   int32_t *d_a_diag = nullptr, *d_a_tpos = nullptr;  // diagonal block of each row, transpose map

@@ -1131,11 +1131,11 @@ __global__ void __launch_bounds__(NT) k_gj_panel_rows(const InvTaskP* __restrict
   }
 }
 
-// Pivot choice for a panel of more rows than a cluster's registers hold: one CTA of 1024 threads; the first RS rows of the panel copy
-// live in shared memory (row stride NB + 1), the rest in the global scratch; the column
-// maximum is found with warp shuffles (largest magnitude, smallest row on ties -- the same
-// pivots as the tree reduction above), and the rank-1 elimination runs one warp per row,
-// lane = column.  Only the pivot rows are used afterwards.
+// Pivot choice for a panel of more rows than a cluster's registers hold: one CTA of 1024 threads.  The first
+// RS rows of the panel copy live in shared memory (row stride NB + 1), the rest in the global scratch; the
+// column maximum is found with warp shuffles (largest magnitude, smallest row on ties, the pivots of
+// k_gj_panel_rows), and the rank-1 elimination runs one warp per row, lane = column.  Only the pivot rows
+// are used afterwards.
 template <typename T>
 __device__ __forceinline__ T& panel_at(T* Ps, T* Pg, int RS, int r, int c) {
   return r < RS ? Ps[r * (GJ_NB + 1) + c] : Pg[int64_t(r) * GJ_NB + c];

@@ -21,11 +21,10 @@ __host__ __device__ constexpr double q2_d(int a, int q) {
 // of 243).  Thread q = 0..26 of the element owns node q, then the partial results of index q, then
 // Gauss point q (x fastest throughout); u, s, t are the element's shared arrays [c][27], `sync` is
 // a barrier over the element's threads.
-template <typename T>
 struct Grad1D {
-  T v[3][3], d[3][3];   // [basis][point]
+  double v[3][3], d[3][3];   // [basis][point]
 };
-__device__ __forceinline__ void fill_grad1d(Grad1D<double>& B, int tid) {
+__device__ __forceinline__ void fill_grad1d(Grad1D& B, int tid) {
   if (tid < 9) {
     B.v[tid / 3][tid % 3] = q2_v(tid / 3, tid % 3);
     B.d[tid / 3][tid % 3] = q2_d(tid / 3, tid % 3);
@@ -34,64 +33,64 @@ __device__ __forceinline__ void fill_grad1d(Grad1D<double>& B, int tid) {
 // acc + sum over k of p[k step] times the values (DER: derivatives) of basis k at point i, or (TEST) of
 // basis i at point k
 template <bool DER, bool TEST>
-__device__ __forceinline__ double line(const Grad1D<double>& B, int i, const double* p, int step, double acc) {
+__device__ __forceinline__ double line(const Grad1D& B, int i, const double* p, int step, double acc) {
   const double(*b)[3] = DER ? B.d : B.v;
   return fma(p[2 * step], TEST ? b[i][2] : b[2][i],
              fma(p[step], TEST ? b[i][1] : b[1][i], fma(p[0], TEST ? b[i][0] : b[0][i], acc)));
 }
-template <typename T, typename Sync>
-__device__ __forceinline__ void element_gradient(const Grad1D<T>& B, int q, bool active, const T (*u)[27],
-                                                 T (*s)[3][27], T (*t)[3][27], T gr[3][3], Sync sync) {
+template <typename Sync>
+__device__ __forceinline__ void element_gradient(const Grad1D& B, int q, bool active, const double (*u)[27],
+                                                 double (*s)[3][27], double (*t)[3][27], double gr[3][3], Sync sync) {
   const int x = q % 3, y = (q / 3) % 3, z = q / 9;
   if (active)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {  // along x: values s[0], derivatives s[1]
-      s[0][c][q] = line<false, false>(B, x, u[c] + q - x, 1, T(0));
-      s[1][c][q] = line<true, false>(B, x, u[c] + q - x, 1, T(0));
+      s[0][c][q] = line<false, false>(B, x, u[c] + q - x, 1, 0.0);
+      s[1][c][q] = line<true, false>(B, x, u[c] + q - x, 1, 0.0);
     }
   sync();
   if (active)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {  // along y: dx t[0], dy t[1], no derivative t[2]
-      t[0][c][q] = line<false, false>(B, y, s[1][c] + q - 3 * y, 3, T(0));
-      t[1][c][q] = line<true, false>(B, y, s[0][c] + q - 3 * y, 3, T(0));
-      t[2][c][q] = line<false, false>(B, y, s[0][c] + q - 3 * y, 3, T(0));
+      t[0][c][q] = line<false, false>(B, y, s[1][c] + q - 3 * y, 3, 0.0);
+      t[1][c][q] = line<true, false>(B, y, s[0][c] + q - 3 * y, 3, 0.0);
+      t[2][c][q] = line<false, false>(B, y, s[0][c] + q - 3 * y, 3, 0.0);
     }
   sync();
   if (active)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {  // along z
-      gr[c][0] = line<false, false>(B, z, t[0][c] + q - 9 * z, 9, T(0));
-      gr[c][1] = line<false, false>(B, z, t[1][c] + q - 9 * z, 9, T(0));
-      gr[c][2] = line<true, false>(B, z, t[2][c] + q - 9 * z, 9, T(0));
+      gr[c][0] = line<false, false>(B, z, t[0][c] + q - 9 * z, 9, 0.0);
+      gr[c][1] = line<false, false>(B, z, t[1][c] + q - 9 * z, 9, 0.0);
+      gr[c][2] = line<true, false>(B, z, t[2][c] + q - 9 * z, 9, 0.0);
     }
 }
 
 // The transposed steps: with the stress s[c][l] (weights included) given at the Gauss points, f[c] =
 // sum over points and l of s[c][l] d_l phi_q for node q.  s and t are overwritten.
-template <typename T, typename Sync>
-__device__ __forceinline__ void element_test(const Grad1D<T>& B, int q, bool active, T (*s)[3][27], T (*t)[3][27],
-                                             T f[3], Sync sync) {
+template <typename Sync>
+__device__ __forceinline__ void element_test(const Grad1D& B, int q, bool active, double (*s)[3][27], double (*t)[3][27],
+                                             double f[3], Sync sync) {
   const int x = q % 3, y = (q / 3) % 3, z = q / 9;
   if (active)  // along z
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      t[c][0][q] = line<false, true>(B, z, s[c][0] + q - 9 * z, 9, T(0));
-      t[c][1][q] = line<false, true>(B, z, s[c][1] + q - 9 * z, 9, T(0));
-      t[c][2][q] = line<true, true>(B, z, s[c][2] + q - 9 * z, 9, T(0));
+      t[c][0][q] = line<false, true>(B, z, s[c][0] + q - 9 * z, 9, 0.0);
+      t[c][1][q] = line<false, true>(B, z, s[c][1] + q - 9 * z, 9, 0.0);
+      t[c][2][q] = line<true, true>(B, z, s[c][2] + q - 9 * z, 9, 0.0);
     }
   sync();
   if (active)  // along y: s[c][0] still needs the x derivative, s[c][1] the x value
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      s[c][0][q] = line<false, true>(B, y, t[c][0] + q - 3 * y, 3, T(0));
-      s[c][1][q] = line<true, true>(B, y, t[c][1] + q - 3 * y, 3, line<false, true>(B, y, t[c][2] + q - 3 * y, 3, T(0)));
+      s[c][0][q] = line<false, true>(B, y, t[c][0] + q - 3 * y, 3, 0.0);
+      s[c][1][q] = line<true, true>(B, y, t[c][1] + q - 3 * y, 3, line<false, true>(B, y, t[c][2] + q - 3 * y, 3, 0.0));
     }
   sync();
   if (active)  // along x
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-      f[c] = line<true, true>(B, x, s[c][0] + q - x, 1, line<false, true>(B, x, s[c][1] + q - x, 1, T(0)));
+      f[c] = line<true, true>(B, x, s[c][0] + q - x, 1, line<false, true>(B, x, s[c][1] + q - x, 1, 0.0));
 }
 
 // ------------------------------------------------------------------ the same in FP32, a line per thread

@@ -32,9 +32,11 @@ constexpr int RT = 256;
 // entry per lane, where the step is bound by its launches.
 // Measured per iteration beside apply and product, ~30 basis vectors, against eleven launches (dots,
 // sum, update, dots, sum, update, sum, norm, norm sum, scaling, rotation): n = 11.5 thousand 82 ->
-// 60 us, 180 thousand 115 -> 104 us, 751 thousand 267 -> 263 us (157 us of FP64 work).  One entry
-// per lane in many CTAs (the form of the separate updates) is slower here: the end of a CTA, a fence
-// and an atomic, is paid per wave (751 thousand: 79 us instead of 57 for update and norm).
+// 60 us, 180 thousand 115 -> 104 us, 656 thousand 276 -> 243, 798 thousand 310 -> 277, 876 thousand 335 -> 320
+// (157 us of FP64 work at 751 thousand).  Above 934 thousand entries, in two waves or more, it is behind: 959
+// thousand 351 -> 378, 1.8 million 573 -> 587; seven and eight entries a lane spill (-Xptxas -v: 48 to 268
+// bytes).  One entry per lane in many CTAs (the form of the separate updates) is slower here: the end of a
+// CTA, a fence and an atomic, is paid per wave (751 thousand: 79 us instead of 57 for update and norm).
 constexpr int AT = 256, AW = AT / 32;  // threads, warps of a CTA
 constexpr int AFLUSH = 64;             // basis vectors whose warp sums are staged at a time
 constexpr int AGROUP = 32, AONE = 96;  // CTAs whose partial sums are added together; one group up to AONE

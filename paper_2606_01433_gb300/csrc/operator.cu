@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256) k_viscosity(const int32_t* __restrict__ f
                                                    const double* __restrict__ uk, Geo G, int form, int has_uk,
                                                    double nu0, double nu_inf, double lam, double ncar,
                                                    double* __restrict__ nu, double* __restrict__ dn) {
-  __shared__ Grad1D<double> B;
+  __shared__ Grad1D B;
   __shared__ double u[kViscElems][3][27], s[kViscElems][2][3][27], w[kViscElems][3][3][27];
   dep_release();
   dep_wait();
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256) k_viscosity(const int32_t* __restrict__ f
   __syncthreads();
   double gr[3][3];
   const int se = active ? el : 0;
-  element_gradient<double>(B, q, active, u[se], s[se], w[se], gr, [] { __syncthreads(); });
+  element_gradient(B, q, active, u[se], s[se], w[se], gr, [] { __syncthreads(); });
   if (!active) return;
   const double sc = 2.0 / G.h;
   double dd = 0.0;  // D : D
@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(128) k_lift_elements(const int32_t* __restrict
                                                        const int32_t* __restrict__ fluid, Geo G, int form, int pdisc,
                                                        const double* __restrict__ nu, const RefTables* __restrict__ T,
                                                        const double* __restrict__ g, double* __restrict__ lw) {
-  __shared__ Grad1D<double> B;
+  __shared__ Grad1D B;
   __shared__ double su[4][3][27], ss[4][3][3][27], st[4][3][3][27];
   __shared__ double sdiv[4][27];
   dep_release();
@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(128) k_lift_elements(const int32_t* __restrict
   }
   __syncwarp();
   double gr[3][3];
-  element_gradient<double>(B, q, active, u, s, t, gr, [] { __syncwarp(); });
+  element_gradient(B, q, active, u, s, t, gr, [] { __syncwarp(); });
   __syncwarp();
   const int x = q % 3, y = (q / 3) % 3, z = q / 9;
   if (active) {
@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(128) k_lift_elements(const int32_t* __restrict
   __syncwarp();
   double* o = lw + le * kLiftValues;
   double f[3];
-  element_test<double>(B, q, active, s, t, f, [] { __syncwarp(); });
+  element_test(B, q, active, s, t, f, [] { __syncwarp(); });
   if (active)
 #pragma unroll
     for (int c = 0; c < 3; ++c) o[3 * q + c] = -f[c];
