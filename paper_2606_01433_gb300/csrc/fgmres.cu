@@ -12,6 +12,7 @@
 
 #include "common.h"
 #include "kernels.h"
+#include "quotient.h"
 
 namespace gdsw {
 
@@ -250,8 +251,12 @@ __global__ void __launch_bounds__(256) k_scale_givens(double* w, int64_t n, doub
   dep_wait();
   const double d = __ldcg(scal + 1);
   if (blockIdx.x > 0) {
-    for (int64_t e = (int64_t(blockIdx.x) - 1) * 1024 + threadIdx.x, k = 0; k < 4 && e < n; ++k, e += 256)
-      w[e] = d > 0.0 ? __ldcg(w + e) / d : 0.0;
+    const double r = 1.0 / d;
+    const bool ok = quotient_ok(d);
+    for (int64_t e = (int64_t(blockIdx.x) - 1) * 1024 + threadIdx.x, k = 0; k < 4 && e < n; ++k, e += 256) {
+      const double v = __ldcg(w + e);
+      w[e] = ok ? quotient_by(v, d, r) : (d > 0.0 ? v / d : 0.0);
+    }
     return;
   }
   // the rotations are a serial chain: their operands are staged in shared memory
