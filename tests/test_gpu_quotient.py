@@ -2,6 +2,7 @@
 exponent down to 2^-900 and divisors over the range that quotient_ok admits, and divisors of all ones and
 one above a power of two, where a reciprocal is at its worst."""
 import os
+import shutil
 import subprocess
 
 import pytest
@@ -58,7 +59,8 @@ def test_quotients_round_like_the_division(tmp_path):
     csrc = os.path.join(os.path.dirname(__file__), "..", "paper_2606_01433_gb300", "csrc")
     (tmp_path / "q.cu").write_text(SRC)
     exe = str(tmp_path / "q")
-    subprocess.run(["nvcc", "-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-I", csrc, "-o", exe,
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    subprocess.run([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-I", csrc, "-o", exe,
                     str(tmp_path / "q.cu")], check=True, timeout=300)
     out = subprocess.run([exe], check=True, timeout=120, capture_output=True, text=True).stdout.split()
     bad, done = int(out[0]), int(out[1])
